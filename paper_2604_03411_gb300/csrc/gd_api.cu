@@ -98,7 +98,7 @@ void free_ckpts(gd::Handle &H);
 void free_handle(gd::Handle &H)
 {
     void *ptrs[] = {H.X, H.conn, H.slot, H.rowptr, H.colidx, H.fixed, H.bc_dof, H.bc_scale, H.react_dof,
-                    H.psi.p, H.psi.W2T, H.yld.p, H.yld.W2T, H.psi.pf, H.psi.W2Tf, H.yld.pf, H.yld.W2Tf, H.netc, H.dofs, H.kappa, H.dofs_prev, H.dofs_pp, H.w_dofs,
+                    H.psi.p, H.psi.W2T, H.yld.p, H.yld.W2T, H.psi.pf, H.psi.W2Tf, H.yld.pf, H.yld.W2Tf, H.psi.fx, H.yld.fx, H.netc, H.dofs, H.kappa, H.dofs_prev, H.dofs_pp, H.w_dofs,
                     H.w_trial, H.R, H.R_trial, H.vals, H.vals_trial, H.kappa_trial, H.kappa_trial2, H.loading,
                     H.loading2, H.counters, H.diag, H.binv, H.vals_f32, H.kx, H.red, H.scal};
     for (void *p : ptrs) dfree(p);
@@ -138,10 +138,10 @@ void free_handle(gd::Handle &H)
         for (void *p : cp) dfree(p);
     }
     for (gd::DevNet &n : H.h_psi_tab) {
-        dfree(n.p); dfree(n.W2T); dfree(n.pf); dfree(n.W2Tf);
+        dfree(n.p); dfree(n.W2T); dfree(n.pf); dfree(n.W2Tf); dfree(n.fx);
     }
     for (gd::DevNet &n : H.h_yld_tab) {
-        dfree(n.p); dfree(n.W2T); dfree(n.pf); dfree(n.W2Tf);
+        dfree(n.p); dfree(n.W2T); dfree(n.pf); dfree(n.W2Tf); dfree(n.fx);
     }
     if (H.ev0) cudaEventDestroy(H.ev0);
     if (H.ev1) cudaEventDestroy(H.ev1);
@@ -1479,9 +1479,11 @@ static gd_status stage_net(gd::Handle &H, gd::DevNet &d, int n_in, int w, const 
     GD_CUDA(&H, dalloc(&d.W2T, (size_t)w * w));
     GD_CUDA(&H, dalloc(&d.pf, d.n_params));
     GD_CUDA(&H, dalloc(&d.W2Tf, (size_t)w * w));
+    GD_CUDA(&H, dalloc(&d.fx, gd::net_fixed_bytes(w)));
     GD_CUDA(&H, cudaMemcpyAsync(d.p, params, sizeof(double) * d.n_params, cudaMemcpyDefault, H.stream));
     GD_CUDA(&H, gd::launch_transpose(d, H.stream));
     GD_CUDA(&H, gd::launch_net_to_float(d, H.stream));
+    GD_CUDA(&H, gd::launch_net_fixed(d, H.stream));
     return GD_OK;
 }
 
@@ -1951,11 +1953,13 @@ gd_status gd_set_params(gd_handle *h, const double *theta_psi, const double *the
         GD_CUDA(&H, cudaMemcpyAsync(H.psi.p, theta_psi, sizeof(double) * H.psi.n_params, cudaMemcpyDefault, H.stream));
         GD_CUDA(&H, gd::launch_transpose(H.psi, H.stream));
         GD_CUDA(&H, gd::launch_net_to_float(H.psi, H.stream));
+        GD_CUDA(&H, gd::launch_net_fixed(H.psi, H.stream));
     }
     if (theta_yield && H.yld.width > 0) {
         GD_CUDA(&H, cudaMemcpyAsync(H.yld.p, theta_yield, sizeof(double) * H.yld.n_params, cudaMemcpyDefault, H.stream));
         GD_CUDA(&H, gd::launch_transpose(H.yld, H.stream));
         GD_CUDA(&H, gd::launch_net_to_float(H.yld, H.stream));
+        GD_CUDA(&H, gd::launch_net_fixed(H.yld, H.stream));
     }
     GD_CUDA(&H, gd::launch_prep_nets(H.psi, H.yld, H.mat.energy, H.netc, H.stream));
     if (H.tc_blob) GD_CUDA(&H, gd::tc_build_blob(H.psi, H.yld, H.tc, H.tc_blob, H.stream));

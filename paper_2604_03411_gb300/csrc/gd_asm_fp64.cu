@@ -1,17 +1,33 @@
 // gd_asm_fp64.cu -- FP64 element kernel of the gradient-enhanced damage model.
 //
-// One warp owns a batch of 32 quadrature points (4 HEX8 or 8 Q4 elements) and
-// switches between three lane mappings:
-//   qp mode    lane = quadrature point: kinematics, invariants, energy chain,
-//              stress and the per-point records of the tangent;
-//   unit mode  lane = network unit, one point at a time: both ICNN layers of the
-//              energy network (value, gradient by forward tangents, Hessian by
-//              one reverse sweep through layer 2) and every yield-network
-//              evaluation of the local damage solve, so the per-point iteration
-//              counts cost no divergence;
-//   row mode   lane = element row (node a, dof i): the row of the consistent
-//              tangent and of the residual, accumulated over the points of one
-//              element and scattered into CSR through the slot map.
+// A CTA of KW warps owns 8 KW quadrature points (KW HEX8 or 2 KW Q4 elements) and switches
+// between three lane mappings:
+//   qp mode    lane = quadrature point (the first 8 KW threads in an order that rotates
+//              with the batch): kinematics, invariants, energy chain, stress and the
+//              point's tangent in reference coordinates;
+//   net mode   warp = eight points, four lanes each: both ICNN layers of the energy
+//              network (value, gradient by forward tangents, Hessian by one reverse sweep
+//              through layer 2) and every yield-network evaluation of the local damage
+//              solve, whose points iterate in lockstep (gd_net_fp64.cuh);
+//   row mode   warp = its eight points' elements, lane = element row (node a, dof i): the
+//              rows of the residual and of the consistent tangent, scattered into CSR
+//              through the slot map.
+//
+// The FP64 pipe bounds the kernel (1.7 lanes per clock and SM), so the design spends as few
+// FP64 operations as it can:
+//  - The point's tangent is formed once per point as the derivative D of (P, Y vector, -Y)
+//    with respect to (grad u, grad phi, phi), both gradients pulled back to the reference
+//    element and weighted by J w, and a row of the element matrix is
+//    K_(a,i),(b,k) = sum_q sum_jl dN_a/dxi_j D_(ij),(kl) dN_b/dxi_l: 3 multiply-adds per
+//    entry of D and row, and the sum over the points and dN_b/dxi_l factorised over the axes
+//    (their values are products of (1 +- 1/sqrt 3) / 2): 20 instead of 64 operations per
+//    derivative and column.  About 100 operations per row and point, against 700 for the
+//    closed form of every (a, b) pair.
+//  - The networks run in 64-bit fixed point (gd_fixed.cuh).
+// Measured (GB300, gd_assemble with tangent; before: FP64 networks one point at a time with
+// a lane per unit, closed-form rows): 140,400 points of HEX8, both widths 64, 33.6 -> 7.5 ms;
+// 159,744 of Q4, widths 32, 10.1 -> 2.4 ms; 256 of Q4, widths 16 and 8, 1.24 -> 0.10 ms;
+// residual alone of 32,640 HEX8 points, widths 24 and 40, 3.55 -> 0.63 ms.
 //
 // Paper passages: Sec. 3.1 (F, phi_q, grad phi_q, element residual, Table
 // kernel_inputs), Sec. 2.1 (P, Y vector, Y), Sec. 2.2 and Sec. 3.2 Eq. (dd_7_no_nn)
@@ -22,6 +38,7 @@
 
 #include "gd_elem32.cuh"
 #include "gd_internal.cuh"
+#include "gd_net_fp64.cuh"
 
 namespace gd {
 namespace {
@@ -33,159 +50,507 @@ constexpr double kTrialMargin = 1e-4;
 
 #include "gd_device_fp64.cuh"
 
-// KW warps per CTA (a tuning choice: warps are independent, so it only sets the
-// granularity of residency and of the persistent grid)
+// Record of a quadrature point for the row mode, in doubles: every quantity pulled back to
+// the reference element and times J w.
+template <int DIM>
+struct Rec {
+    static constexpr int N2 = DIM * DIM, NS = DIM * (DIM + 1) / 2;
+    static constexpr int A = 0;                      // d P_ij / d H_kl, symmetric, packed upper triangle of (ij) x (kl)
+    static constexpr int B = A + N2 * (N2 + 1) / 2;  // d P_ij / d g_l [ij][l]
+    static constexpr int CV = B + N2 * DIM;          // c_d C^-1, packed symmetric
+    static constexpr int PE = CV + NS;               // dpsi_e/dF (undamaged, without J w) [ij]
+    static constexpr int P = PE + N2;                // stress [ij]
+    static constexpr int Y = P + N2;                 // flux [j]
+    static constexpr int FDK = Y + DIM;              // f_d' dkappa/dphi
+    static constexpr int BCK = FDK + 1;              // beta_d c_kappa
+    static constexpr int PP = BCK + 1;               // beta_d (1 - dkappa/dphi)
+    static constexpr int PEN = PP + 1;               // beta_d (phi - kappa)
+    static constexpr int SIZE = (PEN + 1) | 1;       // odd stride: one bank pair per point
+};
+// position of (r, c) in a packed symmetric N x N matrix (upper triangle by rows)
+template <int N>
+__device__ __forceinline__ int sym_pos(int r, int c)
+{
+    const int lo = r < c ? r : c, hi = r < c ? c : r;
+    return lo * N - lo * (lo - 1) / 2 + hi - lo;
+}
+
+// shared-memory layout of a CTA of KW warps, in doubles
 template <int DIM, int KW>
-__global__ void __launch_bounds__(32 * KW) asm_fp64_kernel(AsmArgs A)
+struct Smem {
+    using G_ = Geo<DIM>;
+    static constexpr int NP = 8 * KW, EL = NP / G_::NQ;
+    static constexpr int X = 0;                                      // [EL][NEN][DIM]
+    static constexpr int D = X + EL * G_::NEN * DIM;                 // [EL][NEN][NDOF]
+    static constexpr int REF = D + EL * G_::NEN * G_::NDOF;          // [NQ][NEN][4] dN/dxi, N
+    static constexpr int IN = REF + G_::NQ * G_::NEN * 4;            // [NP][4] network input / psi_e, phi, kappa_n
+    static constexpr int OUT = IN + NP * 4;                          // [NP][10] network output / local update
+    static constexpr int U = OUT + NP * 10;                          // network buffers, then the points' records
+    __host__ __device__ static int net(int wmax) { return (int)(grp::buf_bytes(wmax) / 8); }
+    __host__ __device__ static int total(int wmax)
+    {
+        const int n = KW * net(wmax), r = NP * Rec<DIM>::SIZE;
+        return U + ((n > r ? n : r) + 1) / 2 * 2;
+    }
+};
+template <int KW>
+__device__ __forceinline__ void cta_sync()
+{
+    if (KW == 1) __syncwarp();
+    else __syncthreads();
+}
+
+constexpr double kNp = 0.5 * (1.0 + kGauss), kNm = 0.5 * (1.0 - kGauss);   // 1D shape functions at the Gauss points
+
+// out[b] = sum_q sum_l T[l][q] dN_b/dxi_l(q) (+ sum_q TN[q] N_b(q)), b and q numbered by
+// their axis bits (x lowest).  One axis at a time: the derivative's axis sums its two points,
+// the others mix them with (1 +- 1/sqrt 3) / 2.
+template <bool NPART>
+__device__ __forceinline__ void expand_rows(const double (&T)[2][4], const double *TN, double (&out)[4])
+{
+    // x derivative: S(y), then the y axis; y derivative: S(x), then the x axis
+    const double sx0 = T[0][0] + T[0][1], sx1 = T[0][2] + T[0][3];
+    const double sy0 = T[1][0] + T[1][2], sy1 = T[1][1] + T[1][3];
+    const double hp = 0.5 * kNp, hm = 0.5 * kNm;
+    const double qx0 = hp * sx0 + hm * sx1, qx1 = hm * sx0 + hp * sx1;       // by = 0, 1
+    const double qy0 = hp * sy0 + hm * sy1, qy1 = hm * sy0 + hp * sy1;       // bx = 0, 1
+    out[0] = -qx0 - qy0;
+    out[1] = qx0 - qy1;
+    out[2] = qy0 - qx1;
+    out[3] = qx1 + qy1;
+    if (NPART) {
+        const double a0 = kNp * TN[0] + kNm * TN[1], a1 = kNm * TN[0] + kNp * TN[1];
+        const double b0 = kNp * TN[2] + kNm * TN[3], b1 = kNm * TN[2] + kNp * TN[3];
+        out[0] += kNp * a0 + kNm * b0;
+        out[1] += kNp * a1 + kNm * b1;
+        out[2] += kNm * a0 + kNp * b0;
+        out[3] += kNm * a1 + kNp * b1;
+    }
+}
+template <bool NPART>
+__device__ __forceinline__ void expand_rows(const double (&T)[3][8], const double *TN, double (&out)[8])
+{
+    const double hp = 0.5 * kNp, hm = 0.5 * kNm;
+    double Q[3][4];                      // derivative along axis l; the other two axes (lower first)
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+        const int u = l == 0 ? 1 : 0, v = l == 2 ? 1 : 2;
+        double s[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int q0 = ((m & 1) << u) | ((m >> 1) << v);
+            s[m] = T[l][q0] + T[l][q0 | (1 << l)];
+        }
+        const double a0 = hp * s[0] + hm * s[1], a1 = hm * s[0] + hp * s[1];
+        const double b0 = hp * s[2] + hm * s[3], b1 = hm * s[2] + hp * s[3];
+        Q[l][0] = kNp * a0 + kNm * b0;
+        Q[l][1] = kNp * a1 + kNm * b1;
+        Q[l][2] = kNm * a0 + kNp * b0;
+        Q[l][3] = kNm * a1 + kNp * b1;
+    }
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const int bx = b & 1, by = (b >> 1) & 1, bz = b >> 2;
+        const double x = Q[0][by | (bz << 1)], y = Q[1][bx | (bz << 1)], z = Q[2][bx | (by << 1)];
+        const double xy = (bx == by) ? x + y : x - y;        // sign of x times the sum
+        out[b] = (bx ? xy : -xy) + (bz ? z : -z);
+    }
+    if (NPART) {
+        double a[8], c[8];
+#pragma unroll
+        for (int q = 0; q < 8; q += 2) {
+            a[q] = kNp * TN[q] + kNm * TN[q + 1];
+            a[q + 1] = kNm * TN[q] + kNp * TN[q + 1];
+        }
+#pragma unroll
+        for (int z = 0; z < 8; z += 4)
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                c[z + x] = kNp * a[z + x] + kNm * a[z + x + 2];
+                c[z + x + 2] = kNm * a[z + x] + kNp * a[z + x + 2];
+            }
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            out[b] += kNp * c[b] + kNm * c[b + 4];
+            out[b + 4] += kNm * c[b] + kNp * c[b + 4];
+        }
+    }
+}
+// node with the axis bits l (x lowest): counter-clockwise numbering of each layer
+__device__ __forceinline__ int node_of_bits(int l) { return l ^ ((l >> 1) & 1); }
+
+// Local damage update (Eq. (dd_7_no_nn)) of the points p0 .. p0 + 7 of the warp's batch that
+// belong to specimen sn: psi_e, phi, kappa_n at sIn[p 4 ..], results (kappa, loading, G',
+// dPhi/dkappa, failed) to sOut[p 10 ..].  Four lanes hold each point's state; the points step
+// together, every evaluation running for the points that still need it.  Returns the
+// lane's share of the FP64 evaluations.
+template <int DIM>
+__device__ __forceinline__ int local_update(const AsmArgs &A, const e32::MatF &mf, int64_t e0, int p0, int sn,
+                                            const double *sIn, double *sOut, unsigned char *nbuf, int lane)
+{
+    constexpr int NQ = Geo<DIM>::NQ;
+    constexpr unsigned kAll = 0xffffffffu;
+    const int p = p0 + (lane >> 2);
+    const int64_t e_p = e0 + p / NQ;
+    const bool need = e_p < A.n_elems && spec_of(A, e_p < A.n_elems ? e_p : A.n_elems - 1) == sn;
+    const DevNet &yn = yld_of(A, sn);
+    const NetConst nc = A.netc[sn];
+    const e32::NcF nf = e32::ncf(nc);
+    const int local_max = A.mat.local_max;
+    const double pe = sIn[p * 4], phi = sIn[p * 4 + 1], kn = sIn[p * 4 + 2];
+    const float pef = (float)pe, phf = (float)phi, knf = (float)kn;
+    double kappa = kn, r = 0.0, dr = -1.0, Gp = 0.0;
+    bool fail = false;
+    int n_eval = 0;
+    // Trial Phi_d(kappa_n): the FP32 network decides points clearly off the yield
+    // surface, an FP64 evaluation the others.
+    float r32, dr32, Gp32;
+    grp::residual32(mf, yn, nf, pef, phf, knf, r32, dr32, Gp32, nbuf, lane);
+    const double scale_n = fabs(kn) > 1.0 ? fabs(kn) : 1.0;
+    bool load = need && r32 > 0.0f;
+    const bool close = need && !(fabs((double)r32) > kTrialMargin * scale_n);
+    if (__any_sync(kAll, close)) {
+        double rt, drt, gt;
+        grp::residual<true>(A.mat, yn, nc, pe, phi, kn, rt, drt, gt, nbuf, lane, close);
+        if (close) {
+            ++n_eval;
+            r = rt;
+            dr = drt;
+            Gp = gt;
+            load = rt > 0.0;
+            r32 = (float)rt;
+            dr32 = (float)drt;
+        }
+    }
+    // The root in FP32 (the lazily bracketed Newton iteration of the mixed kernels, from the
+    // warm start), then FP64: one value-only evaluation and a Newton step with the FP32 slope
+    // (its relative error, ~1e-7, times a correction of ~1e-6 leaves ~1e-13), then one full
+    // evaluation and a last Newton step; the slope and G' of that evaluation feed the tangent
+    // (they change by ~1e-12 relative over the last step).  Where the FP32 root is not close
+    // enough, the FP64 bracketed iteration takes over from it.  Both iterations also stop on
+    // the next Newton correction |r / r'| (the step test of the safeguarded Newton-bisection;
+    // FP32: 2e-6 relative, FP64: 4 ulp) once the root is bracketed within 1e-2 relative or the
+    // iteration converges from one side: near full damage r' grows like 1 / f_d, and r itself
+    // cannot get below its rounding.  (A wide bracket does not qualify: far past the root,
+    // where f_d underflows, r' is huge and the correction meaningless.)
+    float k32 = knf;
+    bool ok32 = false;
+    if (__any_sync(kAll, load)) {
+        const float kg = load && A.kappa_guess ? (float)__ldg(A.kappa_guess + e0 * NQ + p) : knf;
+        bool run = load, warm = load && kg > knf && isfinite(kg);
+        float lo = knf, hi = knf, dx = 1.0e30f, dx_prev = 1.0e30f;
+        bool have_hi = false, took_newton = false;
+        int it = 0;
+        if (warm) k32 = kg;
+        else if (r32 > 0.0f) lo = k32;
+        else {
+            hi = k32;
+            have_hi = true;
+            dx = dx_prev = hi - lo;
+        }
+        while (__any_sync(kAll, run)) {
+            if (run && !warm) {
+                const float scale = fabsf(k32) > 1.0f ? fabsf(k32) : 1.0f;
+                if (it >= local_max) {
+                    run = false;
+                } else if (fabsf(r32) <= 2e-6f * scale || (have_hi && (hi - lo) <= 4.0f * e32::kEpsF * scale) ||
+                           (fabsf(r32) <= 2e-6f * scale * fabsf(dr32) &&
+                            (have_hi ? (hi - lo) <= 1e-2f * scale
+                                     : (took_newton && fabsf(2.0f * r32) <= fabsf(dx * dr32))))) {
+                    run = false;
+                    ok32 = true;
+                } else {
+                    const float newton = k32 - r32 / dr32;
+                    const float rr = r32 > 1e-12f ? r32 : 1e-12f;
+                    bool take;
+                    if (have_hi) take = newton > lo && newton < hi && fabsf(2.0f * r32) <= fabsf(dx_prev * dr32);
+                    else take = dr32 < 0.0f && newton > lo && (newton - k32) <= 4.0f * (rr + (k32 - knf));
+                    dx_prev = dx;
+                    took_newton = take;
+                    if (take) {
+                        dx = k32 - newton;
+                        k32 = newton;
+                    } else if (have_hi) {
+                        dx = 0.5f * (hi - lo);
+                        k32 = lo + dx;
+                    } else {
+                        dx = 2.0f * ((k32 - knf) > rr ? (k32 - knf) : rr);
+                        k32 = lo + dx;
+                    }
+                }
+            }
+            if (!__any_sync(kAll, run)) break;
+            float re, dre, ge;
+            grp::residual32(mf, yn, nf, pef, phf, k32, re, dre, ge, nbuf, lane);
+            if (run) {
+                r32 = re;
+                dr32 = dre;
+                if (r32 > 0.0f) lo = k32;
+                else {
+                    hi = k32;
+                    have_hi = true;
+                }
+                if (warm) {
+                    warm = false;
+                    dx = dx_prev = have_hi ? hi - lo : 1.0e30f;
+                } else {
+                    ++it;
+                }
+            }
+        }
+    }
+    bool polish = load && ok32 && isfinite(k32) && (double)k32 >= kn && dr32 < 0.0f;
+    bool done = !load;
+    if (__any_sync(kAll, polish)) {
+        const double sc = fabs((double)k32) > 1.0 ? fabs((double)k32) : 1.0;
+        double r0, d0, g0;
+        grp::residual<false>(A.mat, yn, nc, pe, phi, (double)k32, r0, d0, g0, nbuf, lane, polish);
+        if (polish) ++n_eval;
+        polish = polish && fabs(r0) <= 1e-4 * sc;
+        const double k1 = polish ? (double)k32 - r0 / (double)dr32 : kn;
+        grp::residual<true>(A.mat, yn, nc, pe, phi, k1, r0, d0, g0, nbuf, lane, polish);
+        if (polish) {
+            ++n_eval;
+            r = r0;
+            dr = d0;
+            Gp = g0;
+            if (k1 >= kn && fabs(r) <= 1e-9 * sc && dr < 0.0) {
+                const double k2 = fabs(r) <= 1e-13 * sc ? k1 : k1 - r / dr;
+                kappa = k2 >= kn ? k2 : kn;
+                done = true;
+            }
+        }
+    }
+    if (__any_sync(kAll, !done)) {
+        // FP64 lazily bracketed Newton iteration from kappa_n, then the FP32 result (the
+        // iteration of the FP64 reference path)
+        const double kgd = isfinite(k32) ? (double)k32 : kn;
+        bool run = !done, ok = done;
+        int stage = kgd > kn ? 0 : 1;        // 0: at kappa_n, a guess follows; 1: first point; 2: iterating
+        double lo = kn, hi = kn, dx = 1.0e30, dx_prev = 1.0e30;
+        bool have_hi = false, took_newton = false;
+        int it = 0;
+        while (__any_sync(kAll, run)) {
+            double re, dre, ge;
+            grp::residual<true>(A.mat, yn, nc, pe, phi, kappa, re, dre, ge, nbuf, lane, run);
+            if (run) {
+                ++n_eval;
+                r = re;
+                dr = dre;
+                Gp = ge;
+                if (stage == 0) {
+                    kappa = kgd;
+                    stage = 1;
+                    continue;
+                }
+                if (r > 0.0) lo = kappa;
+                else {
+                    hi = kappa;
+                    have_hi = true;
+                }
+                if (stage == 1) {
+                    dx = dx_prev = have_hi ? hi - lo : 1.0e30;
+                    stage = 2;
+                } else {
+                    ++it;
+                }
+                const double scale = fabs(kappa) > 1.0 ? fabs(kappa) : 1.0;
+                const double ulp4 = 4.0 * 2.220446049250313e-16 * scale;
+                if (it >= local_max) {
+                    run = false;
+                } else if (fabs(r) <= 1e-13 * scale || (have_hi && (hi - lo) <= ulp4) ||
+                           (fabs(r) <= ulp4 * fabs(dr) &&
+                            (have_hi ? (hi - lo) <= 1e-2 * scale : (took_newton && fabs(2.0 * r) <= fabs(dx * dr))))) {
+                    run = false;
+                    ok = true;
+                } else {
+                    const double newton = kappa - r / dr;
+                    const double rr = r > 1e-12 ? r : 1e-12;
+                    bool take;
+                    if (have_hi) take = newton > lo && newton < hi && fabs(2.0 * r) <= fabs(dx_prev * dr);
+                    // forward Newton step, at most a few times the distance covered so far
+                    else take = dr < 0.0 && newton > lo && (newton - kappa) <= 4.0 * (rr + (kappa - kn));
+                    dx_prev = dx;
+                    took_newton = take;
+                    if (take) {
+                        dx = kappa - newton;
+                        kappa = newton;
+                    } else if (have_hi) {
+                        dx = 0.5 * (hi - lo);
+                        kappa = lo + dx;
+                    } else {
+                        dx = 2.0 * ((kappa - kn) > rr ? (kappa - kn) : rr);
+                        kappa = lo + dx;
+                    }
+                }
+            }
+        }
+        if (!ok) fail = true;
+    }
+    if (need && (lane & 3) == 0) {
+        double *o = sOut + p * 10;
+        o[0] = kappa;
+        o[1] = load ? 1.0 : 0.0;
+        o[2] = Gp;
+        o[3] = dr;
+        o[4] = fail ? 1.0 : 0.0;
+    }
+    return (lane & 3) == 0 ? n_eval : 0;
+}
+
+// KW warps per CTA, eight points each (a launch-shape choice: see launch_dim)
+template <int DIM, int KW>
+__global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
 {
     using G_ = Geo<DIM>;
-    constexpr int NEN = G_::NEN, NQ = G_::NQ, NDOF = G_::NDOF, ND = G_::ND, EPW = G_::EPW, EPR = G_::EPR;
-    extern __shared__ double smem[];
+    using S_ = Smem<DIM, KW>;
+    using R_ = Rec<DIM>;
+    constexpr int NEN = G_::NEN, NQ = G_::NQ, NDOF = G_::NDOF, NP = S_::NP, EL = S_::EL, N2 = DIM * DIM;
+    extern __shared__ __align__(16) double smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int wmax = A.wmax;
-    // per-warp scratch
-    const int scratch = EPW * NEN * (DIM + NDOF) + 32 * Q_REC + 32 * 4 + 32 * 10 + 5 * wmax + 2 * NQ * NEN * V_REC;
-    double *ws = smem + warp * scratch;
-    double *sX = ws;                                  // [EPW][NEN][DIM]
-    double *sD = sX + EPW * NEN * DIM;                // [EPW][NEN][NDOF]
-    double *sRec = sD + EPW * NEN * NDOF;             // [32][Q_REC]
-    double *sIn = sRec + 32 * Q_REC;                  // [32][4]: network input x (3), then kappa out
-    double *sOut = sIn + 32 * 4;                      // [32][10]: N, grad, Hess / local-solve results
-    double *sBuf = sOut + 32 * 10;                    // unit-mode buffers
-    double *sVec = sBuf + 5 * wmax;                   // [EPR*NQ*NEN][V_REC]
+    double *sX = smem + S_::X, *sD = smem + S_::D, *sRef = smem + S_::REF, *sIn = smem + S_::IN, *sOut = smem + S_::OUT;
+    double *sRec = smem + S_::U;
+    unsigned char *nbuf = reinterpret_cast<unsigned char *>(smem + S_::U + warp * S_::net(A.wmax));
     const MatConst &m = A.mat;
+    for (int t = threadIdx.x; t < NQ * NEN; t += 32 * KW) {
+        const int qq = t / NEN, a = t % NEN;
+        const double xi[3] = {(qq & 1) ? kGauss : -kGauss, (qq & 2) ? kGauss : -kGauss, (qq & 4) ? kGauss : -kGauss};
+        double N, dN[3] = {0.0, 0.0, 0.0};
+        ref_shape<DIM>(a, xi, N, dN);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) sRef[t * 4 + k] = dN[k];
+        sRef[t * 4 + 3] = N;
+    }
+    const int64_t e_last = A.n_elems - 1;
 
-    const int64_t n_batches = (A.n_elems + EPW - 1) / EPW;
-    for (int64_t batch = (int64_t)blockIdx.x * KW + warp; batch < n_batches;
-         batch += (int64_t)gridDim.x * KW) {
-        const int64_t e0 = batch * EPW;
-        // ---- load element nodes (lane = (element, node)) ----
-        for (int t = lane; t < EPW * NEN; t += 32) {
-            int el = t / NEN, a = t % NEN;
-            int64_t e = e0 + el;
+    const int64_t n_batches = (A.n_elems + EL - 1) / EL;
+    for (int64_t batch = blockIdx.x; batch < n_batches; batch += gridDim.x) {
+        const int64_t e0 = batch * EL;
+        cta_sync<KW>();
+        for (int t = threadIdx.x; t < EL * NEN; t += 32 * KW) {
+            const int64_t e = e0 + t / NEN;
             if (e < A.n_elems) {
-                int32_t n = __ldg(A.conn + e * NEN + a);
+                const int32_t n = __ldg(A.conn + e * NEN + t % NEN);
 #pragma unroll
                 for (int J = 0; J < DIM; ++J) sX[t * DIM + J] = __ldg(A.X + (int64_t)n * DIM + J);
 #pragma unroll
                 for (int c = 0; c < NDOF; ++c) sD[t * NDOF + c] = __ldg(A.dofs + (int64_t)n * NDOF + c);
             } else {
+                // a unit element without displacement
+                const int a = t % NEN;
 #pragma unroll
-                for (int J = 0; J < DIM; ++J) sX[t * DIM + J] = (a & 1) ? 1.0 : 0.0;
+                for (int J = 0; J < DIM; ++J) sX[t * DIM + J] = node_sgn(a, J) > 0.0 ? 1.0 : 0.0;
 #pragma unroll
                 for (int c = 0; c < NDOF; ++c) sD[t * NDOF + c] = 0.0;
             }
         }
-        __syncwarp();
+        cta_sync<KW>();
 
         // ================= qp mode: kinematics and invariants =================
-        const int el = lane / NQ, q = lane % NQ;
+        // the threads that hold the points move on by one warp per batch, so that the SM's
+        // four quarters share this mode's FP64 work
+        const int pt = (threadIdx.x + 32 * (int)((batch / gridDim.x + blockIdx.x) % KW)) % (32 * KW);
+        const bool qp = pt < NP;
+        const int el = pt / NQ, q = pt % NQ;
         const int64_t e_me = e0 + el;
-        const bool valid = e_me < A.n_elems;
-        const NetConst nc = A.netc[valid ? spec_of(A, e_me) : 0];
-        double *rec = sRec + lane * Q_REC;
-        double F[3][3], H[3][3], phi = 0.0, g[3] = {0.0, 0.0, 0.0}, x[3], Jdet;
-        {
-            const double xi[3] = {(q & 1) ? kGauss : -kGauss, (q & 2) ? kGauss : -kGauss,
-                                  (q & 4) ? kGauss : -kGauss};
-            const double *Xe = sX + el * NEN * DIM;
-            const double *De = sD + el * NEN * NDOF;
-            double Jm[3][3] = {{0.0}};
+        const bool valid = qp && e_me < A.n_elems;
+        const double *ref = sRef + q * NEN * 4;
+        double F[DIM][DIM], Ji[DIM][DIM], gx[DIM], x[3], phi = 0.0, det = 1.0, Jdet = 1.0;
+        double Tm[3][3], T2[3][6];   // dy/dx and d2y/dx2 of the network input map (raw: identity)
+        if (qp) {
+            const double *Xe = sX + el * NEN * DIM, *De = sD + el * NEN * NDOF;
+            double Jm[DIM][DIM], Gr[DIM][DIM];
+#pragma unroll
+            for (int i = 0; i < DIM; ++i) {
+                gx[i] = 0.0;
+#pragma unroll
+                for (int k = 0; k < DIM; ++k) Jm[i][k] = Gr[i][k] = 0.0;
+            }
 #pragma unroll
             for (int a = 0; a < NEN; ++a) {
-                double Na, dN[3];
-                ref_shape<DIM>(a, xi, Na, dN);
 #pragma unroll
-                for (int J = 0; J < DIM; ++J)
+                for (int k = 0; k < DIM; ++k) {
+                    const double dN = ref[a * 4 + k];
 #pragma unroll
-                    for (int k = 0; k < DIM; ++k) Jm[J][k] += Xe[a * DIM + J] * dN[k];
+                    for (int J = 0; J < DIM; ++J) {
+                        Jm[J][k] += Xe[a * DIM + J] * dN;
+                        Gr[J][k] += De[a * NDOF + J] * dN;
+                    }
+                    gx[k] += De[a * NDOF + DIM] * dN;
+                }
+                phi += De[a * NDOF + DIM] * ref[a * 4 + 3];
             }
-            double Ji[3][3] = {{0.0}}, det;
             if (DIM == 2) {
                 det = Jm[0][0] * Jm[1][1] - Jm[0][1] * Jm[1][0];
-                Ji[0][0] = Jm[1][1] / det; Ji[0][1] = -Jm[0][1] / det;
-                Ji[1][0] = -Jm[1][0] / det; Ji[1][1] = Jm[0][0] / det;
+                const double di = 1.0 / det;
+                Ji[0][0] = Jm[1][1] * di; Ji[0][1] = -Jm[0][1] * di;
+                Ji[1][0] = -Jm[1][0] * di; Ji[1][1] = Jm[0][0] * di;
             } else {
 #pragma unroll
-                for (int i = 0; i < 3; ++i)
+                for (int i = 0; i < DIM; ++i)
 #pragma unroll
-                    for (int j = 0; j < 3; ++j) {
-                        int i1 = (j + 1) % 3, i2 = (j + 2) % 3, j1 = (i + 1) % 3, j2 = (i + 2) % 3;
+                    for (int j = 0; j < DIM; ++j) {
+                        const int i1 = (j + 1) % DIM, i2 = (j + 2) % DIM, j1 = (i + 1) % DIM, j2 = (i + 2) % DIM;
                         Ji[i][j] = Jm[i1][j1] * Jm[i2][j2] - Jm[i1][j2] * Jm[i2][j1];
                     }
-                det = Jm[0][0] * Ji[0][0] + Jm[0][1] * Ji[1][0] + Jm[0][2] * Ji[2][0];
+                det = 0.0;
 #pragma unroll
-                for (int i = 0; i < 3; ++i)
+                for (int k = 0; k < DIM; ++k) det += Jm[0][k] * Ji[k][0];
+                const double di = 1.0 / det;
 #pragma unroll
-                    for (int j = 0; j < 3; ++j) Ji[i][j] /= det;
+                for (int i = 0; i < DIM; ++i)
+#pragma unroll
+                    for (int j = 0; j < DIM; ++j) Ji[i][j] *= di;
             }
-            rec[Q_JW] = det;
+            // H = grad u; C - I = H + H^T + H^T H; invariants without cancellation
+            double H[DIM][DIM];
 #pragma unroll
-            for (int k = 0; k < 9; ++k) rec[Q_JINV + k] = Ji[k / 3][k % 3];
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int J = 0; J < 3; ++J) H[i][J] = 0.0;
-#pragma unroll
-            for (int a = 0; a < NEN; ++a) {
-                double Na, dN[3], n[3] = {0.0, 0.0, 0.0};
-                ref_shape<DIM>(a, xi, Na, dN);
-#pragma unroll
-                for (int J = 0; J < DIM; ++J)
-#pragma unroll
-                    for (int k = 0; k < DIM; ++k) n[J] += dN[k] * Ji[k][J];
-                const double pa = De[a * NDOF + DIM];
-                phi += Na * pa;
+            for (int i = 0; i < DIM; ++i)
 #pragma unroll
                 for (int J = 0; J < DIM; ++J) {
-                    g[J] += pa * n[J];
+                    double s = 0.0;
 #pragma unroll
-                    for (int i = 0; i < DIM; ++i) H[i][J] += De[a * NDOF + i] * n[J];
+                    for (int k = 0; k < DIM; ++k) s += Gr[i][k] * Ji[k][J];
+                    H[i][J] = s;
+                    F[i][J] = i == J ? s + 1.0 : s;
                 }
-            }
-            // C - I = H + H^T + H^T H ; invariants without cancellation
-            double Am[3][3];
+            double tA = 0.0, AA = 0.0, tH = 0.0, HH = 0.0;
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
+            for (int i = 0; i < DIM; ++i) {
+                tH += H[i][i];
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
+                for (int j = i; j < DIM; ++j) {
                     double s = H[i][j] + H[j][i];
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) s += H[k][i] * H[k][j];
-                    Am[i][j] = s;
+                    for (int k = 0; k < DIM; ++k) s += H[k][i] * H[k][j];
+                    if (i == j) {
+                        tA += s;
+                        AA += s * s;
+                        HH += H[i][i] * H[i][i];
+                    } else {
+                        AA += 2.0 * s * s;
+                        HH += 2.0 * H[i][j] * H[j][i];
+                    }
                 }
-            double tA = Am[0][0] + Am[1][1] + Am[2][2], AA = 0.0, tH = H[0][0] + H[1][1] + H[2][2], HH = 0.0;
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    AA += Am[i][j] * Am[j][i];
-                    HH += H[i][j] * H[j][i];
-                }
-            double detH = H[0][0] * (H[1][1] * H[2][2] - H[1][2] * H[2][1]) -
-                          H[0][1] * (H[1][0] * H[2][2] - H[1][2] * H[2][0]) +
-                          H[0][2] * (H[1][0] * H[2][1] - H[1][1] * H[2][0]);
+            }
             x[0] = tA;
             x[1] = 2.0 * tA + 0.5 * (tA * tA - AA);
-            x[2] = tH + 0.5 * (tH * tH - HH) + detH;
+            x[2] = tH + 0.5 * (tH * tH - HH);
+            if constexpr (DIM == 3)
+                x[2] += H[0][0] * (H[1][1] * H[2][2] - H[1][2] * H[2][1]) -
+                        H[0][1] * (H[1][0] * H[2][2] - H[1][2] * H[2][0]) +
+                        H[0][2] * (H[1][0] * H[2][1] - H[1][1] * H[2][0]);
             Jdet = 1.0 + x[2];
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) F[i][j] = H[i][j] + (i == j ? 1.0 : 0.0);
-        }
-        // network input (raw or isochoric map)
-        double Tm[3][3], T2[3][6];   // dy/dx and d2y/dx2 of the iso map (raw: identity)
-        {
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-#pragma unroll
-                for (int j = 0; j < 3; ++j) Tm[i][j] = (i == j) ? 1.0 : 0.0;
-#pragma unroll
-                for (int j = 0; j < 6; ++j) T2[i][j] = 0.0;
-            }
+            // network input (raw or isochoric map)
             double y[3] = {x[0], x[1], x[2]};
             if (m.energy == GD_ENERGY_ICNN_ISO) {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) Tm[i][j] = (i == j) ? 1.0 : 0.0;
+#pragma unroll
+                    for (int j = 0; j < 6; ++j) T2[i][j] = 0.0;
+                }
                 // I1G = J^-2/3 I1, I2G = I2^3 / (9 J^4) (Eq. (dd_0)); derivatives wrt (I1-3, I2-3, J-1)
                 double L = log1p(x[2]), E = exp(-2.0 / 3.0 * L), I1 = 3.0 + x[0], I2 = 3.0 + x[1], J = Jdet;
                 y[0] = 3.0 * expm1(-2.0 / 3.0 * L) + x[0] * E;
@@ -201,29 +566,35 @@ __global__ void __launch_bounds__(32 * KW) asm_fp64_kernel(AsmArgs A)
                 T2[1][4] = -4.0 * I2 * I2 / (3.0 * J4 * J);          // d2 y2 / dx2 dx3
                 T2[1][5] = 20.0 * I2 * I2 * I2 / (9.0 * J4 * J * J); // d2 y2 / dx3^2
             }
-            sIn[lane * 4 + 0] = y[0];
-            sIn[lane * 4 + 1] = y[1];
-            sIn[lane * 4 + 2] = y[2];
+            sIn[pt * 4 + 0] = y[0];
+            sIn[pt * 4 + 1] = y[1];
+            sIn[pt * 4 + 2] = y[2];
         }
-        __syncwarp();
+        cta_sync<KW>();
 
-        // ================= unit mode: energy network =================
-        if (m.energy != GD_ENERGY_NEO_HOOKE) {
-            for (int p = 0; p < 32; ++p) {
-                if (e0 + p / NQ >= A.n_elems) break;
-                double y[3] = {sIn[p * 4], sIn[p * 4 + 1], sIn[p * 4 + 2]}, out[10];
-                psi_net_unit(psi_of(A, spec_of(A, e0 + p / NQ)), y, out, sBuf, lane, A.tangent != 0);
-                if (lane == 0)
-#pragma unroll
-                    for (int c = 0; c < 10; ++c) sOut[p * 10 + c] = out[c];
-            }
+        // ================= net mode: energy network =================
+        // (points of different specimens take turns: a warp's networks are uniform)
+        const int p0 = warp * grp::kPts;
+        const int64_t e_p0 = e0 + p0 / NQ;
+        int s0 = 0, s1 = -1;                     // the specimens of the warp's points
+        if (e_p0 < A.n_elems) {
+            const int64_t e_l = e0 + (p0 + grp::kPts - 1) / NQ;
+            s0 = spec_of(A, e_p0);
+            s1 = spec_of(A, e_l < e_last ? e_l : e_last);
         }
-        __syncwarp();
+        if (m.energy != GD_ENERGY_NEO_HOOKE) {
+            const int64_t e_p = e0 + (p0 + (lane >> 2)) / NQ;
+            const int sp = e_p <= e_last ? spec_of(A, e_p) : -1;
+            for (int sn = s0; sn <= s1; ++sn)
+                grp::energy(psi_of(A, sn), sIn + p0 * 4, sOut + p0 * 10, nbuf, lane, sp == sn, A.tangent != 0);
+        }
+        cta_sync<KW>();
 
         // ================= qp mode: energy derivatives wrt (I1-3, I2-3, J-1) =================
-        double ps[3], ph[6], pe;
-        {
+        double ps[3], ph[6];
+        if (qp) {
             const double J = Jdet, x3 = x[2];
+            double pe;
             if (m.energy == GD_ENERGY_NEO_HOOKE) {
                 double L = log1p(x3);
                 pe = 0.5 * m.mu_e * x[0] - m.mu_e * L + 0.5 * m.lambda_e * L * L;
@@ -234,32 +605,40 @@ __global__ void __launch_bounds__(32 * KW) asm_fp64_kernel(AsmArgs A)
                 for (int c = 0; c < 6; ++c) ph[c] = 0.0;
                 ph[5] = (m.lambda_e + m.mu_e - m.lambda_e * L) / (J * J);
             } else {
-                const double *o = sOut + lane * 10;
-                double gy[3] = {o[1], o[2], o[3]};
-                double hy[6] = {o[4], o[5], o[6], o[7], o[8], o[9]};
-                // chain through the input map: dN/dx = T^T dN/dy, d2N/dx2 = T^T H T + sum_m dN/dy_m d2y_m/dx2
+                const double *o = sOut + pt * 10;
+                const NetConst nc = A.netc[valid ? spec_of(A, e_me) : 0];
 #pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    double s = 0.0;
+                for (int i = 0; i < 3; ++i) ps[i] = o[1 + i];
 #pragma unroll
-                    for (int mm = 0; mm < 3; ++mm) s += Tm[mm][i] * gy[mm];
-                    ps[i] = s;
-                }
+                for (int c = 0; c < 6; ++c) ph[c] = o[4 + c];
+                if (m.energy == GD_ENERGY_ICNN_ISO) {
+                    // chain through the input map: dN/dx = T^T dN/dy, d2N/dx2 = T^T H T + sum_m dN/dy_m d2y_m/dx2
+                    const double gy[3] = {ps[0], ps[1], ps[2]};
+                    const double hy[6] = {ph[0], ph[1], ph[2], ph[3], ph[4], ph[5]};
 #pragma unroll
-                for (int i = 0; i < 3; ++i)
-#pragma unroll
-                    for (int j = i; j < 3; ++j) {
+                    for (int i = 0; i < 3; ++i) {
                         double s = 0.0;
 #pragma unroll
-                        for (int a = 0; a < 3; ++a)
-#pragma unroll
-                            for (int b = 0; b < 3; ++b) s += Tm[a][i] * hy[sym6(a, b)] * Tm[b][j];
-#pragma unroll
-                        for (int mm = 0; mm < 3; ++mm) s += gy[mm] * T2[mm][sym6(i, j)];
-                        ph[sym6(i, j)] = s;
+                        for (int mm = 0; mm < 3; ++mm) s += Tm[mm][i] * gy[mm];
+                        ps[i] = s;
                     }
+#pragma unroll
+                    for (int i = 0; i < 3; ++i)
+#pragma unroll
+                        for (int j = i; j < 3; ++j) {
+                            double s = 0.0;
+#pragma unroll
+                            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                                for (int b = 0; b < 3; ++b) s += Tm[a][i] * hy[sym6(a, b)] * Tm[b][j];
+#pragma unroll
+                            for (int mm = 0; mm < 3; ++mm) s += gy[mm] * T2[mm][sym6(i, j)];
+                            ph[sym6(i, j)] = s;
+                        }
+                }
                 // psi_e = mu_e (N - N0 - n x3) + lambda_e t^2, t = (J-1)^2 / J
-                double t = x3 * x3 / J, dt = 1.0 - 1.0 / (J * J), d2t = 2.0 / (J * J * J);
+                const double ij = 1.0 / J;
+                double t = x3 * x3 * ij, dt = 1.0 - ij * ij, d2t = 2.0 * ij * ij * ij;
                 pe = m.mu_e * (o[0] - nc.psi_N0 - nc.psi_n * x3) + m.lambda_e * t * t;
 #pragma unroll
                 for (int i = 0; i < 3; ++i) ps[i] *= m.mu_e;
@@ -268,398 +647,291 @@ __global__ void __launch_bounds__(32 * KW) asm_fp64_kernel(AsmArgs A)
                 ps[2] += -m.mu_e * nc.psi_n + m.lambda_e * 2.0 * t * dt;
                 ph[5] += m.lambda_e * 2.0 * (dt * dt + t * d2t);
             }
-            sIn[lane * 4 + 0] = pe;
-            sIn[lane * 4 + 1] = phi;
-            sIn[lane * 4 + 2] = valid ? __ldg(A.kappa_n + e_me * NQ + q) : 0.0;
+            sIn[pt * 4 + 0] = pe;
+            sIn[pt * 4 + 1] = phi;
+            sIn[pt * 4 + 2] = valid ? __ldg(A.kappa_n + e_me * NQ + q) : 0.0;
         }
-        __syncwarp();
+        cta_sync<KW>();
 
-        // ================= unit mode: local damage update per point =================
-        const e32::MatF mf = e32::to_f(A.mat);
-        float *fbuf = reinterpret_cast<float *>(sBuf);   // FP32 network buffers (2 w floats)
+        // ================= net mode: local damage update =================
         if (A.kappa_fixed) {
             // frozen history (staggered scheme): the point keeps the given kappa
-            double *o = sOut + lane * 10;
-            o[0] = valid ? __ldg(A.kappa_fixed + e_me * NQ + q) : 0.0;
-            o[1] = 0.0;
-            o[2] = 0.0;
-            o[3] = -1.0;
-            o[4] = 0.0;
-        } else
-        for (int p = 0; p < 32; ++p) {
-            if (e0 + p / NQ >= A.n_elems) break;
-            const double ppe = sIn[p * 4], pphi = sIn[p * 4 + 1], kn = sIn[p * 4 + 2];
-            const int sp = spec_of(A, e0 + p / NQ);
-            const DevNet &yn = yld_of(A, sp);
-            const NetConst ncp = A.netc[sp];
-            double r = 0.0, dr = -1.0, Gp = 0.0;
+            if (qp) {
+                double *o = sOut + pt * 10;
+                o[0] = valid ? __ldg(A.kappa_fixed + e_me * NQ + q) : 0.0;
+                o[1] = 0.0;
+                o[2] = 0.0;
+                o[3] = -1.0;
+                o[4] = 0.0;
+            }
+        } else {
+            const e32::MatF mf = e32::to_f(A.mat);
             int n_eval = 0;
-            double kappa = kn, fail = 0.0, loading = 0.0;
-            // Trial Phi_d(kappa_n) (Eq. (dd_7_no_nn)): the FP32 network decides points
-            // clearly off the yield surface, an FP64 evaluation the others.
-            const e32::NcF nf = e32::ncf(ncp);
-            float r32, dr32, Gp32;
-            e32::r_slope(yn, mf, nf, (float)ppe, (float)pphi, (float)kn, r32, dr32, Gp32, fbuf, lane);
-            const double scale_n = fabs(kn) > 1.0 ? fabs(kn) : 1.0;
-            bool load;
-            if (fabs((double)r32) > kTrialMargin * scale_n) {
-                load = r32 > 0.0f;
-            } else {
-                r_slope(A.mat, yn, ncp, ppe, pphi, kn, r, dr, Gp, sBuf, lane);
-                ++n_eval;
-                load = r > 0.0;
-                r32 = (float)r;
-                dr32 = (float)dr;
-                Gp32 = (float)Gp;
-            }
-            if (load) {
-                loading = 1.0;
-                // The root in FP32 (the lazily bracketed Newton iteration of the mixed
-                // kernel, from the warm start), then FP64: one value-only evaluation and
-                // a Newton step with the FP32 slope (its relative error, ~1e-7, times a
-                // correction of ~1e-6 leaves ~1e-13), then one full evaluation and a last
-                // Newton step; the slope and G' of that evaluation feed the tangent (they
-                // change by ~1e-12 relative over the last step).  Where the FP32 root is not
-                // close enough, the FP64 bracketed iteration takes over from it.  Both
-                // iterations also stop on the next Newton correction |r / r'| (the step test
-                // of the safeguarded Newton-bisection; FP32: 2e-6 relative, FP64: 4 ulp) once
-                // the root is bracketed within 1e-2 relative or the iteration converges from
-                // one side: near full damage r' grows like 1 / f_d, and r itself cannot get
-                // below its rounding.  (A wide bracket does not qualify: far past the root,
-                // where f_d underflows, r' is huge and the correction meaningless.)
-                const float kg = A.kappa_guess ? (float)__ldg(A.kappa_guess + e0 * NQ + p) : (float)kn;
-                float k32 = (float)kn;
-                int n32 = 0;
-                const bool ok32 = e32::bracketed_newton(yn, mf, nf, (float)ppe, (float)pphi, (float)kn, kg, k32, r32,
-                                                        dr32, Gp32, n32, fbuf, lane, true);
-                bool done = false;
-                if (ok32 && isfinite(k32) && (double)k32 >= kn && dr32 < 0.0f) {
-                    const double sc = fabs((double)k32) > 1.0 ? fabs((double)k32) : 1.0;
-                    const double r0 = r_value(A.mat, yn, ncp, ppe, pphi, (double)k32, sBuf, lane);
-                    ++n_eval;
-                    if (fabs(r0) <= 1e-4 * sc) {
-                        const double k1 = (double)k32 - r0 / (double)dr32;
-                        r_slope(A.mat, yn, ncp, ppe, pphi, k1, r, dr, Gp, sBuf, lane);
-                        ++n_eval;
-                        if (k1 >= kn && fabs(r) <= 1e-9 * sc && dr < 0.0) {
-                            const double k2 = fabs(r) <= 1e-13 * sc ? k1 : k1 - r / dr;
-                            kappa = k2 >= kn ? k2 : kn;
-                            done = true;
-                        }
-                    }
-                }
-                if (!done) {
-                    // FP64 lazily bracketed Newton iteration from the FP32 result (the
-                    // iteration of the FP64 reference path)
-                    r_slope(A.mat, yn, ncp, ppe, pphi, kn, r, dr, Gp, sBuf, lane);
-                    ++n_eval;
-                    const double kgd = isfinite(k32) ? (double)k32 : kn;
-                    if (kgd > kn) {
-                        kappa = kgd;
-                        r_slope(A.mat, yn, ncp, ppe, pphi, kappa, r, dr, Gp, sBuf, lane);
-                        ++n_eval;
-                    }
-                    double lo = kn, hi = kn;
-                    bool have_hi = false;
-                    if (r > 0.0) lo = kappa;
-                    else {
-                        hi = kappa;
-                        have_hi = true;
-                    }
-                    double dx_prev = have_hi ? hi - lo : 1.0e30, dx = dx_prev;
-                    bool took_newton = false;
-                    int it;
-                    for (it = 0; it < m.local_max; ++it) {
-                        const double scale = fabs(kappa) > 1.0 ? fabs(kappa) : 1.0;
-                        const double ulp4 = 4.0 * 2.220446049250313e-16 * scale;
-                        if (fabs(r) <= 1e-13 * scale || (have_hi && (hi - lo) <= ulp4)) break;
-                        if (fabs(r) <= ulp4 * fabs(dr) &&
-                            (have_hi ? (hi - lo) <= 1e-2 * scale : (took_newton && fabs(2.0 * r) <= fabs(dx * dr))))
-                            break;
-                        const double newton = kappa - r / dr;
-                        bool take;
-                        if (have_hi) {
-                            take = (newton > lo) && (newton < hi) && (fabs(2.0 * r) <= fabs(dx_prev * dr));
-                        } else {
-                            // forward Newton step, at most a few times the distance covered so far
-                            const double cap = 4.0 * ((double)(r > 1e-12 ? r : 1e-12) + (kappa - kn));
-                            take = dr < 0.0 && newton > lo && (newton - kappa) <= cap;
-                        }
-                        dx_prev = dx;
-                        took_newton = take;
-                        if (take) {
-                            dx = kappa - newton;
-                            kappa = newton;
-                        } else if (have_hi) {
-                            dx = 0.5 * (hi - lo);
-                            kappa = lo + dx;
-                        } else {
-                            const double step =
-                                2.0 * ((kappa - kn) > (r > 1e-12 ? r : 1e-12) ? (kappa - kn) : (r > 1e-12 ? r : 1e-12));
-                            dx = step;
-                            kappa = lo + step;
-                        }
-                        r_slope(A.mat, yn, ncp, ppe, pphi, kappa, r, dr, Gp, sBuf, lane);
-                        ++n_eval;
-                        if (r > 0.0) {
-                            lo = kappa;
-                        } else {
-                            hi = kappa;
-                            have_hi = true;
-                        }
-                    }
-                    if (it >= m.local_max) fail = 1.0;
-                }
-            }
-            if (lane == 0) {
-                double *o = sOut + p * 10;
-                if (e0 + p / NQ < A.n_elems) atomicAdd(A.counters + 2, n_eval);
-                o[0] = kappa;
-                o[1] = loading;
-                o[2] = Gp;
-                o[3] = dr;
-                o[4] = fail;
-            }
+            for (int sn = s0; sn <= s1; ++sn)
+                n_eval += local_update<DIM>(A, mf, e0, p0, sn, sIn, sOut, nbuf, lane);
+            n_eval = __reduce_add_sync(0xffffffffu, n_eval);
+            if (lane == 0 && n_eval) atomicAdd(A.counters + 2, n_eval);
         }
-        __syncwarp();
+        cta_sync<KW>();
 
-        // ================= qp mode: stress and records =================
-        {
-            const double *o = sOut + lane * 10;
+        // ================= qp mode: stress and the point's tangent =================
+        bool loading = false;
+        if (qp) {
+            const double *o = sOut + pt * 10;
             const double kappa = o[0];
-            const bool loading = o[1] > 0.5;
+            loading = valid && o[1] > 0.5;
             if (valid) {
                 if (A.kappa_new) A.kappa_new[e_me * NQ + q] = kappa;
                 if (A.loading) A.loading[e_me * NQ + q] = loading ? 1 : 0;
                 if (o[4] > 0.5) atomicAdd(A.counters, 1);
-                if (loading) atomicAdd(A.counters + 1, 1);
             }
+            double *rec = sRec + pt * R_::SIZE;
+            const double Jw = valid ? det : 0.0;
             const bool dmg = kappa > m.kappa_d;
             const double fd = dmg ? exp(-m.eta_d * (kappa - m.kappa_d)) : 1.0;
             const double fdp = dmg ? -m.eta_d * fd : 0.0;
             const double ck = loading ? -o[2] / o[3] : 0.0;          // G' / (1 - G' dq/dkappa)
             const double dkdphi = ck * m.qcoef / fd;                  // dq/dphi = qcoef / f_d
-            const double J = Jdet;
-            // F^-1 = cof(F)^T / J
-            double Fi[3][3];
+            const double J = Jdet, I1 = 3.0 + x[0], ij = 1.0 / J;
+            // F^-1 = cof(F)^T / J; pulled back to the reference element: F' = F Ji^T (F_iJ Ji_jJ),
+            // Fi'_ji = Ji_jJ F^-1_Ji
+            double Fp[DIM][DIM], Fi[DIM][DIM], G2[DIM][DIM], h[DIM], mv[DIM];
+            {
+                double Fv[DIM][DIM];
+                if constexpr (DIM == 2) {
+                    Fv[0][0] = F[1][1] * ij; Fv[0][1] = -F[0][1] * ij;
+                    Fv[1][0] = -F[1][0] * ij; Fv[1][1] = F[0][0] * ij;
+                } else {
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
+                    for (int i = 0; i < DIM; ++i)
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    int i1 = (j + 1) % 3, i2 = (j + 2) % 3, j1 = (i + 1) % 3, j2 = (i + 2) % 3;
-                    Fi[i][j] = (F[i1][j1] * F[i2][j2] - F[i1][j2] * F[i2][j1]) / J;
+                        for (int j = 0; j < DIM; ++j) {
+                            const int i1 = (j + 1) % DIM, i2 = (j + 2) % DIM, j1 = (i + 1) % DIM, j2 = (i + 2) % DIM;
+                            Fv[i][j] = (F[i1][j1] * F[i2][j2] - F[i1][j2] * F[i2][j1]) * ij;
+                        }
                 }
-            double C[3][3], b[3][3];
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
+                for (int i = 0; i < DIM; ++i)
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    double s = 0.0, t = 0.0;
+                    for (int j = 0; j < DIM; ++j) {
+                        double s = 0.0, t = 0.0;
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        s += F[k][i] * F[k][j];
-                        t += F[i][k] * F[j][k];
+                        for (int K = 0; K < DIM; ++K) {
+                            s += F[i][K] * Ji[j][K];
+                            t += Ji[j][K] * Fv[K][i];
+                        }
+                        Fp[i][j] = s;
+                        Fi[j][i] = t;
                     }
-                    C[i][j] = s;
-                    b[i][j] = t;
-                }
-            const double I1 = 3.0 + x[0];
-            // h = F^-T g, mvec = F^-1 h = C^-1 g
-            double hv[3], mv[3];
-#pragma unroll
-            for (int i = 0; i < 3; ++i) hv[i] = Fi[0][i] * g[0] + Fi[1][i] * g[1] + Fi[2][i] * g[2];
-#pragma unroll
-            for (int i = 0; i < 3; ++i) mv[i] = Fi[i][0] * hv[0] + Fi[i][1] * hv[1] + Fi[i][2] * hv[2];
-            // P = f_d [2 psi_1 F + 2 psi_2 (I1 F - F C) + psi_3 J F^-T] - c_d h (x) m
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int J2 = 0; J2 < 3; ++J2) {
-                    double FC = F[i][0] * C[0][J2] + F[i][1] * C[1][J2] + F[i][2] * C[2][J2];
-                    double Ph = 2.0 * ps[0] * F[i][J2] + 2.0 * ps[1] * (I1 * F[i][J2] - FC) + ps[2] * J * Fi[J2][i];
-                    rec[Q_P + i * 3 + J2] = fd * Ph - m.c_d * hv[i] * mv[J2];
-                    rec[Q_F + i * 3 + J2] = F[i][J2];
-                    rec[Q_B + i * 3 + J2] = b[i][J2];
-                    rec[Q_FINV + i * 3 + J2] = Fi[i][J2];
-                }
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                rec[Q_M + i] = mv[i];
-                rec[Q_H + i] = hv[i];
             }
-            rec[Q_I1] = I1;
+            // h = F^-T grad phi (= Fi'^T of the reference gradient), C^-1 grad phi pulled back
 #pragma unroll
-            for (int c = 0; c < 6; ++c) rec[Q_HS + c] = fd * ph[c];
-            rec[Q_G1] = fd * ps[0];
-            rec[Q_G2] = fd * ps[1];
-            rec[Q_G3J] = fd * ps[2] * J;
-            rec[Q_PS1] = ps[0];
-            rec[Q_PS2] = ps[1];
-            rec[Q_PS3J] = ps[2] * J;
-            rec[Q_CK] = fdp * ck;
-            rec[Q_BCK] = m.beta_d * ck;
-            rec[Q_FDK] = fdp * dkdphi;
-            rec[Q_PP] = m.beta_d * (1.0 - dkdphi);
-            rec[Q_PEN] = m.beta_d * (phi - kappa);
-            rec[Q_J] = J;
-            if (!valid) rec[Q_JW] = 0.0;
+            for (int i = 0; i < DIM; ++i) {
+                double s = 0.0;
+#pragma unroll
+                for (int k = 0; k < DIM; ++k) s += Fi[k][i] * gx[k];
+                h[i] = s;
+            }
+#pragma unroll
+            for (int j = 0; j < DIM; ++j) {
+                double s = 0.0;
+#pragma unroll
+                for (int i = 0; i < DIM; ++i) s += Fi[j][i] * h[i];
+                mv[j] = s;
+            }
+            double b[DIM][DIM];
+#pragma unroll
+            for (int i = 0; i < DIM; ++i)
+#pragma unroll
+                for (int k = i; k < DIM; ++k) {
+                    double s = 0.0;
+#pragma unroll
+                    for (int K = 0; K < DIM; ++K) s += F[i][K] * F[k][K];
+                    b[i][k] = b[k][i] = s;
+                }
+            // G^2 = dI2/dF pulled back; P = f_d dpsi_e/dF - c_d h (x) m
+            const double ps3J = ps[2] * J, cdw = m.c_d * Jw, fdw = fd * Jw;
+#pragma unroll
+            for (int i = 0; i < DIM; ++i)
+#pragma unroll
+                for (int j = 0; j < DIM; ++j) {
+                    double s = I1 * Fp[i][j];
+#pragma unroll
+                    for (int k = 0; k < DIM; ++k) s -= b[i][k] * Fp[k][j];
+                    G2[i][j] = 2.0 * s;
+                    const double Pe = 2.0 * ps[0] * Fp[i][j] + ps[1] * G2[i][j] + ps3J * Fi[j][i];
+                    rec[R_::PE + i * DIM + j] = Pe;
+                    rec[R_::P + i * DIM + j] = fdw * Pe - cdw * h[i] * mv[j];
+                }
+#pragma unroll
+            for (int j = 0; j < DIM; ++j) rec[R_::Y + j] = cdw * mv[j];
+            rec[R_::PEN] = m.beta_d * (phi - kappa) * Jw;
+            if (A.tangent) {
+                rec[R_::FDK] = fdp * dkdphi * Jw;
+                rec[R_::BCK] = m.beta_d * ck * Jw;
+                rec[R_::PP] = m.beta_d * (1.0 - dkdphi) * Jw;
+                double hw[DIM];                                    // c_d J w h
+#pragma unroll
+                for (int i = 0; i < DIM; ++i) hw[i] = cdw * h[i];
+                double Cv[DIM][DIM], Sj[DIM][DIM], Mj[DIM][DIM];
+                const double g2w = 2.0 * fdw * ps[1], g1w = 2.0 * fdw * ps[0] + g2w * I1;
+#pragma unroll
+                for (int j = 0; j < DIM; ++j)
+#pragma unroll
+                    for (int l = j; l < DIM; ++l) {
+                        double ci = 0.0, mm = 0.0, c = 0.0;
+#pragma unroll
+                        for (int i = 0; i < DIM; ++i) {
+                            ci += Fi[j][i] * Fi[l][i];             // C^-1
+                            mm += Ji[j][i] * Ji[l][i];             // the metric (delta_JL)
+                            c += Fp[i][j] * Fp[i][l];              // C
+                        }
+                        Cv[j][l] = Cv[l][j] = cdw * ci;
+                        rec[R_::CV + sym_pos<DIM>(j, l)] = cdw * ci;
+                        Mj[j][l] = Mj[l][j] = g2w * mm;
+                        Sj[j][l] = Sj[l][j] = g1w * mm - g2w * c;
+                    }
+                // d2 psi_e/dF2 with the kappa coupling, times f_d and J w:
+                //   sum_mn (f_d psi_mn + f_d' c_kappa psi_m psi_n) G^m G^n + f_d (psi_1 D2(I1) + psi_2 D2(I2) + psi_3 D2(J)),
+                //   G^1 = 2 F, G^2 = 2 (I1 F - F F^T F), G^3 = J F^-T,
+                //   D2(I1) = 2 d_ik d_JL,  D2(J) = J (F^-1_Ji F^-1_Lk - F^-1_Jk F^-1_Li),
+                //   D2(I2) = 2 [2 F_iJ F_kL - F_iL F_kJ + (I1 d_JL - C_JL) d_ik - d_JL b_ik];
+                // their products of first derivatives join the G^m G^n sum
+                const double ckw = fdp * ck * Jw, g3w = fdw * ps3J;
+                const double h11 = 4.0 * (fdw * ph[0] + ckw * ps[0] * ps[0]) + 2.0 * g2w;
+                const double h12 = 2.0 * (fdw * ph[1] + ckw * ps[0] * ps[1]);
+                const double h13 = 2.0 * (fdw * ph[2] + ckw * ps[0] * ps[2]) * J;
+                const double h22 = fdw * ph[3] + ckw * ps[1] * ps[1];
+                const double h23 = (fdw * ph[4] + ckw * ps[1] * ps[2]) * J;
+                const double h33 = (fdw * ph[5] + ckw * ps[2] * ps[2]) * J * J + g3w;
+                double V[DIM][DIM];                                // c_d J w h_k m_j - f_d psi_3 J J w F^-1_jk
+#pragma unroll
+                for (int k = 0; k < DIM; ++k)
+#pragma unroll
+                    for (int j = 0; j < DIM; ++j) V[k][j] = hw[k] * mv[j] - g3w * Fi[j][k];
+#pragma unroll
+                for (int i = 0; i < DIM; ++i)
+#pragma unroll
+                    for (int j = 0; j < DIM; ++j) {
+                        const int r = DIM * i + j;
+                        const double t1 = h11 * Fp[i][j] + h12 * G2[i][j] + h13 * Fi[j][i];
+                        const double t2 = h12 * Fp[i][j] + h22 * G2[i][j] + h23 * Fi[j][i];
+                        const double t3 = h13 * Fp[i][j] + h23 * G2[i][j] + h33 * Fi[j][i];
+#pragma unroll
+                        for (int c = r; c < N2; ++c) {
+                            const int k = c / DIM, l = c % DIM;
+                            double v = t1 * Fp[k][l] + t2 * G2[k][l] + t3 * Fi[l][k];
+                            if (i == k) v += Sj[j][l];
+                            v -= Mj[j][l] * b[i][k];
+                            v -= g2w * Fp[i][l] * Fp[k][j];
+                            v += Fi[l][i] * V[k][j];
+                            v += hw[i] * mv[l] * Fi[j][k];
+                            v += Cv[j][l] * (h[i] * h[k]);
+                            rec[R_::A + sym_pos<N2>(r, c)] = v;
+                        }
+#pragma unroll
+                        for (int l = 0; l < DIM; ++l)
+                            rec[R_::B + r * DIM + l] = -(cdw * mv[j] * Fi[l][i] + h[i] * Cv[j][l]);
+                    }
+            }
         }
-        __syncwarp();
+        {
+            const unsigned n_load = __ballot_sync(0xffffffffu, loading);
+            if (lane == 0 && n_load) atomicAdd(A.counters + 1, __popc(n_load));
+        }
+        cta_sync<KW>();
 
         // ================= row mode: element residual and tangent =================
-        for (int pass = 0; pass < EPW / EPR; ++pass) {
-            // per (point, node) vectors of the EPR elements of this pass
-            for (int t = lane; t < EPR * NQ * NEN; t += 32) {
-                const int ee = t / (NQ * NEN), qq = (t / NEN) % NQ, a = t % NEN;
-                const double *R0 = sRec + ((pass * EPR + ee) * NQ + qq) * Q_REC;
-                double *V = sVec + t * V_REC;
-                const double xi[3] = {(qq & 1) ? kGauss : -kGauss, (qq & 2) ? kGauss : -kGauss,
-                                      (qq & 4) ? kGauss : -kGauss};
-                double Na, dN[3], n[3] = {0.0, 0.0, 0.0};
-                ref_shape<DIM>(a, xi, Na, dN);
+        {
+            constexpr int EPWR = grp::kPts / NQ;                 // elements of a warp: HEX8 1, Q4 2
+            const int ee = lane / G_::ND, row = lane % G_::ND, a = row / NDOF, i = row % NDOF;
+            const int el_r = warp * EPWR + ee;
+            const int64_t e = e0 + el_r;
+            if (lane < EPWR * G_::ND && e < A.n_elems) {
+                const double *R0 = sRec + el_r * NQ * R_::SIZE;
+                const bool pr = i == DIM;                        // a phi row
+                double Rr = 0.0;
 #pragma unroll
-                for (int J = 0; J < DIM; ++J)
-#pragma unroll
-                    for (int k = 0; k < DIM; ++k) n[J] += dN[k] * R0[Q_JINV + k * 3 + J];
-                double f[3], bf[3], nt[3], G2[3];
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    f[i] = R0[Q_F + i * 3] * n[0] + R0[Q_F + i * 3 + 1] * n[1] + R0[Q_F + i * 3 + 2] * n[2];
-                    nt[i] = R0[Q_FINV + i] * n[0] + R0[Q_FINV + 3 + i] * n[1] + R0[Q_FINV + 6 + i] * n[2];
-                }
-#pragma unroll
-                for (int i = 0; i < 3; ++i)
-                    bf[i] = R0[Q_B + i * 3] * f[0] + R0[Q_B + i * 3 + 1] * f[1] + R0[Q_B + i * 3 + 2] * f[2];
-#pragma unroll
-                for (int i = 0; i < 3; ++i) G2[i] = 2.0 * (R0[Q_I1] * f[i] - bf[i]);
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    V[V_N + i] = n[i];
-                    V[V_F + i] = f[i];
-                    V[V_G2 + i] = G2[i];
-                    V[V_NT + i] = nt[i];
-                    V[V_PN + i] = 2.0 * R0[Q_PS1] * f[i] + R0[Q_PS2] * G2[i] + R0[Q_PS3J] * nt[i];
-                }
-                V[V_NN] = Na;
-                V[V_MN] = R0[Q_M] * n[0] + R0[Q_M + 1] * n[1] + R0[Q_M + 2] * n[2];
-            }
-            __syncwarp();
-            const int ee = lane / ND, row = lane % ND;
-            const int a = row / NDOF, i = row % NDOF;
-            const int el_local = pass * EPR + ee;
-            const int64_t e = e0 + el_local;
-            const bool active = (lane < EPR * ND) && (e < A.n_elems);
-            double Kr[ND];
-#pragma unroll
-            for (int c = 0; c < ND; ++c) Kr[c] = 0.0;
-            double Rr = 0.0;
-            const double cd = m.c_d;
-            if (active) {
                 for (int qq = 0; qq < NQ; ++qq) {
-                    const double *R0 = sRec + (el_local * NQ + qq) * Q_REC;
-                    const double *Vq = sVec + (ee * NQ + qq) * NEN * V_REC;
-                    const double *Va = Vq + a * V_REC;
-                    const double Jw = R0[Q_JW];
-                    if (i < DIM) {
-                        // r_u,a = P n_a J w (Sec. 3.1)
-                        Rr += Jw * (R0[Q_P + i * 3] * Va[V_N] + R0[Q_P + i * 3 + 1] * Va[V_N + 1] +
-                                    R0[Q_P + i * 3 + 2] * Va[V_N + 2]);
-                        if (!A.tangent) continue;      // residual-only pass: no tangent rows
-                        // d2 psi_e/dF2 contracted with grad N_a, grad N_b:
-                        //   sum_mn psi_mn G^m_a G^n_b + psi_1 D2(I1) + psi_2 D2(I2) + psi_3 D2(J),
-                        // G^1 = 2 F n, G^2 = 2 (I1 F n - F F^T F n), G^3 = J F^-T n,
-                        // D2(I1)_ik = 2 (n_a.n_b) d_ik,
-                        // D2(I2)_ik = 2 [2 f_a,i f_b,k - f_b,i f_a,k + (I1 n_a.n_b - f_a.f_b) d_ik - (n_a.n_b) b_ik],
-                        // D2(J)_ik  = J (nt_a,i nt_b,k - nt_a,k nt_b,i),   f = F n, nt = F^-T n.
-                        const double Jd = R0[Q_J];
-                        const double Gai[3] = {2.0 * Va[V_F + i], Va[V_G2 + i], Jd * Va[V_NT + i]};
-                        const double *HS = R0 + Q_HS;
-                        double tn[3];
+                    const double *rq = R0 + qq * R_::SIZE, *c = sRef + (qq * NEN + a) * 4;
+                    const double *pj = rq + (pr ? R_::Y : R_::P + i * DIM);
 #pragma unroll
-                        for (int nI = 0; nI < 3; ++nI)
-                            tn[nI] = HS[sym6(0, nI)] * Gai[0] + HS[sym6(1, nI)] * Gai[1] + HS[sym6(2, nI)] * Gai[2];
-                        const double g1 = R0[Q_G1], g2 = R0[Q_G2], g3J = R0[Q_G3J], I1 = R0[Q_I1];
-                        const double ck = R0[Q_CK], fdk = R0[Q_FDK];
-                        const double hi_ = R0[Q_H + i], mna = Va[V_MN], Pna = Va[V_PN + i];
-                        const double fai = Va[V_F + i], ntai = Va[V_NT + i];
-#pragma unroll
-                        for (int bN = 0; bN < NEN; ++bN) {
-                            const double *Vb = Vq + bN * V_REC;
-                            const double nn = Va[V_N] * Vb[V_N] + Va[V_N + 1] * Vb[V_N + 1] + Va[V_N + 2] * Vb[V_N + 2];
-                            const double ff = Va[V_F] * Vb[V_F] + Va[V_F + 1] * Vb[V_F + 1] + Va[V_F + 2] * Vb[V_F + 2];
-                            const double tt =
-                                Va[V_NT] * Vb[V_NT] + Va[V_NT + 1] * Vb[V_NT + 1] + Va[V_NT + 2] * Vb[V_NT + 2];
-                            const double mnb = Vb[V_MN], ntbi = Vb[V_NT + i], fbi = Vb[V_F + i];
-#pragma unroll
-                            for (int k = 0; k < DIM; ++k) {
-                                const double fbk = Vb[V_F + k], ntbk = Vb[V_NT + k];
-                                double v = tn[0] * 2.0 * fbk + tn[1] * Vb[V_G2 + k] + tn[2] * Jd * ntbk;
-                                if (k == i) v += 2.0 * g1 * nn + 2.0 * g2 * (I1 * nn - ff);
-                                v += 2.0 * g2 * (2.0 * fai * fbk - fbi * Va[V_F + k] - nn * R0[Q_B + i * 3 + k]);
-                                v += g3J * (ntai * ntbk - Va[V_NT + k] * ntbi);
-                                v += ck * Pna * Vb[V_PN + k];
-                                v += cd * (mna * ntbi * R0[Q_H + k] + tt * hi_ * R0[Q_H + k] + mnb * hi_ * Va[V_NT + k]);
-                                Kr[bN * NDOF + k] += Jw * v;
-                            }
-                            Kr[bN * NDOF + DIM] += Jw * (-cd * (mna * ntbi + hi_ * tt) + fdk * Pna * Vb[V_NN]);
-                        }
-                    } else {
-                        // R_phi,a = (Y . grad N_a - Y N_a) J w, Y vec = c_d C^-1 grad phi, -Y = beta_d (phi - kappa)
-                        const double Na = Va[V_NN];
-                        Rr += Jw * (cd * Va[V_MN] + R0[Q_PEN] * Na);
-                        if (!A.tangent) continue;
-                        const double bck = R0[Q_BCK], pp = R0[Q_PP];
-#pragma unroll
-                        for (int bN = 0; bN < NEN; ++bN) {
-                            const double *Vb = Vq + bN * V_REC;
-                            const double tt =
-                                Va[V_NT] * Vb[V_NT] + Va[V_NT + 1] * Vb[V_NT + 1] + Va[V_NT + 2] * Vb[V_NT + 2];
-                            const double mnb = Vb[V_MN];
-#pragma unroll
-                            for (int k = 0; k < DIM; ++k)
-                                Kr[bN * NDOF + k] += Jw * (-cd * (R0[Q_H + k] * tt + mnb * Va[V_NT + k]) -
-                                                           bck * Na * Vb[V_PN + k]);
-                            Kr[bN * NDOF + DIM] += Jw * (cd * tt + pp * Na * Vb[V_NN]);
-                        }
-                    }
+                    for (int j = 0; j < DIM; ++j) Rr += c[j] * pj[j];
+                    if (pr) Rr += c[3] * rq[R_::PEN];
                 }
-                // scatter through the slot map
                 const int32_t na = __ldg(A.conn + e * NEN + a);
-                const int64_t rdof = (int64_t)na * NDOF + i;
-                if (A.R) atomicAdd(A.R + rdof, Rr);
+                if (A.R) atomicAdd(A.R + (int64_t)na * NDOF + i, Rr);
                 if (A.tangent) {
                     const int32_t rb = __ldg(A.rowptr + (int64_t)na * NDOF);
-                    const int32_t rowlen = __ldg(A.rowptr + (int64_t)na * NDOF + 1) - rb;
+                    const int64_t off = (int64_t)i * (__ldg(A.rowptr + (int64_t)na * NDOF + 1) - rb);
                     const int32_t *sl = A.slot + (e * NEN + a) * NEN;
+                    double T[DIM][NQ], K[NEN];
+                    auto add = [&](int k) {
 #pragma unroll
-                    for (int bN = 0; bN < NEN; ++bN) {
-                        const int64_t pos = (int64_t)__ldg(sl + bN) + (int64_t)i * rowlen;
-#pragma unroll
-                        for (int k = 0; k < NDOF; ++k) {
-                            if (A.vals) atomicAdd(A.vals + pos + k, Kr[bN * NDOF + k]);
-                            else atomicAdd(A.vals32 + pos + k, (float)Kr[bN * NDOF + k]);
+                        for (int l = 0; l < NEN; ++l) {
+                            const int64_t pos = (int64_t)__ldg(sl + node_of_bits(l)) + off + k;
+                            if (A.vals) atomicAdd(A.vals + pos, K[l]);
+                            else atomicAdd(A.vals32 + pos, (float)K[l]);
                         }
+                    };
+#pragma unroll 1
+                    for (int k = 0; k < DIM; ++k) {
+                        // columns (b, u_k)
+                        int at[DIM][DIM];
+#pragma unroll
+                        for (int j = 0; j < DIM; ++j)
+#pragma unroll
+                            for (int l = 0; l < DIM; ++l)
+                                at[j][l] = pr ? R_::B + (DIM * k + l) * DIM + j
+                                              : R_::A + sym_pos<N2>(DIM * i + j, DIM * k + l);
+#pragma unroll
+                        for (int qq = 0; qq < NQ; ++qq) {
+                            const double *rq = R0 + qq * R_::SIZE, *c = sRef + (qq * NEN + a) * 4;
+#pragma unroll
+                            for (int l = 0; l < DIM; ++l) {
+                                double t = 0.0;
+#pragma unroll
+                                for (int j = 0; j < DIM; ++j) t += c[j] * rq[at[j][l]];
+                                T[l][qq] = t;
+                            }
+                            if (pr) {
+                                const double nb = c[3] * rq[R_::BCK];
+#pragma unroll
+                                for (int l = 0; l < DIM; ++l) T[l][qq] -= nb * rq[R_::PE + DIM * k + l];
+                            }
+                        }
+                        expand_rows<false>(T, nullptr, K);
+                        add(k);
                     }
+                    // columns (b, phi)
+                    double TN[NQ];
+#pragma unroll
+                    for (int qq = 0; qq < NQ; ++qq) {
+                        const double *rq = R0 + qq * R_::SIZE, *c = sRef + (qq * NEN + a) * 4;
+                        double t = 0.0;
+#pragma unroll
+                        for (int l = 0; l < DIM; ++l) {
+                            double s = 0.0;
+#pragma unroll
+                            for (int j = 0; j < DIM; ++j)
+                                s += c[j] * rq[pr ? R_::CV + sym_pos<DIM>(j, l) : R_::B + (DIM * i + j) * DIM + l];
+                            T[l][qq] = s;
+                            t += c[l] * rq[R_::PE + (pr ? 0 : i) * DIM + l];
+                        }
+                        TN[qq] = pr ? c[3] * rq[R_::PP] : rq[R_::FDK] * t;
+                    }
+                    expand_rows<true>(T, TN, K);
+                    add(DIM);
                 }
             }
-            __syncwarp();
         }
     }
-}
-
-template <int DIM>
-size_t smem_bytes(int wmax)
-{
-    using G_ = Geo<DIM>;
-    size_t scratch = G_::EPW * G_::NEN * (DIM + G_::NDOF) + 32 * Q_REC + 32 * 4 + 32 * 10 + 5 * wmax +
-                     2 * G_::NQ * G_::NEN * V_REC;
-    return scratch * sizeof(double);          // per warp
 }
 
 template <int DIM, int KW>
 cudaError_t launch_kw(const AsmArgs &a, int num_sms, const AsmTune &t, cudaStream_t s)
 {
-    size_t sm = smem_bytes<DIM>(a.wmax) * KW;
+    const size_t sm = (size_t)Smem<DIM, KW>::total(a.wmax) * sizeof(double);
     int dev = 0, optin = 0;
     cudaError_t e0 = cudaGetDevice(&dev);
     if (e0 == cudaSuccess) e0 = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -672,9 +944,7 @@ cudaError_t launch_kw(const AsmArgs &a, int num_sms, const AsmTune &t, cudaStrea
     if (err != cudaSuccess) return err;
     if (per_sm < 1) per_sm = 1;
     if (t.cta_per_sm > 0 && t.cta_per_sm < per_sm) per_sm = t.cta_per_sm;
-    using G_ = Geo<DIM>;
-    int64_t batches = (a.n_elems + G_::EPW - 1) / G_::EPW;
-    int64_t need = (batches + KW - 1) / KW;
+    const int64_t need = (a.n_elems + Smem<DIM, KW>::EL - 1) / Smem<DIM, KW>::EL;
     int64_t grid = (int64_t)num_sms * per_sm;
     if (grid > need) grid = need;
     if (t.grid_max > 0 && grid > t.grid_max) grid = t.grid_max;
@@ -697,10 +967,15 @@ cudaError_t launch_dim(const AsmArgs &a, int num_sms, const AsmTune &t, cudaStre
         default: return launch_kw<DIM, 4>(a, num_sms, t, s);
         }
     }
+    // small meshes: CTAs of eight or sixteen points until every SM has one (qp mode then
+    // leaves lanes idle, which costs less than idle SMs)
+    int warps = t.warps;
+    const int64_t points = a.n_elems * Geo<DIM>::NQ;
+    while (warps > 1 && (points + 8 * warps - 1) / (8 * warps) < num_sms) warps /= 2;
     cudaError_t e = cudaErrorInvalidConfiguration;
-    if (t.warps >= 8) e = launch_kw<DIM, 8>(a, num_sms, t, s);
-    if (e == cudaErrorInvalidConfiguration && t.warps >= 4) e = launch_kw<DIM, 4>(a, num_sms, t, s);
-    if (e == cudaErrorInvalidConfiguration && t.warps >= 2) e = launch_kw<DIM, 2>(a, num_sms, t, s);
+    if (warps >= 8) e = launch_kw<DIM, 8>(a, num_sms, t, s);
+    if (e == cudaErrorInvalidConfiguration && warps >= 4) e = launch_kw<DIM, 4>(a, num_sms, t, s);
+    if (e == cudaErrorInvalidConfiguration && warps >= 2) e = launch_kw<DIM, 2>(a, num_sms, t, s);
     if (e == cudaErrorInvalidConfiguration) e = launch_kw<DIM, 1>(a, num_sms, t, s);
     return e;
 }
@@ -775,6 +1050,53 @@ cudaError_t launch_net_to_float(const DevNet &net, cudaStream_t s)
     to_float_kernel<<<(net.n_params + 255) / 256, 256, 0, s>>>(net.p, net.pf, net.n_params);
     const int ww = net.width * net.width;
     to_float_kernel<<<(ww + 255) / 256, 256, 0, s>>>(net.W2T, net.W2Tf, ww);
+    return cudaGetLastError();
+}
+
+namespace {
+// fixed-point copies of one network (layout of fx::Net): each weight row and column set is
+// scaled by the power of two above its largest magnitude
+__global__ void net_fixed_kernel(DevNet net)
+{
+    using namespace fx;
+    const int w = net.width, wp = pad16(w), n_in = net.n_in, t0 = threadIdx.x, nt = blockDim.x;
+    const double *W1 = net.p, *W2 = W1 + w * n_in + w, *w3 = W2 + w * w + w * n_in + w;
+    const Net f = net_of(net.fx, w);
+    int *e = const_cast<int *>(f.e);
+    for (int t = t0; t < 2 * w + 2; t += nt) {
+        double m = 0.0;
+        if (t < w) for (int j = 0; j < w; ++j) m = fmax(m, fabs(W2[t * w + j]));
+        else if (t < 2 * w) for (int k = 0; k < w; ++k) m = fmax(m, fabs(W2[k * w + t - w]));
+        else if (t == 2 * w) for (int i = 0; i < w * n_in; ++i) m = fmax(m, fabs(W1[i]));
+        else for (int k = 0; k < w; ++k) m = fmax(m, fabs(w3[k]));
+        e[t] = bound_exp(m);
+    }
+    __syncthreads();
+    for (int t = t0; t < w * wp; t += nt) {
+        const int a = t / wp, b = t % wp, at = a * wp + perm16(b);
+        const bool in = b < w;
+        const_cast<int2 *>(f.W2)[at] = in ? limbs(from_double(W2[b * w + a], kBits - e[b])) : make_int2(0, 0);
+        const_cast<int2 *>(f.W2T)[at] = in ? limbs(from_double(W2[a * w + b], kBits - e[w + b])) : make_int2(0, 0);
+        const_cast<float *>(f.W2P)[at] = in ? (float)W2[b * w + a] : 0.0f;
+    }
+    for (int j = t0; j < w; j += nt) {
+        double v[3] = {0.0, 0.0, 0.0};
+        for (int c = 0; c < n_in && c < 3; ++c) v[c] = W1[j * n_in + c];
+        for (int c = 0; c < 4; ++c) const_cast<i64 *>(f.W1)[4 * j + c] = c < 3 ? from_double(v[c], 62 - e[2 * w]) : 0;
+        const_cast<i64 *>(f.w3)[j] = from_double(w3[j], 62 - e[2 * w + 1]);
+        double *ww = const_cast<double *>(f.WW) + 6 * j;
+        ww[0] = v[0] * v[0]; ww[1] = v[0] * v[1]; ww[2] = v[0] * v[2];
+        ww[3] = v[1] * v[1]; ww[4] = v[1] * v[2]; ww[5] = v[2] * v[2];
+    }
+}
+}  // namespace
+
+size_t net_fixed_bytes(int width) { return fx::net_bytes(width); }
+
+cudaError_t launch_net_fixed(const DevNet &net, cudaStream_t s)
+{
+    if (net.width <= 0) return cudaSuccess;
+    net_fixed_kernel<<<1, 256, 0, s>>>(net);
     return cudaGetLastError();
 }
 

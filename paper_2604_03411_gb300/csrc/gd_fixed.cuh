@@ -1,0 +1,292 @@
+// gd_fixed.cuh -- 64-bit fixed-point arithmetic for the ICNNs of the FP64 element kernel.
+//
+// sm_103a issues FP64 at 1.7 lanes per clock and SM but 32-bit integer multiply-adds
+// (32 x 32 + 64 -> 64) at 62 (both measured with independent chains, 4-16 warps per SM).
+// The networks' layers are sums of bounded terms, so they are evaluated in fixed point:
+//  - softplus and sigmoid of an FP64 argument come from integer polynomials on two
+//    256-entry tables, with absolute errors of a few 2^-58 (exp and log1p in FP64: 43
+//    FP64 operations per unit, here about 170 integer instructions: 3 clocks instead of 25
+//    per unit and SM);
+//  - a layer's product sum_j W_kj z_j runs on 56-bit operands split into two 28-bit limbs,
+//    three multiply-adds per term (lo x lo, below 2^-58 of the largest term, is left out)
+//    with exact 64-bit accumulation, so that its error, about 2^-56 of the largest term
+//    after up to 64 terms, is below the rounding of the FP64 sum, which starts at 2^-53 of
+//    the running sum.  Each weight row and each operand column carries a power-of-two scale.
+// Compiles for the host as well (the tables are constant expressions).
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace gd {
+namespace fx {
+
+using i64 = long long;
+using u64 = unsigned long long;
+#define GD_FX __host__ __device__ __forceinline__
+
+constexpr i64 kOne62 = 1LL << 62;
+constexpr int kBits = 56;                 // operand bits of the layer products
+constexpr int kLimb = 28;
+
+GD_FX u64 mulhi_u(u64 a, u64 b)
+{
+#ifdef __CUDA_ARCH__
+    return __umul64hi(a, b);
+#else
+    return (u64)(((unsigned __int128)a * b) >> 64);
+#endif
+}
+GD_FX i64 mulhi_s(i64 a, i64 b)
+{
+#ifdef __CUDA_ARCH__
+    return __mul64hi(a, b);
+#else
+    return (i64)(((__int128)a * b) >> 64);
+#endif
+}
+GD_FX int mulhi_s32(int a, int b) { return (int)(((i64)a * b) >> 32); }
+GD_FX uint32_t mulhi_u32(uint32_t a, uint32_t b) { return (uint32_t)(((u64)a * b) >> 32); }
+GD_FX u64 bits_of(double v)
+{
+#ifdef __CUDA_ARCH__
+    return (u64)__double_as_longlong(v);
+#else
+    u64 b;
+    __builtin_memcpy(&b, &v, 8);
+    return b;
+#endif
+}
+GD_FX double of_bits(u64 b)
+{
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((i64)b);
+#else
+    double v;
+    __builtin_memcpy(&v, &b, 8);
+    return v;
+#endif
+}
+GD_FX int clz64(u64 a)
+{
+#ifdef __CUDA_ARCH__
+    return __clzll((i64)a);
+#else
+    return a ? __builtin_clzll(a) : 64;
+#endif
+}
+
+// Tables, computed in 110-bit integer arithmetic: e[i] = 2^64 2^(-i/256) (e[0] = 2^64 - 1),
+// n[i] = 2^16 / (1 + (i + 1/2) / 256) rounded to an integer, l[i] = 2^62 ln(2^16 / n[i]).
+struct Tables {
+    u64 e[256];
+    u64 l[256];
+    uint32_t n[256];
+};
+using u128 = unsigned __int128;
+constexpr u128 mul_q110(u128 a, u128 b)   // (a b) >> 110 for operands below 2^111
+{
+    const u128 m = ((u128)1 << 55) - 1;
+    const u128 ah = a >> 55, al = a & m, bh = b >> 55, bl = b & m;
+    return ah * bh + ((ah * bl + al * bh) >> 55) + ((al * bl) >> 110);
+}
+constexpr Tables make_tables()
+{
+    Tables t{};
+    const u128 one = (u128)1 << 110;
+    // ln 2 = 0.B17217F7D1CF79ABC9E3B39803F2F6AF (hexadecimal)
+    const u128 ln2 = (((u128)0xB17217F7D1CF79ABull << 64) | 0xC9E3B39803F2F6AFull) >> 18;
+    const u128 x = ln2 >> 8;
+    u128 q = one, term = one;              // q = exp(-ln2 / 256)
+    for (int n = 1; n < 20; ++n) {
+        term = mul_q110(term, x) / n;
+        q = (n & 1) ? q - term : q + term;
+    }
+    u128 v = one;
+    for (int i = 0; i < 256; ++i) {
+        const u128 r = (v + ((u128)1 << 45)) >> 46;
+        t.e[i] = (r >> 64) ? ~0ull : (u64)r;
+        v = mul_q110(v, q);
+        const uint32_t num = (2u * 65536u * 512u / (513u + 2u * i) + 1u) / 2u;
+        t.n[i] = num;
+        // ln(65536 / num) = 2 atanh z
+        const u128 z = (((u128)(65536u - num)) << 110) / (65536u + num);
+        const u128 z2 = mul_q110(z, z);
+        u128 p = z, s = 0;
+        for (int k = 1; k < 80 && p; k += 2) {
+            s += p / k;
+            p = mul_q110(p, z2);
+        }
+        t.l[i] = (u64)((s + ((u128)1 << 46)) >> 47);
+    }
+    return t;
+}
+#ifdef __CUDACC__
+__device__ const Tables d_tab = make_tables();
+#endif
+#ifndef __CUDA_ARCH__
+constexpr Tables h_tab = make_tables();
+#endif
+GD_FX u64 tab_e(int i)
+{
+#ifdef __CUDA_ARCH__
+    return __ldg(&d_tab.e[i]);
+#else
+    return h_tab.e[i];
+#endif
+}
+GD_FX u64 tab_l(int i)
+{
+#ifdef __CUDA_ARCH__
+    return __ldg(&d_tab.l[i]);
+#else
+    return h_tab.l[i];
+#endif
+}
+GD_FX uint32_t tab_n(int i)
+{
+#ifdef __CUDA_ARCH__
+    return __ldg(&d_tab.n[i]);
+#else
+    return h_tab.n[i];
+#endif
+}
+
+// v 2^e rounded to the nearest double (0 below the normal range, infinity above)
+GD_FX double to_double(i64 v, int e)
+{
+    if (v == 0) return 0.0;
+    const u64 s = (u64)v & (1ull << 63);
+    u64 a = s ? 0ull - (u64)v : (u64)v;
+    const int lz = clz64(a);
+    a <<= lz;
+    const u64 m = (a >> 11) + ((a >> 10) & 1);      // 53 bits; a carry raises the exponent
+    int ex = 1023 + 63 - lz + e;
+    if (ex <= 0) return 0.0;
+    if (ex >= 2046) return of_bits(s | 0x7ff0000000000000ull);
+    return of_bits(s | (((u64)(ex - 1) << 52) + m));
+}
+// z 2^f rounded to an integer; |z| 2^f below 2^62
+GD_FX i64 from_double(double z, int f)
+{
+    const u64 b = bits_of(z), ab = b & 0x7fffffffffffffffull;
+    const int sh = (int)(ab >> 52) - 1075 + f;
+    const u64 m = (ab & 0xfffffffffffffull) | 0x10000000000000ull;
+    i64 x;
+    if (sh >= 0) x = (i64)(m << (sh < 10 ? sh : 10));
+    else x = sh < -53 ? 0 : (i64)((m + (1ull << (-sh - 1))) >> -sh);
+    return (b >> 63) ? -x : x;
+}
+// two signed 28-bit limbs: x = hi 2^28 + lo, |lo| <= 2^27
+GD_FX int2 limbs(i64 x)
+{
+    const i64 hi = (x + (1LL << (kLimb - 1))) >> kLimb;
+    int2 r;
+    r.x = (int)hi;
+    r.y = (int)(x - (hi << kLimb));
+    return r;
+}
+
+// exponent e with |v| < 2^e (0 for v = 0)
+GD_FX int bound_exp(double v)
+{
+    const u64 ab = bits_of(v) & 0x7fffffffffffffffull;
+    return ab == 0 ? 0 : (int)(ab >> 52) - 1022;
+}
+
+// softplus(h) in units of 2^-57 (|h| < 64; beyond, softplus is h or 0 to that precision and
+// the caller takes h itself for h >= 64) and sigmoid(h) in units of 2^-62.
+//   e = exp(-|h|) = 2^-n 2^(-i/256) 2^-r, 2^-r by its Taylor series (r < 2^-8, degree 5);
+//   log(1 + e) = ln(2^16/n_i) + log1p(r'), 1 + r' = (1 + e) n_i / 2^16, |r'| < 2^-8.9, degree 5;
+//   1 / (1 + e) = (n_i / 2^16) / (1 + r'), geometric series to r'^6.
+GD_FX void softplus_sigmoid(double h, i64 &s57, i64 &sg62)
+{
+    const u64 hb = bits_of(h), ab = hb & 0x7fffffffffffffffull;
+    const bool neg = (hb >> 63) != 0;
+    const int sh = (int)(ab >> 52) - 1023 + 5;
+    const u64 m = (ab & 0xfffffffffffffull) | 0x10000000000000ull;
+    u64 T = sh >= 0 ? m << (sh < 10 ? sh : 10) : (sh < -53 ? 0 : m >> -sh);
+    if (sh > 10) T = 63ull << 57;
+    // exponential
+    const u64 y = mulhi_u(T, 0xB8AA3B295C17F0BCull);               // |h| log2(e), 56 fraction bits
+    const int n = (int)(y >> 56);
+    const u64 rr = (y & 0xffffffffffffull) << 8;                   // r, 64 fraction bits
+    const uint32_t rh = (uint32_t)(rr >> 24);                      // r, 40 fraction bits
+    // ln2^3/6, ln2^4/24, ln2^5/120 with 36 fraction bits; ln2^2/2, ln2 with 64
+    const uint32_t q = 3814213304u - (mulhi_u32(rh, 660952799u - (mulhi_u32(rh, 91627514u) >> 8)) >> 8);
+    const u64 a = 4431396893595737425ull - mulhi_u(rr, (u64)q << 28);
+    const u64 b = 12786308645202655660ull - mulhi_u(rr, a);
+    u64 e = mulhi_u(tab_e((int)(y >> 48) & 255), ~mulhi_u(rr, b));
+    e = n > 63 ? 0 : e >> n;                                       // exp(-|h|), 64 fraction bits
+    // logarithm
+    const int i = (int)(e >> 56);
+    const u64 inv = (u64)tab_n(i) << 48;
+    const i64 rs = (i64)(mulhi_u((1ull << 63) | (e >> 1), inv) - (1ull << 63)) << 8;   // r', 71 bits
+    const int rx = (int)(rs >> 32);                                // r', 39 bits
+    const int L = 715827883 - (mulhi_s32(rx, 536870912 - (mulhi_s32(rx, 429496730) >> 7)) >> 7);
+    const i64 x2 = (1LL << 61) - (mulhi_s(rs, (i64)L << 31) >> 7);
+    const i64 x1 = kOne62 - (mulhi_s(rs, x2) >> 7);
+    const i64 lg = (i64)tab_l(i) + (mulhi_s(rs, x1) >> 7);
+    s57 = (i64)(neg ? 0ull : T) + ((lg + 16) >> 5);
+    // sigmoid
+    const int k1 = 1 << 30;
+    const int qs = k1 - (mulhi_s32(rx, k1 - (mulhi_s32(rx, k1 - (rx >> 9)) >> 7)) >> 7);
+    const i64 w2 = kOne62 - (mulhi_s(rs, (i64)qs << 32) >> 7);
+    const i64 w1 = kOne62 - (mulhi_s(rs, w2) >> 7);
+    const i64 w0 = kOne62 - (mulhi_s(rs, w1) >> 7);
+    const i64 sig = (i64)mulhi_u((u64)w0, inv);
+    sg62 = neg ? kOne62 - sig : sig;
+}
+
+// scale of a point's softplus operands: exponent e_p with softplus(h) < 2^e_p for every h
+// whose high word is at most hi_max (the largest signed high word of the point's units)
+GD_FX int softplus_exp(int hi_max)
+{
+    const int ex = hi_max <= 0 ? -1023 : (hi_max >> 20) - 1023;
+    return ex < -1 ? 0 : (ex == -1 ? 1 : ex + 2);
+}
+// softplus as an operand: units of 2^(e_p - 56)
+GD_FX i64 softplus_operand(double h, i64 s57, int e_p)
+{
+    const bool big = (int)(bits_of(h) >> 52) >= 1023 + 6;          // h >= 64 (positive)
+    if (big && !(bits_of(h) >> 63)) return from_double(h, kBits - e_p);
+    const int sh = 1 + e_p;
+    return sh > 62 ? 0 : (s57 + (1LL << (sh - 1))) >> sh;
+}
+
+// Fixed-point copies of one network (built on the device whenever its weights change).
+// Weight tables are stored [j][wp] with the outputs of a 16-wide chunk permuted so that the
+// lane sub = k mod 4 of a point finds its four outputs k = c0 + 4 i + sub in 32 consecutive
+// bytes.
+struct Net {
+    const int2 *W2, *W2T;      // [w][wp] limbs: W2[k][j] at (j, perm k), scaled by 2^(56 - e[k]);
+                               // transposed: W2[k][j] at (k, perm j), scaled by 2^(56 - e[w + j])
+    const float *W2P;          // [w][wp] FP32 W2[k][j] at (j, perm k)
+    const i64 *W1;             // [w][4] first-layer weights in units of 2^(e1 - 62)
+    const i64 *w3;             // [w] output weights in units of 2^(e3 - 62)
+    const double *WW;          // [w][6] products W1_a W1_b (sym6 order; energy network)
+    const int *e;              // [w] rows of W2, [w] rows of W2^T, then e1, e3
+};
+GD_FX int pad16(int w) { return (w + 15) / 16 * 16; }
+GD_FX int perm16(int k) { return (k & ~15) + (k & 3) * 4 + ((k >> 2) & 3); }
+GD_FX size_t net_bytes(int w)
+{
+    const size_t wp = pad16(w);
+    return (size_t)w * wp * 20 + (size_t)w * (32 + 8 + 48) + (size_t)(2 * w + 4) * 4;
+}
+GD_FX Net net_of(const unsigned char *base, int w)
+{
+    const size_t t = (size_t)w * pad16(w);
+    Net n;
+    n.W2 = reinterpret_cast<const int2 *>(base);
+    n.W2T = n.W2 + t;
+    n.W2P = reinterpret_cast<const float *>(n.W2T + t);
+    n.W1 = reinterpret_cast<const i64 *>(n.W2P + t);
+    n.w3 = n.W1 + (size_t)w * 4;
+    n.WW = reinterpret_cast<const double *>(n.w3 + w);
+    n.e = reinterpret_cast<const int *>(n.WW + (size_t)w * 6);
+    return n;
+}
+
+}  // namespace fx
+}  // namespace gd

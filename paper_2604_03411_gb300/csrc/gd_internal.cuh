@@ -31,6 +31,7 @@ struct DevNet {
     double *W2T = nullptr;   // [width * width], W2T[j * w + k] = W2[k * w + j]
     float *pf = nullptr;     // FP32 copies for the mixed-precision kernel
     float *W2Tf = nullptr;
+    unsigned char *fx = nullptr;   // fixed-point copies for the FP64 element kernel (gd_fixed.cuh)
 };
 
 struct MatConst {
@@ -323,6 +324,9 @@ cudaError_t launch_adjoint_globals(const DevNet &psi, const DevNet &yld, int ene
                                    double *theta_bar, cudaStream_t s);
 // FP32 copies of a network's parameters and transposed W2
 cudaError_t launch_net_to_float(const DevNet &net, cudaStream_t s);
+// fixed-point copies of a network (fx; net_fixed_bytes bytes)
+size_t net_fixed_bytes(int width);
+cudaError_t launch_net_fixed(const DevNet &net, cudaStream_t s);
 
 // solver kernels (gd_solver.cu)
 struct SolverCtx {

@@ -1,0 +1,352 @@
+// gd_net_fp64.cuh -- the ICNNs of the FP64 element kernel, four lanes per quadrature
+// point (eight points of a warp at once): lane sub = lane mod 4 of point pt = lane / 4 owns
+// the units j, k = sub (mod 4) of every layer.  Pre-activations and the sums over the second
+// layer's units are FP64; activations and the layer products are 64-bit fixed point
+// (gd_fixed.cuh).  The FP32 evaluations of the local solve use the same mapping.
+// Every function is called by the whole warp; `need` marks the points that take part (all
+// four lanes of a point agree) and net is the same for all of them.
+#pragma once
+
+#include "gd_elem32.cuh"
+#include "gd_fixed.cuh"
+
+namespace gd {
+namespace grp {
+
+using fx::i64;
+
+constexpr int kLanes = 4;                  // lanes per point
+constexpr int kPts = 32 / kLanes;          // points per round
+
+// shared-memory bytes of a warp's network buffers for width w: operands [w][8][4], one
+// 64-bit word [w][8] per unit, reverse operands [w][8]
+__host__ __device__ inline size_t buf_bytes(int w) { return (size_t)w * kPts * (4 + 1 + 1) * 8; }
+
+template <class T>
+__device__ __forceinline__ T sum4(T v)
+{
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    return v;
+}
+__device__ __forceinline__ int max4(int v)
+{
+    v = max(v, __shfl_xor_sync(0xffffffffu, v, 1));
+    return max(v, __shfl_xor_sync(0xffffffffu, v, 2));
+}
+__device__ __forceinline__ int hi_word(double v) { return __double2hiint(v); }
+
+// NC column products of a 16-wide output chunk: V[i][c] = sum_j W(k_i, j) z_c(j) in units of
+// 2^-56 (times the operand and row scales), k_i = c0 + 4 i + sub.  Three multiply-adds per
+// term: hi hi into one sum, hi lo + lo hi into the other.  z: operand c of unit j and point pt
+// at z[(j 8 + pt) ZS + c].
+template <int NC, int ZS>
+__device__ __forceinline__ void chunk_product(const int2 *__restrict__ W, int wp, int c0, const int2 *z, int n, int pt,
+                                              int sub, i64 (&V)[4][NC])
+{
+    i64 hh[4][NC], md[4][NC];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) hh[i][c] = md[i][c] = 0;
+    const int4 *wr = reinterpret_cast<const int4 *>(W + c0 + sub * 4);
+    const int2 *zr = z + pt * ZS;
+#pragma unroll 2
+    for (int j = 0; j < n; ++j) {
+        const int4 wa = __ldg(wr), wb = __ldg(wr + 1);
+        wr += wp / 2;
+        const int wh[4] = {wa.x, wa.z, wb.x, wb.z}, wl[4] = {wa.y, wa.w, wb.y, wb.w};
+        int zh[NC], zl[NC];
+        if (NC == 4) {
+            const int4 a = reinterpret_cast<const int4 *>(zr)[0], b = reinterpret_cast<const int4 *>(zr)[1];
+            zh[0] = a.x; zl[0] = a.y;
+            if (NC > 1) { zh[1 % NC] = a.z; zl[1 % NC] = a.w; }
+            if (NC > 2) { zh[2 % NC] = b.x; zl[2 % NC] = b.y; zh[3 % NC] = b.z; zl[3 % NC] = b.w; }
+        } else if (NC == 2) {
+            const int4 a = reinterpret_cast<const int4 *>(zr)[0];
+            zh[0] = a.x; zl[0] = a.y;
+            zh[1 % NC] = a.z; zl[1 % NC] = a.w;
+        } else {
+            const int2 a = zr[0];
+            zh[0] = a.x; zl[0] = a.y;
+        }
+        zr += kPts * ZS;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                hh[i][c] += (i64)zh[c] * wh[i];
+                md[i][c] += (i64)zh[c] * wl[i];
+                md[i][c] += (i64)zl[c] * wh[i];
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) V[i][c] = hh[i][c] + ((md[i][c] + (1LL << 27)) >> fx::kLimb);
+}
+
+// Energy network N(y) with gradient and (hess) Hessian in sym6 order, for the points with
+// need: y at sY[pt 4 ..], results to sO[pt 10 ..].  Same identities as psi_net_unit:
+//   d2N/dy2 = sum_k w3_k sp''(h2_k) g_k g_k^T + sum_j v_j sp''(h1_j) W1_j W1_j^T,
+//   v = W2^T (w3 o sp'(h2)).
+__device__ __forceinline__ void energy(const DevNet &net, const double *sY, double *sO, unsigned char *buf, int lane,
+                                       bool need, bool hess)
+{
+    const int w = net.width, wp = fx::pad16(w), pt = lane >> 2, sub = lane & 3;
+    const double *W1 = net.p, *b1 = W1 + 3 * w, *A2 = b1 + w + w * w, *b2 = A2 + 3 * w, *w3 = b2 + w, *a3 = w3 + w;
+    const fx::Net fn = fx::net_of(net.fx, w);
+    int2 *z = reinterpret_cast<int2 *>(buf);                    // [w][8][4]
+    i64 *sE = reinterpret_cast<i64 *>(z + w * kPts * 4);        // [w][8]: h1, then sp''(h1)
+    int2 *su = reinterpret_cast<int2 *>(sE + w * kPts);         // [w][8]
+    double y0 = sY[pt * 4], y1 = sY[pt * 4 + 1], y2 = sY[pt * 4 + 2];
+    const bool bad = !(isfinite(y0) && isfinite(y1) && isfinite(y2));
+    if (bad || !need) y0 = y1 = y2 = 0.0;
+    // layer 1: pre-activations and the point's operand scale
+    int hm = 0;
+    for (int j = sub; j < w; j += kLanes) {
+        const double h =
+            fma(__ldg(W1 + 3 * j + 2), y2, fma(__ldg(W1 + 3 * j + 1), y1, fma(__ldg(W1 + 3 * j), y0, __ldg(b1 + j))));
+        sE[j * kPts + pt] = __double_as_longlong(h);
+        hm = max(hm, hi_word(h));
+    }
+    const int ep = fx::softplus_exp(max4(hm)), ew1 = fn.e[2 * w], ew3 = fn.e[2 * w + 1];
+    for (int j = sub; j < w; j += kLanes) {
+        const double h = __longlong_as_double(sE[j * kPts + pt]);
+        i64 s, g;
+        fx::softplus_sigmoid(h, s, g);
+        const i64 *w1 = fn.W1 + 4 * j;
+        const int2 l0 = fx::limbs(fx::softplus_operand(h, s, ep));
+        const int2 l1 = fx::limbs((fx::mulhi_s(g, __ldg(w1)) + 8) >> 4);
+        const int2 l2 = fx::limbs((fx::mulhi_s(g, __ldg(w1 + 1)) + 8) >> 4);
+        const int2 l3 = fx::limbs((fx::mulhi_s(g, __ldg(w1 + 2)) + 8) >> 4);
+        int4 *zz = reinterpret_cast<int4 *>(z + (j * kPts + pt) * 4);
+        zz[0] = make_int4(l0.x, l0.y, l1.x, l1.y);
+        zz[1] = make_int4(l2.x, l2.y, l3.x, l3.y);
+        sE[j * kPts + pt] = fx::mulhi_s(g, fx::kOne62 - g) << 2;
+    }
+    __syncwarp();
+    double acc[10];
+#pragma unroll
+    for (int c = 0; c < 10; ++c) acc[c] = 0.0;
+    for (int c0 = 0; c0 < wp; c0 += 16) {
+        i64 V[4][4];
+        chunk_product<4, 4>(fn.W2, wp, c0, z, w, pt, sub, V);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int k = c0 + 4 * i + sub;
+            if (k < w) {
+                const int er = __ldg(fn.e + k) - fx::kBits;
+                const double q0 = __ldg(A2 + 3 * k), q1 = __ldg(A2 + 3 * k + 1), q2 = __ldg(A2 + 3 * k + 2);
+                const double h =
+                    fx::to_double(V[i][0], er + ep) + fma(q2, y2, fma(q1, y1, fma(q0, y0, __ldg(b2 + k))));
+                const double g0 = fx::to_double(V[i][1], er + ew1) + q0, g1 = fx::to_double(V[i][2], er + ew1) + q1,
+                             g2 = fx::to_double(V[i][3], er + ew1) + q2;
+                i64 s, g;
+                fx::softplus_sigmoid(h, s, g);
+                const i64 uq = fx::mulhi_s(__ldg(fn.w3 + k), g);              // units of 2^(ew3 - 60)
+                const double u = fx::to_double(uq, ew3 - 60);
+                acc[0] += __ldg(w3 + k) * (hi_word(h) >= 0x40500000 ? h : fx::to_double(s, -57));
+                acc[1] += u * g0;
+                acc[2] += u * g1;
+                acc[3] += u * g2;
+                if (hess) {
+                    const double e2 = fx::to_double(fx::mulhi_s(uq, fx::kOne62 - g), ew3 - 58);
+                    const double e0 = e2 * g0, e1 = e2 * g1;
+                    acc[4] += e0 * g0;
+                    acc[5] += e0 * g1;
+                    acc[6] += e0 * g2;
+                    acc[7] += e1 * g1;
+                    acc[8] += e1 * g2;
+                    acc[9] += e2 * g2 * g2;
+                    su[k * kPts + pt] = fx::limbs((uq + 8) >> 4);
+                }
+            }
+        }
+    }
+    if (hess) {
+        __syncwarp();
+        for (int c0 = 0; c0 < wp; c0 += 16) {
+            i64 V[4][1];
+            chunk_product<1, 1>(fn.W2T, wp, c0, su, w, pt, sub, V);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int j = c0 + 4 * i + sub;
+                if (j < w) {
+                    const double c =
+                        fx::to_double(fx::mulhi_s(V[i][0], sE[j * kPts + pt]), __ldg(fn.e + w + j) + ew3 - 54);
+                    const double *ww = fn.WW + 6 * j;
+#pragma unroll
+                    for (int m = 0; m < 6; ++m) acc[4 + m] += c * __ldg(ww + m);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 10; ++c)
+        if (c < 4 || hess) acc[c] = sum4(acc[c]);
+    if (sub == 0 && need) {
+        double *o = sO + pt * 10;
+        const double nan = __longlong_as_double(0x7ff8000000000000LL);
+        o[0] = acc[0] + __ldg(a3) * y0 + __ldg(a3 + 1) * y1 + __ldg(a3 + 2) * y2;
+        o[1] = acc[1] + __ldg(a3);
+        o[2] = acc[2] + __ldg(a3 + 1);
+        o[3] = acc[3] + __ldg(a3 + 2);
+#pragma unroll
+        for (int c = 4; c < 10; ++c) o[c] = hess ? acc[c] : 0.0;
+        if (bad)
+#pragma unroll
+            for (int c = 0; c < 10; ++c) o[c] = nan;
+    }
+    __syncwarp();
+}
+
+// Yield network N_k(q) and, with SLOPE, N_k'(q) (parameters p and fixed-point copy fxp of a
+// network of width w > 0).  Every lane of a point returns the same values.
+template <bool SLOPE>
+static __device__ __noinline__ double2 yield(const double *p, const unsigned char *fxp, int w, double q,
+                                             unsigned char *buf, int lane, bool need)
+{
+    constexpr int NC = SLOPE ? 2 : 1;
+    const int wp = fx::pad16(w), pt = lane >> 2, sub = lane & 3;
+    const double *V1 = p, *c1 = V1 + w, *B2 = c1 + w + w * w, *c2 = B2 + w, *v3 = c2 + w, *b3 = v3 + w;
+    const fx::Net fn = fx::net_of(fxp, w);
+    int2 *z = reinterpret_cast<int2 *>(buf);                       // [w][8][NC]
+    i64 *sE = reinterpret_cast<i64 *>(z + w * kPts * NC);
+    const bool bad = !isfinite(q);
+    if (bad || !need) q = 0.0;
+    int hm = 0;
+    for (int j = sub; j < w; j += kLanes) {
+        const double h = fma(__ldg(V1 + j), q, __ldg(c1 + j));
+        sE[j * kPts + pt] = __double_as_longlong(h);
+        hm = max(hm, hi_word(h));
+    }
+    const int ep = fx::softplus_exp(max4(hm)), ew1 = fn.e[2 * w], ew3 = fn.e[2 * w + 1];
+    for (int j = sub; j < w; j += kLanes) {
+        const double h = __longlong_as_double(sE[j * kPts + pt]);
+        i64 s, g;
+        fx::softplus_sigmoid(h, s, g);
+        int2 *zz = z + (j * kPts + pt) * NC;
+        zz[0] = fx::limbs(fx::softplus_operand(h, s, ep));
+        if (SLOPE) zz[NC - 1] = fx::limbs((fx::mulhi_s(g, __ldg(fn.W1 + 4 * j)) + 8) >> 4);
+    }
+    __syncwarp();
+    double n0 = 0.0, n1 = 0.0;
+    for (int c0 = 0; c0 < wp; c0 += 16) {
+        i64 V[4][NC];
+        chunk_product<NC, NC>(fn.W2, wp, c0, z, w, pt, sub, V);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int k = c0 + 4 * i + sub;
+            if (k < w) {
+                const int er = __ldg(fn.e + k) - fx::kBits;
+                const double b = __ldg(B2 + k);
+                const double h = fx::to_double(V[i][0], er + ep) + fma(b, q, __ldg(c2 + k));
+                i64 s, g;
+                fx::softplus_sigmoid(h, s, g);
+                n0 += __ldg(v3 + k) * (hi_word(h) >= 0x40500000 ? h : fx::to_double(s, -57));
+                if (SLOPE)
+                    n1 += fx::to_double(fx::mulhi_s(__ldg(fn.w3 + k), g), ew3 - 60) *
+                          (fx::to_double(V[i][NC - 1], er + ew1) + b);
+            }
+        }
+    }
+    const double b = __ldg(b3), nan = __longlong_as_double(0x7ff8000000000000LL);
+    double2 r = make_double2(sum4(n0) + b * q, 0.0);
+    if (SLOPE) r.y = sum4(n1) + b;
+    if (bad) r = make_double2(nan, nan);
+    __syncwarp();
+    return r;
+}
+
+// r(kappa) = G(q(kappa)) - kappa (Eq. (potential_function)), q = psi_e + qcoef (phi - kappa) /
+// f_d(kappa) (Eq. (ostwald_potential)); SLOPE: dr/dkappa and G' too
+template <bool SLOPE>
+__device__ __forceinline__ void residual(const MatConst &m, const DevNet &yld, const NetConst &nc, double pe,
+                                         double phi, double kappa, double &r, double &dr, double &Gp,
+                                         unsigned char *buf, int lane, bool need)
+{
+    const bool dmg = kappa > m.kappa_d;
+    const double f = dmg ? exp(-m.eta_d * (kappa - m.kappa_d)) : 1.0;
+    const double q = pe + m.qcoef * (phi - kappa) / f;
+    // G(q) = s (N_k(q) - N_k(0)) (Eq. (Gq_NN)); width 0 is the identity G(q) = q
+    double G = q, Gs = 1.0;
+    if (yld.width > 0) {
+        const double2 n = yield<SLOPE>(yld.p, yld.fx, yld.width, q, buf, lane, need);
+        G = nc.y_s * (n.x - nc.y_N0);
+        Gs = nc.y_s * n.y;
+    }
+    r = G - kappa;
+    if (SLOPE) {
+        Gp = Gs;
+        dr = Gs * (m.qcoef * ((dmg ? (phi - kappa) * m.eta_d - 1.0 : -1.0) / f)) - 1.0;
+    }
+}
+
+// N_k(q) and N_k'(q) in FP32
+static __device__ __noinline__ float2 yield32(const float *p, const unsigned char *fxp, int w, float q,
+                                              unsigned char *buf, int lane)
+{
+    const int wp = fx::pad16(w), pt = lane >> 2, sub = lane & 3;
+    const float *V1 = p, *c1 = V1 + w, *B2 = c1 + w + w * w, *c2 = B2 + w, *v3 = c2 + w, *b3 = v3 + w;
+    const float4 *W2P = reinterpret_cast<const float4 *>(fx::net_of(fxp, w).W2P);
+    float2 *z = reinterpret_cast<float2 *>(buf);                   // [w][8]
+    for (int j = sub; j < w; j += kLanes) {
+        const float a = __ldg(V1 + j);
+        float s, g;
+        e32::sp_sig(__ldg(c1 + j) + a * q, s, g);
+        z[j * kPts + pt] = make_float2(s, g * a);
+    }
+    __syncwarp();
+    float n0 = 0.0f, n1 = 0.0f;
+    for (int c0 = 0; c0 < wp; c0 += 16) {
+        float h[4] = {0.0f, 0.0f, 0.0f, 0.0f}, t[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        const float4 *wr = W2P + c0 / 4 + sub;
+#pragma unroll 4
+        for (int j = 0; j < w; ++j) {
+            const float4 a = __ldg(wr + j * (wp / 4));
+            const float2 v = z[j * kPts + pt];
+            h[0] += a.x * v.x; t[0] += a.x * v.y;
+            h[1] += a.y * v.x; t[1] += a.y * v.y;
+            h[2] += a.z * v.x; t[2] += a.z * v.y;
+            h[3] += a.w * v.x; t[3] += a.w * v.y;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int k = c0 + 4 * i + sub;
+            if (k < w) {
+                const float b = __ldg(B2 + k), vk = __ldg(v3 + k);
+                float s, g;
+                e32::sp_sig(h[i] + __ldg(c2 + k) + b * q, s, g);
+                n0 += vk * s;
+                n1 += vk * g * (t[i] + b);
+            }
+        }
+    }
+    const float b = __ldg(b3);
+    const float2 r = make_float2(sum4(n0) + b * q, sum4(n1) + b);
+    __syncwarp();
+    return r;
+}
+
+__device__ __forceinline__ void residual32(const e32::MatF &m, const DevNet &yld, const e32::NcF &nc, float pe,
+                                           float phi, float kappa, float &r, float &dr, float &Gp, unsigned char *buf,
+                                           int lane)
+{
+    const bool dmg = kappa > m.kappa_d;
+    const float f = dmg ? expf(-m.eta_d * (kappa - m.kappa_d)) : 1.0f;
+    const float q = pe + m.qcoef * (phi - kappa) / f;
+    const float dq = m.qcoef * (-1.0f / f + (dmg ? (phi - kappa) * m.eta_d / f : 0.0f));
+    float G = q;
+    Gp = 1.0f;
+    if (yld.width > 0) {
+        const float2 n = yield32(yld.pf, yld.fx, yld.width, q, buf, lane);
+        G = nc.y_s * (n.x - nc.y_N0);
+        Gp = nc.y_s * n.y;
+    }
+    r = G - kappa;
+    dr = Gp * dq - 1.0f;
+}
+
+}  // namespace grp
+}  // namespace gd
