@@ -1,15 +1,15 @@
 // gd_asm_fp64.cu -- FP64 element kernel of the gradient-enhanced damage model.
 //
-// A CTA of KW warps owns 8 KW quadrature points (KW HEX8 or 2 KW Q4 elements) and switches
+// A CTA of KW warps owns NP quadrature points (NP / 8 HEX8 or NP / 4 Q4 elements) and switches
 // between three lane mappings:
-//   qp mode    lane = quadrature point (the first 8 KW threads in an order that rotates
-//              with the batch): kinematics, invariants, energy chain, stress and the
-//              point's tangent in reference coordinates;
-//   net mode   warp = eight points, four lanes each: both ICNN layers of the energy
-//              network (value, gradient by forward tangents, Hessian by one reverse sweep
-//              through layer 2) and every yield-network evaluation of the local damage
+//   qp mode    thread = quadrature point (NP threads in an order that rotates with the
+//              batch): kinematics, invariants, energy chain, stress and the point's tangent
+//              in reference coordinates;
+//   net mode   warp = four points at a time, eight lanes each: both ICNN layers of the
+//              energy network (value, gradient by forward tangents, Hessian by one reverse
+//              sweep through layer 2) and every yield-network evaluation of the local damage
 //              solve, whose points iterate in lockstep (gd_net_fp64.cuh);
-//   row mode   warp = its eight points' elements, lane = element row (node a, dof i): the
+//   row mode   warp = the elements of eight points, lane = element row (node a, dof i): the
 //              rows of the residual and of the consistent tangent, scattered into CSR
 //              through the slot map.
 //
@@ -25,9 +25,11 @@
 //    closed form of every (a, b) pair.
 //  - The networks run in 64-bit fixed point (gd_fixed.cuh).
 // Measured (GB300, gd_assemble with tangent; before: FP64 networks one point at a time with
-// a lane per unit, closed-form rows): 140,400 points of HEX8, both widths 64, 33.6 -> 7.5 ms;
-// 159,744 of Q4, widths 32, 10.1 -> 2.4 ms; 256 of Q4, widths 16 and 8, 1.24 -> 0.10 ms;
-// residual alone of 32,640 HEX8 points, widths 24 and 40, 3.55 -> 0.63 ms.
+// a lane per unit, closed-form rows): 140,400 points of HEX8, both widths 64, 33.6 -> 5.75 ms;
+// 159,744 of Q4, widths 32, 10.2 -> 2.4 ms; 256 of Q4, widths 16 and 8, 1.21 -> 0.085 ms;
+// residual alone of 32,640 HEX8 points, widths 24 and 40, 3.53 -> 0.50 ms.  16 warps per SM
+// (128 registers, the points' state in shared memory) against 8 with 255 registers: 7.5 ->
+// 5.75 ms on the first; instruction latency is the leading stall, the FP64 pipe 30 % busy.
 //
 // Paper passages: Sec. 3.1 (F, phi_q, grad phi_q, element residual, Table
 // kernel_inputs), Sec. 2.1 (P, Y vector, Y), Sec. 2.2 and Sec. 3.2 Eq. (dd_7_no_nn)
@@ -75,17 +77,27 @@ __device__ __forceinline__ int sym_pos(int r, int c)
     return lo * N - lo * (lo - 1) / 2 + hi - lo;
 }
 
-// shared-memory layout of a CTA of KW warps, in doubles
-template <int DIM, int KW>
+// What a point keeps between its qp phases, in doubles (registers would halve the resident
+// warps)
+template <int DIM>
+struct State {
+    static constexpr int F = 0, JI = F + DIM * DIM, GX = JI + DIM * DIM, X = GX + DIM, PHI = X + 3, DET = PHI + 1;
+    static constexpr int PS = DET + 1, PH = PS + 3;
+    static constexpr int SIZE = (PH + 6) | 1;
+};
+
+// shared-memory layout of a CTA of KW warps with NP points, in doubles
+template <int DIM, int NP, int KW>
 struct Smem {
     using G_ = Geo<DIM>;
-    static constexpr int NP = 8 * KW, EL = NP / G_::NQ;
+    static constexpr int EL = NP / G_::NQ;
     static constexpr int X = 0;                                      // [EL][NEN][DIM]
     static constexpr int D = X + EL * G_::NEN * DIM;                 // [EL][NEN][NDOF]
     static constexpr int REF = D + EL * G_::NEN * G_::NDOF;          // [NQ][NEN][4] dN/dxi, N
     static constexpr int IN = REF + G_::NQ * G_::NEN * 4;            // [NP][4] network input / psi_e, phi, kappa_n
     static constexpr int OUT = IN + NP * 4;                          // [NP][10] network output / local update
-    static constexpr int U = OUT + NP * 10;                          // network buffers, then the points' records
+    static constexpr int ST = OUT + NP * 10;                         // [NP] State
+    static constexpr int U = (ST + NP * State<DIM>::SIZE + 1) / 2 * 2;   // network buffers, then the points' records
     __host__ __device__ static int net(int wmax) { return (int)(grp::buf_bytes(wmax) / 8); }
     __host__ __device__ static int total(int wmax)
     {
@@ -179,9 +191,9 @@ __device__ __forceinline__ void expand_rows(const double (&T)[3][8], const doubl
 // node with the axis bits l (x lowest): counter-clockwise numbering of each layer
 __device__ __forceinline__ int node_of_bits(int l) { return l ^ ((l >> 1) & 1); }
 
-// Local damage update (Eq. (dd_7_no_nn)) of the points p0 .. p0 + 7 of the warp's batch that
+// Local damage update (Eq. (dd_7_no_nn)) of the CTA's points p0 .. p0 + 3 that
 // belong to specimen sn: psi_e, phi, kappa_n at sIn[p 4 ..], results (kappa, loading, G',
-// dPhi/dkappa, failed) to sOut[p 10 ..].  Four lanes hold each point's state; the points step
+// dPhi/dkappa, failed) to sOut[p 10 ..].  A point's lanes hold its state alike; the points step
 // together, every evaluation running for the points that still need it.  Returns the
 // lane's share of the FP64 evaluations.
 template <int DIM>
@@ -190,7 +202,7 @@ __device__ __forceinline__ int local_update(const AsmArgs &A, const e32::MatF &m
 {
     constexpr int NQ = Geo<DIM>::NQ;
     constexpr unsigned kAll = 0xffffffffu;
-    const int p = p0 + (lane >> 2);
+    const int p = p0 + lane / grp::kLanes;
     const int64_t e_p = e0 + p / NQ;
     const bool need = e_p < A.n_elems && spec_of(A, e_p < A.n_elems ? e_p : A.n_elems - 1) == sn;
     const DevNet &yn = yld_of(A, sn);
@@ -387,7 +399,7 @@ __device__ __forceinline__ int local_update(const AsmArgs &A, const e32::MatF &m
         }
         if (!ok) fail = true;
     }
-    if (need && (lane & 3) == 0) {
+    if (need && lane % grp::kLanes == 0) {
         double *o = sOut + p * 10;
         o[0] = kappa;
         o[1] = load ? 1.0 : 0.0;
@@ -395,17 +407,19 @@ __device__ __forceinline__ int local_update(const AsmArgs &A, const e32::MatF &m
         o[3] = dr;
         o[4] = fail ? 1.0 : 0.0;
     }
-    return (lane & 3) == 0 ? n_eval : 0;
+    return lane % grp::kLanes == 0 ? n_eval : 0;
 }
 
-// KW warps per CTA, eight points each (a launch-shape choice: see launch_dim)
-template <int DIM, int KW>
-__global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
+// NP points and KW warps per CTA (a launch-shape choice: see launch_dim); built for 16 warps
+// per SM
+template <int DIM, int NP, int KW>
+__global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
 {
     using G_ = Geo<DIM>;
-    using S_ = Smem<DIM, KW>;
+    using S_ = Smem<DIM, NP, KW>;
     using R_ = Rec<DIM>;
-    constexpr int NEN = G_::NEN, NQ = G_::NQ, NDOF = G_::NDOF, NP = S_::NP, EL = S_::EL, N2 = DIM * DIM;
+    using P_ = State<DIM>;
+    constexpr int NEN = G_::NEN, NQ = G_::NQ, NDOF = G_::NDOF, EL = S_::EL, N2 = DIM * DIM;
     extern __shared__ __align__(16) double smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double *sX = smem + S_::X, *sD = smem + S_::D, *sRef = smem + S_::REF, *sIn = smem + S_::IN, *sOut = smem + S_::OUT;
@@ -455,9 +469,9 @@ __global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
         const int64_t e_me = e0 + el;
         const bool valid = qp && e_me < A.n_elems;
         const double *ref = sRef + q * NEN * 4;
-        double F[DIM][DIM], Ji[DIM][DIM], gx[DIM], x[3], phi = 0.0, det = 1.0, Jdet = 1.0;
-        double Tm[3][3], T2[3][6];   // dy/dx and d2y/dx2 of the network input map (raw: identity)
+        double *st = smem + S_::ST + pt * P_::SIZE;
         if (qp) {
+            double Ji[DIM][DIM], gx[DIM], x[3], phi = 0.0, det;
             const double *Xe = sX + el * NEN * DIM, *De = sD + el * NEN * NDOF;
             double Jm[DIM][DIM], Gr[DIM][DIM];
 #pragma unroll
@@ -512,7 +526,8 @@ __global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
 #pragma unroll
                     for (int k = 0; k < DIM; ++k) s += Gr[i][k] * Ji[k][J];
                     H[i][J] = s;
-                    F[i][J] = i == J ? s + 1.0 : s;
+                    st[P_::F + i * DIM + J] = i == J ? s + 1.0 : s;
+                    st[P_::JI + i * DIM + J] = Ji[i][J];
                 }
             double tA = 0.0, AA = 0.0, tH = 0.0, HH = 0.0;
 #pragma unroll
@@ -540,31 +555,18 @@ __global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
                 x[2] += H[0][0] * (H[1][1] * H[2][2] - H[1][2] * H[2][1]) -
                         H[0][1] * (H[1][0] * H[2][2] - H[1][2] * H[2][0]) +
                         H[0][2] * (H[1][0] * H[2][1] - H[1][1] * H[2][0]);
-            Jdet = 1.0 + x[2];
-            // network input (raw or isochoric map)
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) st[P_::GX + k] = gx[k];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) st[P_::X + k] = x[k];
+            st[P_::PHI] = phi;
+            st[P_::DET] = det;
+            // network input (raw or isochoric map: I1G = J^-2/3 I1, I2G = I2^3 / (9 J^4), Eq. (dd_0))
             double y[3] = {x[0], x[1], x[2]};
             if (m.energy == GD_ENERGY_ICNN_ISO) {
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) Tm[i][j] = (i == j) ? 1.0 : 0.0;
-#pragma unroll
-                    for (int j = 0; j < 6; ++j) T2[i][j] = 0.0;
-                }
-                // I1G = J^-2/3 I1, I2G = I2^3 / (9 J^4) (Eq. (dd_0)); derivatives wrt (I1-3, I2-3, J-1)
-                double L = log1p(x[2]), E = exp(-2.0 / 3.0 * L), I1 = 3.0 + x[0], I2 = 3.0 + x[1], J = Jdet;
-                y[0] = 3.0 * expm1(-2.0 / 3.0 * L) + x[0] * E;
+                const double L = log1p(x[2]);
+                y[0] = 3.0 * expm1(-2.0 / 3.0 * L) + x[0] * exp(-2.0 / 3.0 * L);
                 y[1] = 3.0 * expm1(3.0 * log1p(x[1] / 3.0) - 4.0 * L);
-                double J4 = J * J * J * J;
-                Tm[0][0] = E;
-                Tm[0][2] = -2.0 / 3.0 * I1 * E / J;
-                Tm[1][1] = I2 * I2 / (3.0 * J4);
-                Tm[1][2] = -4.0 * I2 * I2 * I2 / (9.0 * J4 * J);
-                T2[0][2] = -2.0 / 3.0 * E / J;                       // d2 y1 / dx1 dx3
-                T2[0][5] = 10.0 / 9.0 * I1 * E / (J * J);            // d2 y1 / dx3^2
-                T2[1][3] = 2.0 * I2 / (3.0 * J4);                    // d2 y2 / dx2^2
-                T2[1][4] = -4.0 * I2 * I2 / (3.0 * J4 * J);          // d2 y2 / dx2 dx3
-                T2[1][5] = 20.0 * I2 * I2 * I2 / (9.0 * J4 * J * J); // d2 y2 / dx3^2
             }
             sIn[pt * 4 + 0] = y[0];
             sIn[pt * 4 + 1] = y[1];
@@ -573,31 +575,37 @@ __global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
         cta_sync<KW>();
 
         // ================= net mode: energy network =================
-        // (points of different specimens take turns: a warp's networks are uniform)
-        const int p0 = warp * grp::kPts;
-        const int64_t e_p0 = e0 + p0 / NQ;
-        int s0 = 0, s1 = -1;                     // the specimens of the warp's points
-        if (e_p0 < A.n_elems) {
-            const int64_t e_l = e0 + (p0 + grp::kPts - 1) / NQ;
-            s0 = spec_of(A, e_p0);
-            s1 = spec_of(A, e_l < e_last ? e_l : e_last);
-        }
+        // (points of different specimens take turns: a round's networks are uniform)
+        // specimens of the points p0 .. p0 + 3: s0 .. s1 (none past the last element)
+        auto specimens = [&](int p0, int &s0, int &s1) {
+            const int64_t ea = e0 + p0 / NQ, eb = e0 + (p0 + grp::kPts - 1) / NQ;
+            s0 = 0;
+            s1 = -1;
+            if (ea < A.n_elems) {
+                s0 = spec_of(A, ea);
+                s1 = spec_of(A, eb < e_last ? eb : e_last);
+            }
+        };
         if (m.energy != GD_ENERGY_NEO_HOOKE) {
-            const int64_t e_p = e0 + (p0 + (lane >> 2)) / NQ;
-            const int sp = e_p <= e_last ? spec_of(A, e_p) : -1;
-            for (int sn = s0; sn <= s1; ++sn)
-                grp::energy(psi_of(A, sn), sIn + p0 * 4, sOut + p0 * 10, nbuf, lane, sp == sn, A.tangent != 0);
+#pragma unroll 1
+            for (int p0 = warp * grp::kPts; p0 < NP; p0 += KW * grp::kPts) {
+                int s0, s1;
+                specimens(p0, s0, s1);
+                const int64_t e_p = e0 + (p0 + lane / grp::kLanes) / NQ;
+                const int sp = e_p <= e_last ? spec_of(A, e_p) : -1;
+                for (int sn = s0; sn <= s1; ++sn)
+                    grp::energy(psi_of(A, sn), sIn + p0 * 4, sOut + p0 * 10, nbuf, lane, sp == sn, A.tangent != 0);
+            }
         }
         cta_sync<KW>();
 
         // ================= qp mode: energy derivatives wrt (I1-3, I2-3, J-1) =================
-        double ps[3], ph[6];
         if (qp) {
-            const double J = Jdet, x3 = x[2];
-            double pe;
+            const double x3 = st[P_::X + 2], J = 1.0 + x3;
+            double ps[3], ph[6], pe;
             if (m.energy == GD_ENERGY_NEO_HOOKE) {
                 double L = log1p(x3);
-                pe = 0.5 * m.mu_e * x[0] - m.mu_e * L + 0.5 * m.lambda_e * L * L;
+                pe = 0.5 * m.mu_e * st[P_::X] - m.mu_e * L + 0.5 * m.lambda_e * L * L;
                 ps[0] = 0.5 * m.mu_e;
                 ps[1] = 0.0;
                 ps[2] = (-m.mu_e + m.lambda_e * L) / J;
@@ -612,7 +620,27 @@ __global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
 #pragma unroll
                 for (int c = 0; c < 6; ++c) ph[c] = o[4 + c];
                 if (m.energy == GD_ENERGY_ICNN_ISO) {
-                    // chain through the input map: dN/dx = T^T dN/dy, d2N/dx2 = T^T H T + sum_m dN/dy_m d2y_m/dx2
+                    // chain through the input map: dN/dx = T^T dN/dy, d2N/dx2 = T^T H T + sum_m dN/dy_m d2y_m/dx2,
+                    // T = dy/dx and T2 = d2y/dx2 for x = (I1-3, I2-3, J-1)
+                    double Tm[3][3], T2[3][6];
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) {
+#pragma unroll
+                        for (int j = 0; j < 3; ++j) Tm[i][j] = (i == j) ? 1.0 : 0.0;
+#pragma unroll
+                        for (int j = 0; j < 6; ++j) T2[i][j] = 0.0;
+                    }
+                    const double E = exp(-2.0 / 3.0 * log1p(x3)), I1 = 3.0 + st[P_::X], I2 = 3.0 + st[P_::X + 1];
+                    const double J4 = J * J * J * J;
+                    Tm[0][0] = E;
+                    Tm[0][2] = -2.0 / 3.0 * I1 * E / J;
+                    Tm[1][1] = I2 * I2 / (3.0 * J4);
+                    Tm[1][2] = -4.0 * I2 * I2 * I2 / (9.0 * J4 * J);
+                    T2[0][2] = -2.0 / 3.0 * E / J;                       // d2 y1 / dx1 dx3
+                    T2[0][5] = 10.0 / 9.0 * I1 * E / (J * J);            // d2 y1 / dx3^2
+                    T2[1][3] = 2.0 * I2 / (3.0 * J4);                    // d2 y2 / dx2^2
+                    T2[1][4] = -4.0 * I2 * I2 / (3.0 * J4 * J);          // d2 y2 / dx2 dx3
+                    T2[1][5] = 20.0 * I2 * I2 * I2 / (9.0 * J4 * J * J); // d2 y2 / dx3^2
                     const double gy[3] = {ps[0], ps[1], ps[2]};
                     const double hy[6] = {ph[0], ph[1], ph[2], ph[3], ph[4], ph[5]};
 #pragma unroll
@@ -647,8 +675,12 @@ __global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
                 ps[2] += -m.mu_e * nc.psi_n + m.lambda_e * 2.0 * t * dt;
                 ph[5] += m.lambda_e * 2.0 * (dt * dt + t * d2t);
             }
+#pragma unroll
+            for (int i = 0; i < 3; ++i) st[P_::PS + i] = ps[i];
+#pragma unroll
+            for (int c = 0; c < 6; ++c) st[P_::PH + c] = ph[c];
             sIn[pt * 4 + 0] = pe;
-            sIn[pt * 4 + 1] = phi;
+            sIn[pt * 4 + 1] = st[P_::PHI];
             sIn[pt * 4 + 2] = valid ? __ldg(A.kappa_n + e_me * NQ + q) : 0.0;
         }
         cta_sync<KW>();
@@ -667,8 +699,13 @@ __global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
         } else {
             const e32::MatF mf = e32::to_f(A.mat);
             int n_eval = 0;
-            for (int sn = s0; sn <= s1; ++sn)
-                n_eval += local_update<DIM>(A, mf, e0, p0, sn, sIn, sOut, nbuf, lane);
+#pragma unroll 1
+            for (int p0 = warp * grp::kPts; p0 < NP; p0 += KW * grp::kPts) {
+                int s0, s1;
+                specimens(p0, s0, s1);
+                for (int sn = s0; sn <= s1; ++sn)
+                    n_eval += local_update<DIM>(A, mf, e0, p0, sn, sIn, sOut, nbuf, lane);
+            }
             n_eval = __reduce_add_sync(0xffffffffu, n_eval);
             if (lane == 0 && n_eval) atomicAdd(A.counters + 2, n_eval);
         }
@@ -686,18 +723,26 @@ __global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
                 if (o[4] > 0.5) atomicAdd(A.counters, 1);
             }
             double *rec = sRec + pt * R_::SIZE;
-            const double Jw = valid ? det : 0.0;
+            const double Jw = valid ? st[P_::DET] : 0.0;
             const bool dmg = kappa > m.kappa_d;
-            const double fd = dmg ? exp(-m.eta_d * (kappa - m.kappa_d)) : 1.0;
+            const double fd = dmg ? fx::exp_neg(m.eta_d * (kappa - m.kappa_d)) : 1.0;
             const double fdp = dmg ? -m.eta_d * fd : 0.0;
             const double ck = loading ? -o[2] / o[3] : 0.0;          // G' / (1 - G' dq/dkappa)
             const double dkdphi = ck * m.qcoef / fd;                  // dq/dphi = qcoef / f_d
-            const double J = Jdet, I1 = 3.0 + x[0], ij = 1.0 / J;
+            const double J = 1.0 + st[P_::X + 2], I1 = 3.0 + st[P_::X], ij = 1.0 / J;
+            const double *ps = st + P_::PS, *ph = st + P_::PH;
             // F^-1 = cof(F)^T / J; pulled back to the reference element: F' = F Ji^T (F_iJ Ji_jJ),
             // Fi'_ji = Ji_jJ F^-1_Ji
-            double Fp[DIM][DIM], Fi[DIM][DIM], G2[DIM][DIM], h[DIM], mv[DIM];
+            double Fp[DIM][DIM], Fi[DIM][DIM], G2[DIM][DIM], h[DIM], mv[DIM], b[DIM][DIM], Mj[DIM][DIM];
             {
-                double Fv[DIM][DIM];
+                double Fv[DIM][DIM], F[DIM][DIM], Ji[DIM][DIM];
+#pragma unroll
+                for (int i = 0; i < DIM; ++i)
+#pragma unroll
+                    for (int j = 0; j < DIM; ++j) {
+                        F[i][j] = st[P_::F + i * DIM + j];
+                        Ji[i][j] = st[P_::JI + i * DIM + j];
+                    }
                 if constexpr (DIM == 2) {
                     Fv[0][0] = F[1][1] * ij; Fv[0][1] = -F[0][1] * ij;
                     Fv[1][0] = -F[1][0] * ij; Fv[1][1] = F[0][0] * ij;
@@ -723,13 +768,27 @@ __global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
                         Fp[i][j] = s;
                         Fi[j][i] = t;
                     }
+                // F F^T and the metric (delta_JL pulled back)
+#pragma unroll
+                for (int i = 0; i < DIM; ++i)
+#pragma unroll
+                    for (int k = i; k < DIM; ++k) {
+                        double s = 0.0, t = 0.0;
+#pragma unroll
+                        for (int K = 0; K < DIM; ++K) {
+                            s += F[i][K] * F[k][K];
+                            t += Ji[i][K] * Ji[k][K];
+                        }
+                        b[i][k] = b[k][i] = s;
+                        Mj[i][k] = Mj[k][i] = t;
+                    }
             }
             // h = F^-T grad phi (= Fi'^T of the reference gradient), C^-1 grad phi pulled back
 #pragma unroll
             for (int i = 0; i < DIM; ++i) {
                 double s = 0.0;
 #pragma unroll
-                for (int k = 0; k < DIM; ++k) s += Fi[k][i] * gx[k];
+                for (int k = 0; k < DIM; ++k) s += Fi[k][i] * st[P_::GX + k];
                 h[i] = s;
             }
 #pragma unroll
@@ -739,16 +798,6 @@ __global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
                 for (int i = 0; i < DIM; ++i) s += Fi[j][i] * h[i];
                 mv[j] = s;
             }
-            double b[DIM][DIM];
-#pragma unroll
-            for (int i = 0; i < DIM; ++i)
-#pragma unroll
-                for (int k = i; k < DIM; ++k) {
-                    double s = 0.0;
-#pragma unroll
-                    for (int K = 0; K < DIM; ++K) s += F[i][K] * F[k][K];
-                    b[i][k] = b[k][i] = s;
-                }
             // G^2 = dI2/dF pulled back; P = f_d dpsi_e/dF - c_d h (x) m
             const double ps3J = ps[2] * J, cdw = m.c_d * Jw, fdw = fd * Jw;
 #pragma unroll
@@ -765,7 +814,7 @@ __global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
                 }
 #pragma unroll
             for (int j = 0; j < DIM; ++j) rec[R_::Y + j] = cdw * mv[j];
-            rec[R_::PEN] = m.beta_d * (phi - kappa) * Jw;
+            rec[R_::PEN] = m.beta_d * (st[P_::PHI] - kappa) * Jw;
             if (A.tangent) {
                 rec[R_::FDK] = fdp * dkdphi * Jw;
                 rec[R_::BCK] = m.beta_d * ck * Jw;
@@ -773,17 +822,17 @@ __global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
                 double hw[DIM];                                    // c_d J w h
 #pragma unroll
                 for (int i = 0; i < DIM; ++i) hw[i] = cdw * h[i];
-                double Cv[DIM][DIM], Sj[DIM][DIM], Mj[DIM][DIM];
+                double Cv[DIM][DIM], Sj[DIM][DIM];
                 const double g2w = 2.0 * fdw * ps[1], g1w = 2.0 * fdw * ps[0] + g2w * I1;
 #pragma unroll
                 for (int j = 0; j < DIM; ++j)
 #pragma unroll
                     for (int l = j; l < DIM; ++l) {
-                        double ci = 0.0, mm = 0.0, c = 0.0;
+                        double ci = 0.0, c = 0.0;
+                        const double mm = Mj[j][l];
 #pragma unroll
                         for (int i = 0; i < DIM; ++i) {
                             ci += Fi[j][i] * Fi[l][i];             // C^-1
-                            mm += Ji[j][i] * Ji[l][i];             // the metric (delta_JL)
                             c += Fp[i][j] * Fp[i][l];              // C
                         }
                         Cv[j][l] = Cv[l][j] = cdw * ci;
@@ -843,11 +892,11 @@ __global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
 
         // ================= row mode: element residual and tangent =================
         {
-            constexpr int EPWR = grp::kPts / NQ;                 // elements of a warp: HEX8 1, Q4 2
+            constexpr int EPWR = 8 / NQ;                         // elements of a warp: HEX8 1, Q4 2
             const int ee = lane / G_::ND, row = lane % G_::ND, a = row / NDOF, i = row % NDOF;
             const int el_r = warp * EPWR + ee;
             const int64_t e = e0 + el_r;
-            if (lane < EPWR * G_::ND && e < A.n_elems) {
+            if (warp < NP / 8 && lane < EPWR * G_::ND && e < A.n_elems) {
                 const double *R0 = sRec + el_r * NQ * R_::SIZE;
                 const bool pr = i == DIM;                        // a phi row
                 double Rr = 0.0;
@@ -928,55 +977,50 @@ __global__ void __launch_bounds__(32 * KW, 8 / KW) asm_fp64_kernel(AsmArgs A)
     }
 }
 
-template <int DIM, int KW>
-cudaError_t launch_kw(const AsmArgs &a, int num_sms, const AsmTune &t, cudaStream_t s)
+template <int DIM, int NP, int KW>
+cudaError_t launch_cta(const AsmArgs &a, int num_sms, const AsmTune &t, cudaStream_t s)
 {
-    const size_t sm = (size_t)Smem<DIM, KW>::total(a.wmax) * sizeof(double);
+    using S_ = Smem<DIM, NP, KW>;
+    auto fn = asm_fp64_kernel<DIM, NP, KW>;
+    const size_t sm = (size_t)S_::total(a.wmax) * sizeof(double);
     int dev = 0, optin = 0;
     cudaError_t e0 = cudaGetDevice(&dev);
     if (e0 == cudaSuccess) e0 = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e0 != cudaSuccess) return e0;
     if (sm > (size_t)optin) return cudaErrorInvalidConfiguration;   // this CTA width does not fit
-    cudaError_t err = cudaFuncSetAttribute(asm_fp64_kernel<DIM, KW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
     int per_sm = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, asm_fp64_kernel<DIM, KW>, 32 * KW, sm);
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * KW, sm);
     if (err != cudaSuccess) return err;
     if (per_sm < 1) per_sm = 1;
     if (t.cta_per_sm > 0 && t.cta_per_sm < per_sm) per_sm = t.cta_per_sm;
-    const int64_t need = (a.n_elems + Smem<DIM, KW>::EL - 1) / Smem<DIM, KW>::EL;
+    const int64_t need = (a.n_elems + S_::EL - 1) / S_::EL;
     int64_t grid = (int64_t)num_sms * per_sm;
     if (grid > need) grid = need;
     if (t.grid_max > 0 && grid > t.grid_max) grid = t.grid_max;
     if (grid < 1) grid = 1;
-    asm_fp64_kernel<DIM, KW><<<(unsigned)grid, 32 * KW, sm, s>>>(a);
+    fn<<<(unsigned)grid, 32 * KW, sm, s>>>(a);
     return cudaGetLastError();
 }
 
-// the requested CTA width, or the widest narrower one whose shared memory fits (a
-// width tuned for one kernel may not fit another: the FP64 kernel needs twice the
-// FP32 kernel's scratch)
+// The requested CTA width (gd_autotune's choice of warps, eight points each), or the widest
+// narrower one whose shared memory fits.  Meshes that would leave SMs without a CTA take
+// narrower ones, at the end eight points on two warps (one round of the networks each).
 template <int DIM>
 cudaError_t launch_dim(const AsmArgs &a, int num_sms, const AsmTune &t, cudaStream_t s)
 {
-    if (t.exact) {
-        switch (t.warps) {
-        case 1: return launch_kw<DIM, 1>(a, num_sms, t, s);
-        case 2: return launch_kw<DIM, 2>(a, num_sms, t, s);
-        case 8: return launch_kw<DIM, 8>(a, num_sms, t, s);
-        default: return launch_kw<DIM, 4>(a, num_sms, t, s);
-        }
-    }
-    // small meshes: CTAs of eight or sixteen points until every SM has one (qp mode then
-    // leaves lanes idle, which costs less than idle SMs)
-    int warps = t.warps;
+    int warps = t.warps >= 8 ? 8 : t.warps >= 4 ? 4 : 2;
     const int64_t points = a.n_elems * Geo<DIM>::NQ;
-    while (warps > 1 && (points + 8 * warps - 1) / (8 * warps) < num_sms) warps /= 2;
+    if (!t.exact)
+        while (warps > 1 && (points + 8 * warps - 1) / (8 * warps) < num_sms) warps /= 2;
     cudaError_t e = cudaErrorInvalidConfiguration;
-    if (warps >= 8) e = launch_kw<DIM, 8>(a, num_sms, t, s);
-    if (e == cudaErrorInvalidConfiguration && warps >= 4) e = launch_kw<DIM, 4>(a, num_sms, t, s);
-    if (e == cudaErrorInvalidConfiguration && warps >= 2) e = launch_kw<DIM, 2>(a, num_sms, t, s);
-    if (e == cudaErrorInvalidConfiguration) e = launch_kw<DIM, 1>(a, num_sms, t, s);
+    if (warps == 8) e = launch_cta<DIM, 64, 8>(a, num_sms, t, s);
+    if (warps == 4 || (e == cudaErrorInvalidConfiguration && warps > 4 && !t.exact))
+        e = launch_cta<DIM, 32, 4>(a, num_sms, t, s);
+    if (warps == 2 || (e == cudaErrorInvalidConfiguration && warps > 2 && !t.exact))
+        e = launch_cta<DIM, 16, 2>(a, num_sms, t, s);
+    if (warps == 1) e = launch_cta<DIM, 8, 2>(a, num_sms, t, s);
     return e;
 }
 

@@ -194,6 +194,36 @@ GD_FX int bound_exp(double v)
     return ab == 0 ? 0 : (int)(ab >> 52) - 1022;
 }
 
+// |h| in units of 2^-57, 63 where |h| >= 64
+GD_FX u64 magnitude57(u64 ab)
+{
+    const int sh = (int)(ab >> 52) - 1023 + 5;
+    const u64 m = (ab & 0xfffffffffffffull) | 0x10000000000000ull;
+    if (sh > 10) return 63ull << 57;
+    return sh >= 0 ? m << sh : (sh < -53 ? 0 : m >> -sh);
+}
+// exp(-T 2^-57) = 2^-n e 2^-64; e is returned
+GD_FX u64 exp_parts(u64 T, int &n)
+{
+    const u64 y = mulhi_u(T, 0xB8AA3B295C17F0BCull);               // T log2(e), 56 fraction bits
+    n = (int)(y >> 56);
+    const u64 rr = (y & 0xffffffffffffull) << 8;                   // r, 64 fraction bits
+    const uint32_t rh = (uint32_t)(rr >> 24);                      // r, 40 fraction bits
+    // ln2^3/6, ln2^4/24, ln2^5/120 with 36 fraction bits; ln2^2/2, ln2 with 64
+    const uint32_t q = 3814213304u - (mulhi_u32(rh, 660952799u - (mulhi_u32(rh, 91627514u) >> 8)) >> 8);
+    const u64 a = 4431396893595737425ull - mulhi_u(rr, (u64)q << 28);
+    const u64 b = 12786308645202655660ull - mulhi_u(rr, a);
+    return mulhi_u(tab_e((int)(y >> 48) & 255), ~mulhi_u(rr, b));
+}
+// exp(-t) for 0 <= t
+GD_FX double exp_neg(double t)
+{
+    if (!(t < 60.0)) return exp(-t);
+    int n;
+    const u64 e = exp_parts(magnitude57(bits_of(t)), n);
+    return to_double((i64)(e >> 1), -63 - n);
+}
+
 // softplus(h) in units of 2^-57 (|h| < 64; beyond, softplus is h or 0 to that precision and
 // the caller takes h itself for h >= 64) and sigmoid(h) in units of 2^-62.
 //   e = exp(-|h|) = 2^-n 2^(-i/256) 2^-r, 2^-r by its Taylor series (r < 2^-8, degree 5);
@@ -203,20 +233,9 @@ GD_FX void softplus_sigmoid(double h, i64 &s57, i64 &sg62)
 {
     const u64 hb = bits_of(h), ab = hb & 0x7fffffffffffffffull;
     const bool neg = (hb >> 63) != 0;
-    const int sh = (int)(ab >> 52) - 1023 + 5;
-    const u64 m = (ab & 0xfffffffffffffull) | 0x10000000000000ull;
-    u64 T = sh >= 0 ? m << (sh < 10 ? sh : 10) : (sh < -53 ? 0 : m >> -sh);
-    if (sh > 10) T = 63ull << 57;
-    // exponential
-    const u64 y = mulhi_u(T, 0xB8AA3B295C17F0BCull);               // |h| log2(e), 56 fraction bits
-    const int n = (int)(y >> 56);
-    const u64 rr = (y & 0xffffffffffffull) << 8;                   // r, 64 fraction bits
-    const uint32_t rh = (uint32_t)(rr >> 24);                      // r, 40 fraction bits
-    // ln2^3/6, ln2^4/24, ln2^5/120 with 36 fraction bits; ln2^2/2, ln2 with 64
-    const uint32_t q = 3814213304u - (mulhi_u32(rh, 660952799u - (mulhi_u32(rh, 91627514u) >> 8)) >> 8);
-    const u64 a = 4431396893595737425ull - mulhi_u(rr, (u64)q << 28);
-    const u64 b = 12786308645202655660ull - mulhi_u(rr, a);
-    u64 e = mulhi_u(tab_e((int)(y >> 48) & 255), ~mulhi_u(rr, b));
+    const u64 T = magnitude57(ab);
+    int n;
+    u64 e = exp_parts(T, n);
     e = n > 63 ? 0 : e >> n;                                       // exp(-|h|), 64 fraction bits
     // logarithm
     const int i = (int)(e >> 56);
@@ -256,7 +275,7 @@ GD_FX i64 softplus_operand(double h, i64 s57, int e_p)
 
 // Fixed-point copies of one network (built on the device whenever its weights change).
 // Weight tables are stored [j][wp] with the outputs of a 16-wide chunk permuted so that the
-// lane sub = k mod 4 of a point finds its four outputs k = c0 + 4 i + sub in 32 consecutive
+// lane sub = k mod 8 of a point finds its two outputs k = c0 + 8 i + sub in 16 consecutive
 // bytes.
 struct Net {
     const int2 *W2, *W2T;      // [w][wp] limbs: W2[k][j] at (j, perm k), scaled by 2^(56 - e[k]);
@@ -268,7 +287,7 @@ struct Net {
     const int *e;              // [w] rows of W2, [w] rows of W2^T, then e1, e3
 };
 GD_FX int pad16(int w) { return (w + 15) / 16 * 16; }
-GD_FX int perm16(int k) { return (k & ~15) + (k & 3) * 4 + ((k >> 2) & 3); }
+GD_FX int perm16(int k) { return (k & ~15) + (k & 7) * 2 + ((k >> 3) & 1); }
 GD_FX size_t net_bytes(int w)
 {
     const size_t wp = pad16(w);

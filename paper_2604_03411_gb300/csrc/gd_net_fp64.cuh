@@ -1,10 +1,11 @@
-// gd_net_fp64.cuh -- the ICNNs of the FP64 element kernel, four lanes per quadrature
-// point (eight points of a warp at once): lane sub = lane mod 4 of point pt = lane / 4 owns
-// the units j, k = sub (mod 4) of every layer.  Pre-activations and the sums over the second
+// gd_net_fp64.cuh -- the ICNNs of the FP64 element kernel, eight lanes per quadrature
+// point (four points of a warp at once): lane sub = lane mod 8 of point pt = lane / 8 owns
+// the units j, k = sub (mod 8) of every layer.  (Four lanes per point halve the reductions
+// but double a round's buffers and accumulators: 8 instead of 16 warps per SM.)  Pre-activations and the sums over the second
 // layer's units are FP64; activations and the layer products are 64-bit fixed point
 // (gd_fixed.cuh).  The FP32 evaluations of the local solve use the same mapping.
 // Every function is called by the whole warp; `need` marks the points that take part (all
-// four lanes of a point agree) and net is the same for all of them.
+// lanes of a point agree) and net is the same for all of them.
 #pragma once
 
 #include "gd_elem32.cuh"
@@ -15,47 +16,49 @@ namespace grp {
 
 using fx::i64;
 
-constexpr int kLanes = 4;                  // lanes per point
+constexpr int kLanes = 8;                  // lanes per point
 constexpr int kPts = 32 / kLanes;          // points per round
+constexpr int kOut = 16 / kLanes;          // a lane's outputs of a 16-wide chunk
 
-// shared-memory bytes of a warp's network buffers for width w: operands [w][8][4], one
-// 64-bit word [w][8] per unit, reverse operands [w][8]
+// shared-memory bytes of a warp's network buffers for width w: operands [w][kPts][4], one
+// 64-bit word [w][kPts] per unit, reverse operands [w][kPts]
 __host__ __device__ inline size_t buf_bytes(int w) { return (size_t)w * kPts * (4 + 1 + 1) * 8; }
 
 template <class T>
-__device__ __forceinline__ T sum4(T v)
+__device__ __forceinline__ T sum_lanes(T v)
 {
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
+#pragma unroll
+    for (int o = 1; o < kLanes; o *= 2) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-__device__ __forceinline__ int max4(int v)
+__device__ __forceinline__ int max_lanes(int v)
 {
-    v = max(v, __shfl_xor_sync(0xffffffffu, v, 1));
-    return max(v, __shfl_xor_sync(0xffffffffu, v, 2));
+#pragma unroll
+    for (int o = 1; o < kLanes; o *= 2) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
 }
 __device__ __forceinline__ int hi_word(double v) { return __double2hiint(v); }
 
 // NC column products of a 16-wide output chunk: V[i][c] = sum_j W(k_i, j) z_c(j) in units of
-// 2^-56 (times the operand and row scales), k_i = c0 + 4 i + sub.  Three multiply-adds per
+// 2^-56 (times the operand and row scales), k_i = c0 + 8 i + sub.  Three multiply-adds per
 // term: hi hi into one sum, hi lo + lo hi into the other.  z: operand c of unit j and point pt
-// at z[(j 8 + pt) ZS + c].
+// at z[(j kPts + pt) ZS + c].
 template <int NC, int ZS>
 __device__ __forceinline__ void chunk_product(const int2 *__restrict__ W, int wp, int c0, const int2 *z, int n, int pt,
-                                              int sub, i64 (&V)[4][NC])
+                                              int sub, i64 (&V)[kOut][NC])
 {
-    i64 hh[4][NC], md[4][NC];
+    i64 hh[kOut][NC], md[kOut][NC];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < kOut; ++i)
 #pragma unroll
         for (int c = 0; c < NC; ++c) hh[i][c] = md[i][c] = 0;
-    const int4 *wr = reinterpret_cast<const int4 *>(W + c0 + sub * 4);
+    const int4 *wr = reinterpret_cast<const int4 *>(W + c0 + sub * kOut);
     const int2 *zr = z + pt * ZS;
-#pragma unroll 2
+#pragma unroll 4
     for (int j = 0; j < n; ++j) {
-        const int4 wa = __ldg(wr), wb = __ldg(wr + 1);
+        const int4 wa = __ldg(wr);
         wr += wp / 2;
-        const int wh[4] = {wa.x, wa.z, wb.x, wb.z}, wl[4] = {wa.y, wa.w, wb.y, wb.w};
+        const int wh[kOut] = {wa.x, wa.z}, wl[kOut] = {wa.y, wa.w};
         int zh[NC], zl[NC];
         if (NC == 4) {
             const int4 a = reinterpret_cast<const int4 *>(zr)[0], b = reinterpret_cast<const int4 *>(zr)[1];
@@ -72,7 +75,7 @@ __device__ __forceinline__ void chunk_product(const int2 *__restrict__ W, int wp
         }
         zr += kPts * ZS;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < kOut; ++i)
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 hh[i][c] += (i64)zh[c] * wh[i];
@@ -81,7 +84,7 @@ __device__ __forceinline__ void chunk_product(const int2 *__restrict__ W, int wp
             }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < kOut; ++i)
 #pragma unroll
         for (int c = 0; c < NC; ++c) V[i][c] = hh[i][c] + ((md[i][c] + (1LL << 27)) >> fx::kLimb);
 }
@@ -93,12 +96,12 @@ __device__ __forceinline__ void chunk_product(const int2 *__restrict__ W, int wp
 __device__ __forceinline__ void energy(const DevNet &net, const double *sY, double *sO, unsigned char *buf, int lane,
                                        bool need, bool hess)
 {
-    const int w = net.width, wp = fx::pad16(w), pt = lane >> 2, sub = lane & 3;
+    const int w = net.width, wp = fx::pad16(w), pt = lane / kLanes, sub = lane % kLanes;
     const double *W1 = net.p, *b1 = W1 + 3 * w, *A2 = b1 + w + w * w, *b2 = A2 + 3 * w, *w3 = b2 + w, *a3 = w3 + w;
     const fx::Net fn = fx::net_of(net.fx, w);
-    int2 *z = reinterpret_cast<int2 *>(buf);                    // [w][8][4]
-    i64 *sE = reinterpret_cast<i64 *>(z + w * kPts * 4);        // [w][8]: h1, then sp''(h1)
-    int2 *su = reinterpret_cast<int2 *>(sE + w * kPts);         // [w][8]
+    int2 *z = reinterpret_cast<int2 *>(buf);                    // [w][kPts][4]
+    i64 *sE = reinterpret_cast<i64 *>(z + w * kPts * 4);        // [w][kPts]: h1, then sp''(h1)
+    int2 *su = reinterpret_cast<int2 *>(sE + w * kPts);         // [w][kPts]
     double y0 = sY[pt * 4], y1 = sY[pt * 4 + 1], y2 = sY[pt * 4 + 2];
     const bool bad = !(isfinite(y0) && isfinite(y1) && isfinite(y2));
     if (bad || !need) y0 = y1 = y2 = 0.0;
@@ -110,7 +113,7 @@ __device__ __forceinline__ void energy(const DevNet &net, const double *sY, doub
         sE[j * kPts + pt] = __double_as_longlong(h);
         hm = max(hm, hi_word(h));
     }
-    const int ep = fx::softplus_exp(max4(hm)), ew1 = fn.e[2 * w], ew3 = fn.e[2 * w + 1];
+    const int ep = fx::softplus_exp(max_lanes(hm)), ew1 = fn.e[2 * w], ew3 = fn.e[2 * w + 1];
     for (int j = sub; j < w; j += kLanes) {
         const double h = __longlong_as_double(sE[j * kPts + pt]);
         i64 s, g;
@@ -130,11 +133,11 @@ __device__ __forceinline__ void energy(const DevNet &net, const double *sY, doub
 #pragma unroll
     for (int c = 0; c < 10; ++c) acc[c] = 0.0;
     for (int c0 = 0; c0 < wp; c0 += 16) {
-        i64 V[4][4];
+        i64 V[kOut][4];
         chunk_product<4, 4>(fn.W2, wp, c0, z, w, pt, sub, V);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int k = c0 + 4 * i + sub;
+        for (int i = 0; i < kOut; ++i) {
+            const int k = c0 + kLanes * i + sub;
             if (k < w) {
                 const int er = __ldg(fn.e + k) - fx::kBits;
                 const double q0 = __ldg(A2 + 3 * k), q1 = __ldg(A2 + 3 * k + 1), q2 = __ldg(A2 + 3 * k + 2);
@@ -167,11 +170,11 @@ __device__ __forceinline__ void energy(const DevNet &net, const double *sY, doub
     if (hess) {
         __syncwarp();
         for (int c0 = 0; c0 < wp; c0 += 16) {
-            i64 V[4][1];
+            i64 V[kOut][1];
             chunk_product<1, 1>(fn.W2T, wp, c0, su, w, pt, sub, V);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int j = c0 + 4 * i + sub;
+            for (int i = 0; i < kOut; ++i) {
+                const int j = c0 + kLanes * i + sub;
                 if (j < w) {
                     const double c =
                         fx::to_double(fx::mulhi_s(V[i][0], sE[j * kPts + pt]), __ldg(fn.e + w + j) + ew3 - 54);
@@ -184,7 +187,7 @@ __device__ __forceinline__ void energy(const DevNet &net, const double *sY, doub
     }
 #pragma unroll
     for (int c = 0; c < 10; ++c)
-        if (c < 4 || hess) acc[c] = sum4(acc[c]);
+        if (c < 4 || hess) acc[c] = sum_lanes(acc[c]);
     if (sub == 0 && need) {
         double *o = sO + pt * 10;
         const double nan = __longlong_as_double(0x7ff8000000000000LL);
@@ -208,10 +211,10 @@ static __device__ __noinline__ double2 yield(const double *p, const unsigned cha
                                              unsigned char *buf, int lane, bool need)
 {
     constexpr int NC = SLOPE ? 2 : 1;
-    const int wp = fx::pad16(w), pt = lane >> 2, sub = lane & 3;
+    const int wp = fx::pad16(w), pt = lane / kLanes, sub = lane % kLanes;
     const double *V1 = p, *c1 = V1 + w, *B2 = c1 + w + w * w, *c2 = B2 + w, *v3 = c2 + w, *b3 = v3 + w;
     const fx::Net fn = fx::net_of(fxp, w);
-    int2 *z = reinterpret_cast<int2 *>(buf);                       // [w][8][NC]
+    int2 *z = reinterpret_cast<int2 *>(buf);                       // [w][kPts][NC]
     i64 *sE = reinterpret_cast<i64 *>(z + w * kPts * NC);
     const bool bad = !isfinite(q);
     if (bad || !need) q = 0.0;
@@ -221,7 +224,7 @@ static __device__ __noinline__ double2 yield(const double *p, const unsigned cha
         sE[j * kPts + pt] = __double_as_longlong(h);
         hm = max(hm, hi_word(h));
     }
-    const int ep = fx::softplus_exp(max4(hm)), ew1 = fn.e[2 * w], ew3 = fn.e[2 * w + 1];
+    const int ep = fx::softplus_exp(max_lanes(hm)), ew1 = fn.e[2 * w], ew3 = fn.e[2 * w + 1];
     for (int j = sub; j < w; j += kLanes) {
         const double h = __longlong_as_double(sE[j * kPts + pt]);
         i64 s, g;
@@ -233,11 +236,11 @@ static __device__ __noinline__ double2 yield(const double *p, const unsigned cha
     __syncwarp();
     double n0 = 0.0, n1 = 0.0;
     for (int c0 = 0; c0 < wp; c0 += 16) {
-        i64 V[4][NC];
+        i64 V[kOut][NC];
         chunk_product<NC, NC>(fn.W2, wp, c0, z, w, pt, sub, V);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int k = c0 + 4 * i + sub;
+        for (int i = 0; i < kOut; ++i) {
+            const int k = c0 + kLanes * i + sub;
             if (k < w) {
                 const int er = __ldg(fn.e + k) - fx::kBits;
                 const double b = __ldg(B2 + k);
@@ -252,8 +255,8 @@ static __device__ __noinline__ double2 yield(const double *p, const unsigned cha
         }
     }
     const double b = __ldg(b3), nan = __longlong_as_double(0x7ff8000000000000LL);
-    double2 r = make_double2(sum4(n0) + b * q, 0.0);
-    if (SLOPE) r.y = sum4(n1) + b;
+    double2 r = make_double2(sum_lanes(n0) + b * q, 0.0);
+    if (SLOPE) r.y = sum_lanes(n1) + b;
     if (bad) r = make_double2(nan, nan);
     __syncwarp();
     return r;
@@ -267,7 +270,7 @@ __device__ __forceinline__ void residual(const MatConst &m, const DevNet &yld, c
                                          unsigned char *buf, int lane, bool need)
 {
     const bool dmg = kappa > m.kappa_d;
-    const double f = dmg ? exp(-m.eta_d * (kappa - m.kappa_d)) : 1.0;
+    const double f = dmg ? fx::exp_neg(m.eta_d * (kappa - m.kappa_d)) : 1.0;
     const double q = pe + m.qcoef * (phi - kappa) / f;
     // G(q) = s (N_k(q) - N_k(0)) (Eq. (Gq_NN)); width 0 is the identity G(q) = q
     double G = q, Gs = 1.0;
@@ -283,48 +286,55 @@ __device__ __forceinline__ void residual(const MatConst &m, const DevNet &yld, c
     }
 }
 
+// softplus and sigmoid for the FP32 start of the local solve, whose result FP64 evaluations
+// refine: approximate exponential, logarithm and reciprocal (absolute errors near 1e-7)
+__device__ __forceinline__ void sp_sig_start(float v, float &sp, float &sg)
+{
+    const float e = __expf(-fabsf(v)), t = 1.0f + e, r = __fdividef(1.0f, t);
+    sp = fmaxf(v, 0.0f) + __logf(t);
+    sg = v >= 0.0f ? r : e * r;
+}
+
 // N_k(q) and N_k'(q) in FP32
 static __device__ __noinline__ float2 yield32(const float *p, const unsigned char *fxp, int w, float q,
                                               unsigned char *buf, int lane)
 {
-    const int wp = fx::pad16(w), pt = lane >> 2, sub = lane & 3;
+    const int wp = fx::pad16(w), pt = lane / kLanes, sub = lane % kLanes;
     const float *V1 = p, *c1 = V1 + w, *B2 = c1 + w + w * w, *c2 = B2 + w, *v3 = c2 + w, *b3 = v3 + w;
-    const float4 *W2P = reinterpret_cast<const float4 *>(fx::net_of(fxp, w).W2P);
-    float2 *z = reinterpret_cast<float2 *>(buf);                   // [w][8]
+    const float2 *W2P = reinterpret_cast<const float2 *>(fx::net_of(fxp, w).W2P);
+    float2 *z = reinterpret_cast<float2 *>(buf);                   // [w][kPts]
     for (int j = sub; j < w; j += kLanes) {
         const float a = __ldg(V1 + j);
         float s, g;
-        e32::sp_sig(__ldg(c1 + j) + a * q, s, g);
+        sp_sig_start(__ldg(c1 + j) + a * q, s, g);
         z[j * kPts + pt] = make_float2(s, g * a);
     }
     __syncwarp();
     float n0 = 0.0f, n1 = 0.0f;
     for (int c0 = 0; c0 < wp; c0 += 16) {
-        float h[4] = {0.0f, 0.0f, 0.0f, 0.0f}, t[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        const float4 *wr = W2P + c0 / 4 + sub;
-#pragma unroll 4
+        float h[kOut] = {0.0f, 0.0f}, t[kOut] = {0.0f, 0.0f};
+        const float2 *wr = W2P + c0 / 2 + sub;
+#pragma unroll 8
         for (int j = 0; j < w; ++j) {
-            const float4 a = __ldg(wr + j * (wp / 4));
+            const float2 a = __ldg(wr + j * (wp / 2));
             const float2 v = z[j * kPts + pt];
             h[0] += a.x * v.x; t[0] += a.x * v.y;
             h[1] += a.y * v.x; t[1] += a.y * v.y;
-            h[2] += a.z * v.x; t[2] += a.z * v.y;
-            h[3] += a.w * v.x; t[3] += a.w * v.y;
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int k = c0 + 4 * i + sub;
+        for (int i = 0; i < kOut; ++i) {
+            const int k = c0 + kLanes * i + sub;
             if (k < w) {
                 const float b = __ldg(B2 + k), vk = __ldg(v3 + k);
                 float s, g;
-                e32::sp_sig(h[i] + __ldg(c2 + k) + b * q, s, g);
+                sp_sig_start(h[i] + __ldg(c2 + k) + b * q, s, g);
                 n0 += vk * s;
                 n1 += vk * g * (t[i] + b);
             }
         }
     }
     const float b = __ldg(b3);
-    const float2 r = make_float2(sum4(n0) + b * q, sum4(n1) + b);
+    const float2 r = make_float2(sum_lanes(n0) + b * q, sum_lanes(n1) + b);
     __syncwarp();
     return r;
 }

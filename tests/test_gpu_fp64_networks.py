@@ -6,7 +6,7 @@ are FP64 sums, so max|gpu - oracle| <= 1e-10 max|oracle|."""
 import numpy as np
 import pytest
 
-from gpu_common import compare_assembly, gpu_assemble, oracle_assemble
+from gpu_common import compare_assembly, gpu_assemble, oracle_assemble, smooth_state
 from paper_2604_03411_gb300 import inputs as I
 
 pytestmark = pytest.mark.gpu
@@ -37,10 +37,13 @@ def make(dim, shape, w_psi, w_y, seed=7, scale=None):
     return I.Problem("t", mesh, psi, yld, I.Material(), np.array([0.1]))
 
 
-def check(env, prob, u_amp=0.06, phi_amp=0.3):
+def check(env, prob, u_amp=0.06, phi_amp=0.3, smooth=False):
     torch, B, oracle = env
     rng = np.random.default_rng(3)
-    dofs, kappa = I.random_state(prob.mesh, rng, u_amp=u_amp, phi_amp=phi_amp, kappa_amp=0.3)
+    if smooth:          # nodal noise scaled by the element size: fine meshes stay far from inversion
+        dofs, kappa = smooth_state(prob.mesh, rng, u_amp=u_amp, phi_amp=phi_amp, kappa_amp=0.3)
+    else:
+        dofs, kappa = I.random_state(prob.mesh, rng, u_amp=u_amp, phi_amp=phi_amp, kappa_amp=0.3)
     h = B.gd_create(prob, B.gd_default_options())
     Rg, Kg, kg, lg = gpu_assemble(B, torch, h, dofs, kappa)
     Ro, Ko, ko, qi = oracle_assemble(oracle, prob, dofs, kappa)
@@ -69,9 +72,9 @@ def test_large_pre_activations(env):
 @pytest.mark.parametrize("shape", [(1, 1), (2, 1), (13, 47), (31, 41), (37, 67), (70, 71)])
 def test_cta_widths_q4(env, shape):
     """8, 16 and 32 points per CTA, full and ragged, one and several batches per CTA."""
-    check(env, make(2, shape, 8, 8))
+    check(env, make(2, shape, 8, 8), smooth=True)
 
 
 @pytest.mark.parametrize("shape", [(1, 1, 1), (5, 6, 7), (7, 9, 8), (11, 10, 11)])
 def test_cta_widths_hex8(env, shape):
-    check(env, make(3, shape, 8, 8))
+    check(env, make(3, shape, 8, 8), smooth=True)
