@@ -397,8 +397,9 @@ typedef struct gd_tune_report {
                                     co-resident                                                 */
     int32_t krylov_up;           /* node groups per lane in the Krylov products (1, 2 or 4)     */
     double krylov_us_up[3];      /* iteration time with 1, 2, 4 node groups at the chosen grid  */
-    int32_t krylov_lanes;        /* lanes per node of 3D solves with FP32 vectors (32, 8 or 4)  */
-    double krylov_us_lanes[3];   /* iteration time with 32, 8, 4 lanes per node; -1: not timed */
+    int32_t krylov_lanes;        /* lanes per node of the products of 3D solves (8)             */
+    double krylov_us_lanes[3];   /* iteration time with 32, 8, 4 lanes per node; -1: not timed
+                                    (the mapping is fixed at 8; GD_MIXED 3D solves report it)   */
 } gd_tune_report;
 
 /* Times the element kernel (one tangent pass at the committed state) for each CTA

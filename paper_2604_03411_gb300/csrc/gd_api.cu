@@ -104,6 +104,7 @@ void free_handle(gd::Handle &H)
     for (void *p : ptrs) dfree(p);
     for (double *p : H.kv) dfree(p);
     free_ckpts(H);
+    dfree(H.bcol);
     dfree(H.perm_T);
     dfree(H.vals_T);
     dfree(H.vals64);
@@ -134,7 +135,7 @@ void free_handle(gd::Handle &H)
     dfree(H.gm_binv);
     {
         gd::CoarseSpace &c = H.coarse;
-        void *cp[] = {c.agg, c.coff, c.node_co, c.P, c.Ac, c.X32, c.X64, c.rc, c.cc, c.status};
+        void *cp[] = {c.agg, c.coff, c.node_co, c.P, c.Ac, c.X32, c.rc, c.cc, c.status};
         for (void *p : cp) dfree(p);
     }
     for (gd::DevNet &n : H.h_psi_tab) {
@@ -352,7 +353,7 @@ gd_status krylov(gd::Handle &H, const void *vals, const double *b, double *x, in
     kc.up = H.krylov_up;
     kc.lmax = H.krylov_lmax;
     kc.row_cache = H.opt.krylov_row_cache;
-    kc.lanes = H.krylov_lanes;
+    kc.bcol = H.bcol;
     kc.coarse = H.coarse.nc > 0 ? &H.coarse : nullptr;
     bool refresh =
         kind == kCallerMatrix || H.coarse_age < 0 || H.coarse_kind != kind || H.coarse_age >= kCoarseReuse;
@@ -1748,6 +1749,16 @@ static gd_status create_impl(int32_t n_spec, const gd_mesh *meshes, const gd_icn
         GD_CREATE_CUDA(cudaMemcpy(H.slot, slot.data(), sizeof(int32_t) * slot.size(), cudaMemcpyHostToDevice));
     }
     GD_CREATE_CUDA(cudaMemcpy(H.rowptr, H.h_rowptr.data(), sizeof(int32_t) * H.h_rowptr.size(), cudaMemcpyHostToDevice));
+    if (ndof == 4 && nnz > 0) {
+        // node of every 4 x 4 block, in pattern order
+        std::vector<int32_t> bcol((size_t)(nnz / 16));
+        for (int64_t n = 0; n < NN; ++n) {
+            const int32_t r0 = H.h_rowptr[4 * n], len = H.h_rowptr[4 * n + 1] - r0;
+            for (int32_t j = 0; j < len; j += 4) bcol[(size_t)(r0 / 16 + j / 4)] = H.h_colidx[r0 + j] / 4;
+        }
+        GD_CREATE_CUDA(dalloc(&H.bcol, bcol.size()));
+        GD_CREATE_CUDA(cudaMemcpy(H.bcol, bcol.data(), sizeof(int32_t) * bcol.size(), cudaMemcpyHostToDevice));
+    }
     if (nnz > 0)
         GD_CREATE_CUDA(cudaMemcpy(H.colidx, H.h_colidx.data(), sizeof(int32_t) * nnz, cudaMemcpyHostToDevice));
     GD_CREATE_CUDA(cudaMemcpy(H.fixed, fixed.data(), fixed.size(), cudaMemcpyHostToDevice));
@@ -1876,7 +1887,6 @@ static gd_status create_impl(int32_t n_spec, const gd_mesh *meshes, const gd_icn
             GD_CREATE_CUDA(dalloc(&C.P, Pc.size()));
             GD_CREATE_CUDA(dalloc(&C.Ac, nc * nc));
             GD_CREATE_CUDA(dalloc(&C.X32, nc * nc));
-            GD_CREATE_CUDA(dalloc(&C.X64, nc * nc));
             GD_CREATE_CUDA(dalloc(&C.rc, 2 * nc));
             GD_CREATE_CUDA(dalloc(&C.cc, nc));
             GD_CREATE_CUDA(dalloc(&C.status, 1));
@@ -2178,31 +2188,10 @@ gd_status gd_autotune(gd_handle *h, gd_tune_report *rep)
     }
     H.krylov_up = upick;
     r.krylov_up = upick ? upick : 1;
-    // lanes per node of the 3D FP32 solve (32: a warp per node; 8 or 4: four or
-    // eight nodes per warp, more lanes busy in the vector phases)
-    const int lanes[3] = {32, 8, 4};
-    double lbest = 1e300;
-    int lpick = H.krylov_lanes;
+    // 3D solves have one mapping (eight lanes per node in the products)
     for (double &v : r.krylov_us_lanes) v = -1.0;
-    for (int li = 0; li < 3 && st == GD_OK && H.ndof == 4 && fp32; ++li) {
-        H.krylov_lanes = lanes[li];
-        double tmin = 1e300;
-        for (int rep_i = 0; rep_i < 2; ++rep_i) {
-            int kit = 0;
-            double rel = 0.0;
-            const double k0 = H.krylov_ms;
-            st = krylov(H, H.vals, H.kv[9], H.kv[8], kit, rel, 1e-300, fp32, 1e300);
-            if (st) break;
-            if (rep_i > 0 && kit > 0) tmin = std::min(tmin, (H.krylov_ms - k0) * 1e3 / kit);
-        }
-        r.krylov_us_lanes[li] = st ? -1.0 : tmin;
-        if (!st && tmin < lbest) {
-            lbest = tmin;
-            lpick = lanes[li];
-        }
-    }
-    H.krylov_lanes = lpick;
-    r.krylov_lanes = lpick ? lpick : 32;
+    r.krylov_lanes = 8;
+    if (st == GD_OK && H.ndof == 4 && fp32) r.krylov_us_lanes[1] = ubest;
     std::swap(H.vals, H.vals_trial);
     H.opt.krylov_max = keep_max;
     if (st) return st;

@@ -372,8 +372,7 @@ constexpr int kGjThreads = 512;  // threads per CTA; C columns per thread (nc <=
 // so each panel value read from shared memory serves kGjRows rows).  That is the
 // unblocked in-place elimination reordered by panels, one grid barrier per panel.
 template <int C>
-__global__ void __launch_bounds__(kGjThreads) coarse_invert_kernel(const double *Ac, float *X, double *X64, int nc,
-                                                                   int *status)
+__global__ void __launch_bounds__(kGjThreads) coarse_invert_kernel(const double *Ac, float *X, int nc, int *status)
 {
     cg::grid_group grid = cg::this_grid();
     extern __shared__ __align__(16) float gsh[];
@@ -475,10 +474,6 @@ __global__ void __launch_bounds__(kGjThreads) coarse_invert_kernel(const double 
         }
     }
     if (bad) atomicOr(status, 1);
-    if (X64) {
-        grid.sync();
-        for (int64_t k = gtid; k < n2; k += nt) X64[k] = (double)X[k];
-    }
 }
 
 }  // namespace
@@ -508,7 +503,7 @@ cudaError_t launch_coarse_asm_smem(const CoarseSpace &cs, int64_t n_nodes, const
 }
 
 cudaError_t coarse_setup(const CoarseSpace &cs, int ndof, int64_t n_nodes, const int32_t *rowptr,
-                         const int32_t *colidx, const void *vals, bool fp32_vals, bool want_x64, int num_sms,
+                         const int32_t *colidx, const void *vals, bool fp32_vals, int num_sms,
                          cudaStream_t s, int lmax)
 {
     const int nc = cs.nc;
@@ -555,10 +550,9 @@ cudaError_t coarse_setup(const CoarseSpace &cs, int ndof, int64_t n_nodes, const
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const double *Ac = cs.Ac;
     float *X = cs.X32;
-    double *X64 = want_x64 ? cs.X64 : nullptr;
     int ncv = nc;
     int *st = cs.status;
-    void *args[] = {(void *)&Ac, (void *)&X, (void *)&X64, (void *)&ncv, (void *)&st};
+    void *args[] = {(void *)&Ac, (void *)&X, (void *)&ncv, (void *)&st};
     return cudaLaunchCooperativeKernel(fn, dim3(num_sms), dim3(kGjThreads), args, smem, s);
 }
 

@@ -173,7 +173,6 @@ struct CoarseSpace {
     float *P = nullptr;           // [n_nodes][ndof][nm] basis values (zero beyond the kept columns)
     double *Ac = nullptr;         // [nc][nc] Galerkin matrix
     float *X32 = nullptr;         // [nc][nc] its inverse
-    double *X64 = nullptr;        // [nc][nc] the same values in FP64
     double *rc = nullptr;         // [2][nc] restriction sums (FP32 solves use them as float storage)
     double *cc = nullptr;         // [nc] coarse solution (likewise)
     int *status = nullptr;        // device: 0 when X holds the inverse
@@ -265,7 +264,7 @@ struct Handle {
     std::vector<double> noise_ratio;
     int noise_age = 0;
     int krylov_up = 0;                                   // 0: the precision's default
-    int krylov_lanes = 0;                                // 3D FP32 solves: lanes per node (0: 32)
+    int32_t *bcol = nullptr;                             // node of every 4 x 4 block (3D), in pattern order
     double *gm_ws = nullptr;                             // GMRES work space (allocated on first use)
     double *gm_binv = nullptr;                           // its node-block inverses (FP64)
     long long gmres_iterations = 0;                      // GMRES iterations run by this handle
@@ -392,10 +391,10 @@ int32_t coarse_aggregate(int64_t n_nodes, int ndof, const std::vector<int32_t> &
 // the displacement; zero on prescribed dofs); P [n_nodes][ndof][nm], coff [n_agg + 1]
 void coarse_basis(int dim, int64_t n_nodes, const double *coords, const uint8_t *fixed,
                   const std::vector<int32_t> &agg, int32_t n_agg, std::vector<float> &P, std::vector<int32_t> &coff);
-// Ac = P^T A P for the tangent values vals, X32 = Ac^-1 (and X64 when want_x64)
+// Ac = P^T A P for the tangent values vals, X32 = Ac^-1
 // lmax: the longest row (columns); rows up to 256 columns take the shared-memory kernel
 cudaError_t coarse_setup(const CoarseSpace &cs, int ndof, int64_t n_nodes, const int32_t *rowptr,
-                         const int32_t *colidx, const void *vals, bool fp32_vals, bool want_x64, int num_sms,
+                         const int32_t *colidx, const void *vals, bool fp32_vals, int num_sms,
                          cudaStream_t s, int lmax = 0);
 
 // persistent cooperative Krylov solve (gd_krylov.cu)
@@ -417,7 +416,7 @@ struct KrylovCtx {
     const CoarseSpace *coarse = nullptr;   // two-level preconditioner (single systems; null: Jacobi only)
     bool coarse_refresh = true;            // recompute P^T A P and its inverse before the solve
     int row_cache = 0;                     // gd_options.krylov_row_cache: 0 automatic, 1 column lists only, 2 none
-    int lanes = 0;                         // lanes per node of the 3D FP32-vector solve: 4, 8 or 32 (0: 32)
+    const int32_t *bcol = nullptr;         // node of every node block of the pattern (4 dofs per node; may be null)
 };
 cudaError_t krylov_solve_batch(const KrylovCtx &c, const BatchKrylov &L, const void *vals, bool fp32_vals,
                                const double *b, double *x, int max_it, bool fp32_vectors);

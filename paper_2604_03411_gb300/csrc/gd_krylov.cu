@@ -31,6 +31,7 @@ template <class V, class T>
 struct KArgs {
     int64_t n_nodes;
     const int32_t *rowptr, *colidx;
+    const int32_t *bcol;      // node of every NDOF x NDOF block (4 dofs per node; null: scalar columns)
     const V *vals;
     const uint8_t *fixed;
     const T *binv;            // [n_nodes][NDOF][NDOF] inverse diagonal node blocks
@@ -47,14 +48,12 @@ struct KArgs {
     int cache;
     int lmax;
     // coarse level (single-system kernel with CO): P [n_nodes][NDOF][nm], the coarse
-    // unknowns of every node's aggregate, the inverse coarse matrix
-    // (FP32 for FP32 vectors, FP64 otherwise), restriction sums [2][nc] and coarse
-    // solution [nc] in the vector type, status word of the inversion
+    // unknowns of every node's aggregate, the inverse coarse matrix (FP32), restriction
+    // sums [2][nc] and coarse solution [nc] in the vector type, status word of the inversion
     int c_nc;
     const float *c_P;
     const int32_t *c_node;    // 8 x first coarse unknown + count, per node
     const float *c_X32;
-    const double *c_X64;
     T *c_rc, *c_cc;
     const int *c_status;
     int c_xs;                 // 1: each CTA keeps its rows of the inverse in shared memory
@@ -65,13 +64,20 @@ struct CoarseModes {
     static constexpr int NM = NDOF == 3 ? 4 : 7;     // ndof constants + rigid rotations (2D: 1, 3D: 3)
 };
 
-template <class T>
-__device__ __forceinline__ T warp_sum_t(T v)
+// An FP32 value in the vector type.  To FP64 by integer operations: the conversion
+// instruction issues at half a lane per clock and SM on this part (measured), a hundredth
+// of the integer rate.  Infinities and NaN keep their exponent; subnormal values (below
+// 1.2e-38) become 0 to FP64 precision.  No branch: one per value would keep the compiler
+// from interleaving the products.
+__device__ __forceinline__ float widen(float v, float) { return v; }
+__device__ __forceinline__ double widen(float v, double)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+    const uint32_t u = __float_as_uint(v), a = u & 0x7fffffffu;
+    uint32_t hi = (a >> 3) + (a >= 0x7f800000u ? 0x70000000u : 0x38000000u);
+    hi = a < 0x00800000u ? 0u : hi;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
 }
+__device__ __forceinline__ double widen(double v, double) { return v; }
 
 // restriction P^T w of the node whose NDOF values sit in lanes base..base+NDOF-1:
 // the node's lanes split its nm coarse components and add them to rc (atomics).
@@ -90,7 +96,7 @@ __device__ __forceinline__ void coarse_restrict(bool node_ok, int sub, int base,
     for (int m = sub; m < n; m += LPN) {
         T sum = T(0);
 #pragma unroll
-        for (int k = 0; k < NDOF; ++k) sum += (T)pP[k * NM + m] * wk[k];
+        for (int k = 0; k < NDOF; ++k) sum += widen(pP[k * NM + m], T()) * wk[k];
         atomicAdd(rc + o + m, sum);
     }
 }
@@ -98,18 +104,20 @@ __device__ __forceinline__ void coarse_restrict(bool node_ok, int sub, int base,
 // cc = Ac^-1 rc: the coarse rows go to the CTAs in turn (rows b, b + grid, ...),
 // up to eight rows of a CTA at once, its threads along the rows.  Each thread
 // first loads all of its rc values (independent loads in flight together) and
-// reuses them for every row.  sX: the CTA's rows in shared memory (row q of the
-// CTA at sX + q nc), or null to read them from the global inverse.
+// reuses them for every row (1,528 unknowns, FP64: 14 -> 6.7 us per application with FP32
+// rows in shared memory and the joint reduction below).  sX: the CTA's rows in shared memory (row q of the
+// CTA at sX + q nc), or null to read them from the global inverse (FP32 for both vector
+// types: FP64 solves widen its values).  The eight sums are reduced together: each
+// exchange halves the rows a lane holds, 9 additions per lane instead of 40 (in FP64
+// these cost as much as the products).
 template <class V, class T>
-__device__ __forceinline__ void coarse_solve(const KArgs<V, T> &A, const T *rc, T *cc, const T *sX)
+__device__ __forceinline__ void coarse_solve(const KArgs<V, T> &A, const T *rc, T *cc, const float *sX)
 {
     constexpr int JMAX = (kCoarseMax + kThreads - 1) / kThreads;
+    constexpr unsigned kAll = 0xffffffffu;
     __shared__ T part[8][kThreads / 32];
     const int32_t nc = A.c_nc, nb = gridDim.x, b = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
-    const T *Xg;
-    if constexpr (std::is_same<T, double>::value) Xg = A.c_X64;
-    else Xg = A.c_X32;
     T rv[JMAX];
 #pragma unroll
     for (int jj = 0; jj < JMAX; ++jj) {
@@ -127,24 +135,30 @@ __device__ __forceinline__ void coarse_solve(const KArgs<V, T> &A, const T *rc, 
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const int32_t k = b + (q0 + q) * nb;
-                    if (k < nc) acc[q] += (sX ? sX[(q0 + q) * nc + j] : Xg[(int64_t)k * nc + j]) * rv[jj];
+                    if (k < nc)
+                        acc[q] += widen(sX ? sX[(q0 + q) * nc + j] : A.c_X32[(int64_t)k * nc + j], T()) * rv[jj];
                 }
             }
         }
+        const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+        T a4[4], a2[2];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const T s = warp_sum_t(acc[q]);
-            if (lane == 0) part[q][wib] = s;
-        }
+        for (int q = 0; q < 4; ++q)
+            a4[q] = (h4 ? acc[4 + q] : acc[q]) + __shfl_xor_sync(kAll, h4 ? acc[q] : acc[4 + q], 16);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) a2[q] = (h3 ? a4[2 + q] : a4[q]) + __shfl_xor_sync(kAll, h3 ? a4[q] : a4[2 + q], 8);
+        T v = (h2 ? a2[1] : a2[0]) + __shfl_xor_sync(kAll, h2 ? a2[0] : a2[1], 4);
+        v += __shfl_xor_sync(kAll, v, 2);
+        v += __shfl_xor_sync(kAll, v, 1);
+        if ((lane & 3) == 0) part[lane >> 2][wib] = v;
         __syncthreads();
-        if (tid < 8) {
-            const int32_t k = b + (q0 + tid) * nb;
-            if (k < nc) {
-                T s = T(0);
-#pragma unroll
-                for (int w = 0; w < kThreads / 32; ++w) s += part[tid][w];
-                cc[k] = s;
-            }
+        if (tid < 64) {
+            T s = part[tid >> 3][tid & 7];
+            s += __shfl_xor_sync(kAll, s, 4);
+            s += __shfl_xor_sync(kAll, s, 2);
+            s += __shfl_xor_sync(kAll, s, 1);
+            const int32_t k = b + (q0 + (tid >> 3)) * nb;
+            if ((tid & 7) == 0 && k < nc) cc[k] = s;
         }
         __syncthreads();
     }
@@ -159,7 +173,7 @@ __device__ __forceinline__ T coarse_prolong(int sub, const T *cc, int32_t co, co
     T s = T(0);
 #pragma unroll
     for (int m = 0; m < NM; ++m)
-        if (m < n) s += (T)pP[sub * NM + m] * cc[o + m];
+        if (m < n) s += widen(pP[sub * NM + m], T()) * cc[o + m];
     return s;
 }
 
@@ -181,24 +195,30 @@ __device__ __forceinline__ double warp_sum(double v)
 // one when it reads the current one, which is safe because every block read the
 // other one two barriers earlier and the next adds into it come two barriers
 // later.  acc[2 slot + parity]; the launcher clears all of them before the launch.
+static_assert(kThreads == 256, "eight warps per CTA");
 template <int K>
 __device__ __forceinline__ void acc_add(double (&v)[K], double *acc, const int (&slot)[K], int par)
 {
-    __shared__ double sh[K][kThreads / 32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        double s = warp_sum(v[k]);
-        if (lane == 0) sh[k][w] = s;
+    // K = 2: each half of a warp reduces one of the sums
+    __shared__ double sh[2][kThreads / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, hf = lane >> 4;
+    constexpr unsigned kAll = 0xffffffffu;
+    double s = v[0];
+    if (K == 2) {
+        const double t = hf ? v[0] : v[K - 1];
+        s = (hf ? v[K - 1] : v[0]) + __shfl_xor_sync(kAll, t, 16);
+    } else {
+        s += __shfl_xor_sync(kAll, s, 16);
     }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(kAll, s, o);
+    if ((lane & 15) == 0) sh[hf][w] = s;
     __syncthreads();
     if (threadIdx.x < 32) {
+        s = sh[hf][lane & 7];
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            double s = lane < kThreads / 32 ? sh[k][lane] : 0.0;
-            s = warp_sum(s);
-            if (lane == 0) atomicAdd(acc + 2 * slot[k] + par, s);
-        }
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(kAll, s, o);
+        if ((lane & 15) == 0 && hf < K) atomicAdd(acc + 2 * slot[hf < K ? hf : 0] + par, s);
     }
     __syncthreads();
 }
@@ -314,7 +334,7 @@ __device__ __forceinline__ void row_products(const KArgs<V, T> &A, const int32_t
                 if (j < len[u]) {
                     const int32_t col = cs[u] ? cs[u][1 + j] : A.colidx[base[u] + j];
                     const V a = cv[u] ? cv[u][sub * A.lmax + j] : A.vals[base[u] + sub * len[u] + j];
-                    out[u] += (T)a * x[col];
+                    out[u] += widen(a, T()) * x[col];
                 }
         }
     } else {
@@ -347,6 +367,101 @@ __device__ __forceinline__ void row_products(const KArgs<V, T> &A, const int32_t
             out[u] = v;
         }
     }
+}
+
+// Row products of a warp's eight consecutive nodes n0 .. n0 + 7 for matrices of 4 x 4 node
+// blocks (rowptr, bcol: the node of every block): eight lanes per node take its blocks in
+// turn, one vector load per block row and one for the block's four x values, so that a row
+// of values is read in consecutive 128-byte (FP64: 256-byte) pieces.  Bound by the FP64
+// pipe with FP64 vectors (48^3 HEX8 cube: 100 us per product at its rate, 190 measured; 315
+// with one lane per row), by memory with FP32 vectors (75 us per product on that cube, 165
+// with a scalar column per lane; the values at the copy rate take 30).  The eight partial sums of the four rows are reduced together; lane
+// 4 n + r returns row r of node n0 + n, the mapping of the vector phases.
+template <class T>
+struct Vec4 {
+    T x, y, z, w;
+};
+__device__ __forceinline__ Vec4<float> ld4(const float *p, bool ro)
+{
+    const float4 v = ro ? __ldg(reinterpret_cast<const float4 *>(p)) : *reinterpret_cast<const float4 *>(p);
+    return {v.x, v.y, v.z, v.w};
+}
+__device__ __forceinline__ Vec4<double> ld4(const double *p, bool ro)
+{
+    const double2 *q = reinterpret_cast<const double2 *>(p);
+    const double2 a = ro ? __ldg(q) : q[0], b = ro ? __ldg(q + 1) : q[1];
+    return {a.x, a.y, b.x, b.y};
+}
+template <class V, class T>
+__device__ __forceinline__ T block_products(const KArgs<V, T> &A, int32_t n0, const T *x)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, k = lane >> 3, s = lane & 7;
+    int32_t base[2], len[2];
+#pragma unroll
+    for (int hp = 0; hp < 2; ++hp) {
+        const int32_t nd = n0 + hp * 4 + k;
+        const bool ok = nd < (int32_t)A.n_nodes;
+        base[hp] = ok ? __ldg(A.rowptr + 4 * (int64_t)nd) : 0;
+        len[hp] = ok ? __ldg(A.rowptr + 4 * (int64_t)nd + 1) - base[hp] : 0;
+    }
+    T res[2];
+#pragma unroll
+    for (int hp = 0; hp < 2; ++hp) {
+        const int32_t nblk = len[hp] >> 2, *bc = A.bcol + (base[hp] >> 4);
+        const V *va = A.vals + base[hp];
+        T acc[4] = {T(0), T(0), T(0), T(0)};
+        auto load = [&](int32_t b, Vec4<V> (&v)[4], Vec4<T> &xv) {
+            xv = ld4(x + 4 * (int64_t)__ldg(bc + b), false);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = ld4(va + i * len[hp] + 4 * b, true);
+        };
+        auto add = [&](const Vec4<V> (&v)[4], const Vec4<T> &xv) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] += widen(v[i].x, T()) * xv.x;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] += widen(v[i].y, T()) * xv.y;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] += widen(v[i].z, T()) * xv.z;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] += widen(v[i].w, T()) * xv.w;
+        };
+        if constexpr (std::is_same<V, T>::value) {
+#pragma unroll 2
+            for (int32_t b = s; b < nblk; b += 8) {
+                Vec4<V> v[4];
+                Vec4<T> xv;
+                load(b, v, xv);
+                add(v, xv);
+            }
+        } else {
+            // FP32 values, FP64 vectors: the next block's loads ahead of the current block's
+            // conversions and products (890 -> 590 -> 500 us per iteration on the 48^3 cube
+            // with the integer conversion and this; the other types would spill)
+            Vec4<V> v[4];
+            Vec4<T> xv;
+            if (s < nblk) load(s, v, xv);
+            for (int32_t b = s; b < nblk;) {
+                const Vec4<T> xc = xv;
+                Vec4<V> vc[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) vc[i] = v[i];
+                b += 8;
+                if (b < nblk) load(b, v, xv);
+                add(vc, xc);
+            }
+        }
+        // lane 8 k + s ends with row 2 (s / 4) + (s / 2) mod 2 of its node
+        const bool h2 = lane & 4, h1 = lane & 2;
+        T a2[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) a2[i] = (h2 ? acc[2 + i] : acc[i]) + __shfl_xor_sync(kAll, h2 ? acc[i] : acc[2 + i], 4);
+        T r = (h1 ? a2[1] : a2[0]) + __shfl_xor_sync(kAll, h1 ? a2[0] : a2[1], 2);
+        res[hp] = r + __shfl_xor_sync(kAll, r, 1);
+    }
+    const int src = 8 * ((lane >> 2) & 3) + 2 * (lane & 3);
+    const T r0 = __shfl_sync(kAll, res[0], src), r1 = __shfl_sync(kAll, res[1], src);
+    return lane & 16 ? r1 : r0;
 }
 
 // row sub of M^-1 w for the node whose NDOF row values sit in lanes base..base+NDOF-1
@@ -399,6 +514,7 @@ __global__ void __launch_bounds__(kThreads, std::is_same<T, float>::value ? 4 : 
     // slot): [row length, column indices ...] with stride lmax + 1, then the values,
     // NDOF x lmax per record; the launcher sizes the dynamic shared memory for
     // passes x warps x NPW records
+    const bool blocks = NDOF == 4 && A.bcol != nullptr;
     extern __shared__ __align__(16) unsigned char kdyn[];
     const int wib = threadIdx.x >> 5;
     const int32_t n_rec = passes * (kThreads / 32) * NPW;
@@ -418,24 +534,34 @@ __global__ void __launch_bounds__(kThreads, std::is_same<T, float>::value ? 4 : 
         sP = reinterpret_cast<float *>(kdyn + off + (((size_t)n_rec * sizeof(int32_t) + 15) & ~(size_t)15));
     }
     // the CTA's rows of the coarse inverse (CO with c_xs): after the coarse records
-    T *sX = nullptr;
+    float *sX = nullptr;
     if constexpr (CO) {
         if (co && A.c_xs) {
-            size_t off = (((size_t)n_rec * (A.lmax + 1) * sizeof(int32_t)) + 15) & ~(size_t)15;
-            if (A.cache == 2) off += ((size_t)n_rec * NDOF * A.lmax * sizeof(V) + 15) & ~(size_t)15;
-            off += (((size_t)n_rec * sizeof(int32_t) + 15) & ~(size_t)15) +
-                   (((size_t)n_rec * NDOF * NM * sizeof(float) + 15) & ~(size_t)15);
-            sX = reinterpret_cast<T *>(kdyn + off);
-            const T *Xg;
-            if constexpr (std::is_same<T, double>::value) Xg = A.c_X64;
-            else Xg = A.c_X32;
+            size_t off = 0;
+            if (A.cache > 0) {
+                off = (((size_t)n_rec * (A.lmax + 1) * sizeof(int32_t)) + 15) & ~(size_t)15;
+                if (A.cache == 2) off += ((size_t)n_rec * NDOF * A.lmax * sizeof(V) + 15) & ~(size_t)15;
+                off += (((size_t)n_rec * sizeof(int32_t) + 15) & ~(size_t)15) +
+                       (((size_t)n_rec * NDOF * NM * sizeof(float) + 15) & ~(size_t)15);
+            }
+            sX = reinterpret_cast<float *>(kdyn + off);
             const int32_t nc = A.c_nc;
             for (int32_t q = 0; blockIdx.x + q * gridDim.x < nc; ++q)
                 for (int32_t j = threadIdx.x; j < nc; j += kThreads)
-                    sX[(size_t)q * nc + j] = Xg[(int64_t)(blockIdx.x + q * gridDim.x) * nc + j];
+                    sX[(size_t)q * nc + j] = A.c_X32[(int64_t)(blockIdx.x + q * gridDim.x) * nc + j];
             __syncthreads();
         }
     }
+    auto products = [&](int32_t ps0, const int32_t (&ndu)[UP], const bool (&oku)[UP], const T *xv, T (&au)[UP],
+                        const int32_t *const (&csu)[UP], const V *const (&cvu)[UP]) {
+        if constexpr (NDOF == 4 && UP == 1) {
+            if (blocks) {
+                au[0] = block_products<V, T>(A, (gw + ps0 * nw) * NPW, xv);
+                return;
+            }
+        }
+        row_products<NDOF, LPN, UP, V, T>(A, ndu, oku, sub, xv, au, csu, cvu);
+    };
     // a node's coarse data (node_ok lanes only)
     auto cnode = [&](int32_t ps, int32_t nd, int32_t &c, const float *&pp) {
         if (cco) {
@@ -552,7 +678,7 @@ __global__ void __launch_bounds__(kThreads, std::is_same<T, float>::value ? 4 : 
             const V *cvu[UP];
 #pragma unroll
             for (int k = 0; k < UP; ++k) cvu[k] = A.cache == 2 ? sval + (size_t)rec_of(ps0 + k) * NDOF * A.lmax : nullptr;
-            row_products<NDOF, LPN, UP, V, T>(A, ndu, oku, sub, wv, au, csu, cvu);
+            products(ps0, ndu, oku, wv, au, csu, cvu);
 #pragma unroll
             for (int k = 0; k < UP; ++k)
                 if (oku[k] && sub < NDOF) {
@@ -615,7 +741,7 @@ __global__ void __launch_bounds__(kThreads, std::is_same<T, float>::value ? 4 : 
             const V *cvu[UP];
 #pragma unroll
             for (int k = 0; k < UP; ++k) cvu[k] = A.cache == 2 ? sval + (size_t)rec_of(ps0 + k) * NDOF * A.lmax : nullptr;
-            row_products<NDOF, LPN, UP, V, T>(A, ndu, oku, sub, y, au, csu, cvu);
+            products(ps0, ndu, oku, y, au, csu, cvu);
 #pragma unroll
                     for (int k = 0; k < UP; ++k)
                         if (oku[k] && sub < NDOF) {
@@ -717,7 +843,7 @@ __global__ void __launch_bounds__(kThreads, std::is_same<T, float>::value ? 4 : 
             const V *cvu[UP];
 #pragma unroll
             for (int k = 0; k < UP; ++k) cvu[k] = A.cache == 2 ? sval + (size_t)rec_of(ps0 + k) * NDOF * A.lmax : nullptr;
-            row_products<NDOF, LPN, UP, V, T>(A, ndu, oku, sub, wv, au, csu, cvu);
+            products(ps0, ndu, oku, wv, au, csu, cvu);
 #pragma unroll
                 for (int k = 0; k < UP; ++k)
                     if (oku[k] && sub < NDOF) {
@@ -1277,8 +1403,8 @@ __global__ void block_inverse_kernel(int64_t n_nodes, const int32_t *rowptr, con
     }
 }
 
-// G: lanes per node of the FP32-vector kernels (FP64 vectors use one lane per row)
-template <int NDOF, class V, class T, int G = (NDOF == 3 ? 8 : 32)>
+// G: lanes per node of the FP32-vector kernels in 2D (otherwise one lane per row)
+template <int NDOF, class V, class T, int G = (NDOF == 3 ? 8 : 4)>
 cudaError_t solve_t(const KrylovCtx &c, const V *vals, const double *b, double *x, double rtol, int max_it)
 {
     T *binv = (T *)c.binv;
@@ -1290,6 +1416,9 @@ cudaError_t solve_t(const KrylovCtx &c, const V *vals, const double *b, double *
     A.n_nodes = c.n_nodes;
     A.rowptr = c.rowptr;
     A.colidx = c.colidx;
+    // vector loads of the values and of the vectors that the products read
+    const bool aligned = ((uintptr_t)vals | (uintptr_t)c.work[6] | (uintptr_t)c.work[8]) % 16 == 0;
+    A.bcol = NDOF == 4 && aligned ? c.bcol : nullptr;
     A.vals = vals;
     A.fixed = c.fixed;
     A.binv = binv;
@@ -1318,14 +1447,13 @@ cudaError_t solve_t(const KrylovCtx &c, const V *vals, const double *b, double *
     A.c_P = nullptr;
     A.c_node = nullptr;
     A.c_X32 = nullptr;
-    A.c_X64 = nullptr;
     A.c_rc = A.c_cc = nullptr;
     A.c_status = nullptr;
     const bool co = c.coarse && c.coarse->nc > 0;
     if (co) {
         const CoarseSpace &cs = *c.coarse;
         if (c.coarse_refresh) {
-            e = coarse_setup(cs, NDOF, c.n_nodes, c.rowptr, c.colidx, vals, std::is_same<V, float>::value, true,
+            e = coarse_setup(cs, NDOF, c.n_nodes, c.rowptr, c.colidx, vals, std::is_same<V, float>::value,
                              c.num_sms, c.stream, c.lmax);
             if (e != cudaSuccess) return e;
         }
@@ -1335,7 +1463,6 @@ cudaError_t solve_t(const KrylovCtx &c, const V *vals, const double *b, double *
         A.c_P = cs.P;
         A.c_node = cs.node_co;
         A.c_X32 = cs.X32;
-        A.c_X64 = cs.X64;
         A.c_rc = (T *)cs.rc;
         A.c_cc = (T *)cs.cc;
         A.c_status = cs.status;
@@ -1344,21 +1471,40 @@ cudaError_t solve_t(const KrylovCtx &c, const V *vals, const double *b, double *
     e = cudaMemsetAsync(c.red, 0, 10 * sizeof(double), c.stream);
     if (e != cudaSuccess) return e;
     void *args[] = {&A};
-    const int up = c.up ? c.up : 1;
-    // the two-level variant takes one or two node groups per lane and product round
-    const void *fn = co        ? (up == 2 ? (const void *)bicgstab3_kernel<NDOF, G, 2, V, T, true>
-                                          : (const void *)bicgstab3_kernel<NDOF, G, 1, V, T, true>)
-                     : up == 1 ? (const void *)bicgstab3_kernel<NDOF, G, 1, V, T>
-                     : up == 4 ? (const void *)bicgstab3_kernel<NDOF, G, 4, V, T>
-                               : (const void *)bicgstab3_kernel<NDOF, G, 2, V, T>;
-    // Shared-memory copy of each block's rows: column lists and, when they fit,
-    // values, for as long as the grid stays co-resident with that shared memory.
+    // node groups per lane and product round: 4 x 4 blocks take one (each group keeps 8 block
+    // rows in flight), the two-level variant one or two
+    const int up = NDOF == 4 || !c.up ? 1 : c.up;
+    const void *fn = nullptr;
+    if constexpr (NDOF == 4)
+        fn = co ? (const void *)bicgstab3_kernel<NDOF, G, 1, V, T, true> : (const void *)bicgstab3_kernel<NDOF, G, 1, V, T>;
+    else
+        fn = co        ? (up == 2 ? (const void *)bicgstab3_kernel<NDOF, G, 2, V, T, true>
+                                  : (const void *)bicgstab3_kernel<NDOF, G, 1, V, T, true>)
+             : up == 1 ? (const void *)bicgstab3_kernel<NDOF, G, 1, V, T>
+             : up == 4 ? (const void *)bicgstab3_kernel<NDOF, G, 4, V, T>
+                       : (const void *)bicgstab3_kernel<NDOF, G, 2, V, T>;
+    using M = RowMap<NDOF, G, T>;
+    // Small systems take fewer CTAs than the co-resident grid: one per four node groups (one
+    // warp per SM quarter), or per eight coarse rows (one round of the coarse solve).  A
+    // 243-dof system with 87 coarse unknowns on 304 CTAs spent 60 us per iteration on
+    // barriers among CTAs without rows.
+    int blocks = c.blocks;
+    {
+        const int64_t groups = (c.n_nodes + M::NPW - 1) / M::NPW;
+        int64_t want = (groups + 3) / 4;
+        if (co && (c.coarse->nc + 7) / 8 > want) want = (c.coarse->nc + 7) / 8;
+        if (want < 1) want = 1;
+        if (want < blocks) blocks = (int)want;
+    }
+    // Shared-memory copy of each block's rows (3 dofs per node): column lists and, when they
+    // fit, values, for as long as the grid stays co-resident with that shared memory.
     // The products then wait on the gathered x alone instead of the chain
-    // row pointer -> column index -> x.
+    // row pointer -> column index -> x.  4 x 4 blocks read theirs in vector loads, for which
+    // the L1 cache serves as well.  Beside them, where it fits, each CTA's rows of the coarse
+    // inverse.
     size_t smem = 0;
-    if (c.lmax > 0 && c.row_cache < 2) {
-        using M = RowMap<NDOF, G, T>;
-        const int64_t nw = (int64_t)c.blocks * (kThreads / 32);
+    {
+        const int64_t nw = (int64_t)blocks * (kThreads / 32);
         const int64_t passes = (c.n_nodes + nw * M::NPW - 1) / (nw * M::NPW);
         const int64_t n_rec = passes * (kThreads / 32) * M::NPW;
         const size_t colb = ((size_t)n_rec * (c.lmax + 1) * sizeof(int32_t) + 15) & ~(size_t)15;
@@ -1367,19 +1513,16 @@ cudaError_t solve_t(const KrylovCtx &c, const V *vals, const double *b, double *
         const size_t cob = co ? (((size_t)n_rec * sizeof(int32_t) + 15) & ~(size_t)15) +
                                     (((size_t)n_rec * NDOF * CoarseModes<NDOF>::NM * sizeof(float) + 15) & ~(size_t)15)
                               : 0;
-        // and, for FP32 vectors where it fits, each CTA's rows of the coarse inverse (with
-        // FP64 rows the shared memory they take from the L1 cache slows the products more
-        // than it speeds the coarse solve: measured 108 against 100 us per iteration)
-        const bool want_xs = co && std::is_same<T, float>::value;
-        const size_t xsb = want_xs ? (size_t)((c.coarse->nc + c.blocks - 1) / c.blocks) * c.coarse->nc * sizeof(T) : 0;
-        const int need = (c.blocks + c.num_sms - 1) / c.num_sms;      // CTAs per SM of this grid
-        // preference: values and inverse rows, columns and inverse rows, values, columns
-        const int modes[4][2] = {{2, 1}, {1, 1}, {2, 0}, {1, 0}};
-        for (int mi = 0; mi < 4 && A.cache == 0; ++mi) {
-            const int mode = modes[mi][0], xs = want_xs ? modes[mi][1] : 0;
-            if (!want_xs && modes[mi][1]) continue;
-            if (mode == 2 && c.row_cache == 1) continue;      // column lists only
-            const size_t sm = colb + (mode == 2 ? valb : 0) + cob + (xs ? xsb : 0);
+        const size_t xsb = co ? (size_t)((c.coarse->nc + blocks - 1) / blocks) * c.coarse->nc * sizeof(float) : 0;
+        const int need = (blocks + c.num_sms - 1) / c.num_sms;        // CTAs per SM of this grid
+        // preference: values and inverse rows, columns and inverse rows, inverse rows, values, columns
+        const int modes[5][2] = {{2, 1}, {1, 1}, {2, 0}, {1, 0}, {0, 1}};
+        const bool rows = c.lmax > 0 && c.row_cache < 2 && !A.bcol;
+        for (const auto &mode : modes) {
+            if (mode[0] && !rows) continue;
+            if (mode[1] && !co) continue;
+            if (mode[0] == 2 && c.row_cache == 1) continue;           // column lists only
+            const size_t sm = (mode[0] ? colb + cob : 0) + (mode[0] == 2 ? valb : 0) + (mode[1] ? xsb : 0);
             if (sm > 200 * 1024) continue;
             if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) {
                 cudaGetLastError();
@@ -1390,15 +1533,15 @@ cudaError_t solve_t(const KrylovCtx &c, const V *vals, const double *b, double *
                 cudaGetLastError();
                 continue;
             }
-            if (per_sm >= need) {
-                A.cache = mode;
-                A.lmax = c.lmax;
-                A.c_xs = xs;
-                smem = sm;
-            }
+            if (per_sm < need) continue;
+            A.cache = mode[0];
+            A.lmax = mode[0] ? c.lmax : 0;
+            A.c_xs = mode[1];
+            smem = sm;
+            break;
         }
     }
-    return cudaLaunchCooperativeKernel(fn, dim3(c.blocks), dim3(kThreads), args, smem, c.stream);
+    return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(kThreads), args, smem, c.stream);
 }
 
 template <int NDOF, class V, class T>
@@ -1451,34 +1594,41 @@ cudaError_t solve_batch_t(const KrylovCtx &c, const gd::BatchKrylov &L, const V 
                                        args, 0, c.stream);
 }
 
-// co-resident CTAs per SM of the solve kernels of one variant (every UP)
+// smallest number of co-resident CTAs per SM over the given kernels
+int coop_min(const void *const *fns, int n)
+{
+    int best = 1 << 30;
+    for (int i = 0; i < n; ++i) {
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fns[i], kThreads, 0) != cudaSuccess) return 0;
+        if (per_sm < best) best = per_sm;
+    }
+    return best;
+}
+// of the single-system kernels of one variant
+template <int NDOF, class V, class T>
+int coop_single()
+{
+    if constexpr (NDOF == 4) {
+        const void *fns[] = {(const void *)bicgstab3_kernel<4, 4, 1, V, T>, (const void *)bicgstab3_kernel<4, 4, 1, V, T, true>};
+        return coop_min(fns, 2);
+    } else {
+        const void *fns[] = {(const void *)bicgstab3_kernel<3, 8, 1, V, T>, (const void *)bicgstab3_kernel<3, 8, 2, V, T>,
+                             (const void *)bicgstab3_kernel<3, 8, 4, V, T>, (const void *)bicgstab3_kernel<3, 8, 1, V, T, true>,
+                             (const void *)bicgstab3_kernel<3, 8, 2, V, T, true>};
+        return coop_min(fns, 5);
+    }
+}
+// of the single-system and batch kernels of one variant
 template <int NDOF, class V, class T>
 int coop_per_sm()
 {
     constexpr int G = NDOF == 3 ? 8 : 32;
-    constexpr int G2 = (NDOF == 4 && std::is_same<T, float>::value) ? 8 : G;   // the other lane counts
-    constexpr int G3 = (NDOF == 4 && std::is_same<T, float>::value) ? 4 : G;   // of the 3D FP32 solve
-    const void *fns[16] = {(const void *)bicgstab3_kernel<NDOF, G, 1, V, T>, (const void *)bicgstab3_kernel<NDOF, G, 2, V, T>,
-                          (const void *)bicgstab3_kernel<NDOF, G, 4, V, T>,
-                          (const void *)bicgstab3_kernel<NDOF, G, 1, V, T, true>,
-                          (const void *)bicgstab3_batch_kernel<NDOF, G, 1, V, T>,
-                          (const void *)bicgstab3_batch_kernel<NDOF, G, 2, V, T>,
-                          (const void *)bicgstab3_batch_kernel<NDOF, G, 4, V, T>,
-                          (const void *)bicgstab3_kernel<NDOF, G2, 1, V, T>, (const void *)bicgstab3_kernel<NDOF, G2, 2, V, T>,
-                          (const void *)bicgstab3_kernel<NDOF, G2, 4, V, T>,
-                          (const void *)bicgstab3_kernel<NDOF, G2, 1, V, T, true>,
-                          (const void *)bicgstab3_kernel<NDOF, G3, 1, V, T>,
-                          (const void *)bicgstab3_kernel<NDOF, G3, 1, V, T, true>,
-                          (const void *)bicgstab3_kernel<NDOF, G, 2, V, T, true>,
-                          (const void *)bicgstab3_kernel<NDOF, G2, 2, V, T, true>,
-                          (const void *)bicgstab3_kernel<NDOF, G3, 2, V, T, true>};
-    int best = 1 << 30;
-    for (const void *f : fns) {
-        int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kThreads, 0) != cudaSuccess) return 0;
-        if (per_sm < best) best = per_sm;
-    }
-    return best;
+    const void *fns[] = {(const void *)bicgstab3_batch_kernel<NDOF, G, 1, V, T>,
+                         (const void *)bicgstab3_batch_kernel<NDOF, G, 2, V, T>,
+                         (const void *)bicgstab3_batch_kernel<NDOF, G, 4, V, T>};
+    const int a = coop_min(fns, 3), b = coop_single<NDOF, V, T>();
+    return a < b ? a : b;
 }
 
 __global__ void narrow_kernel(const double *in, float *out, int64_t n)
@@ -1489,36 +1639,9 @@ __global__ void narrow_kernel(const double *in, float *out, int64_t n)
 
 }  // namespace
 
-template <int NDOF>
-int coop_per_sm_fp32()
-{
-    constexpr int G = NDOF == 3 ? 8 : 32;
-    constexpr int G2 = NDOF == 4 ? 8 : G, G3 = NDOF == 4 ? 4 : G;
-    const void *fns[] = {
-        (const void *)bicgstab3_kernel<NDOF, G, 1, float, float>, (const void *)bicgstab3_kernel<NDOF, G, 2, float, float>,
-        (const void *)bicgstab3_kernel<NDOF, G, 4, float, float>,
-        (const void *)bicgstab3_kernel<NDOF, G, 1, float, float, true>,
-        (const void *)bicgstab3_kernel<NDOF, G, 2, float, float, true>,
-        (const void *)bicgstab3_kernel<NDOF, G2, 1, float, float>, (const void *)bicgstab3_kernel<NDOF, G2, 2, float, float>,
-        (const void *)bicgstab3_kernel<NDOF, G2, 4, float, float>,
-        (const void *)bicgstab3_kernel<NDOF, G2, 1, float, float, true>,
-        (const void *)bicgstab3_kernel<NDOF, G2, 2, float, float, true>,
-        (const void *)bicgstab3_kernel<NDOF, G3, 1, float, float>, (const void *)bicgstab3_kernel<NDOF, G3, 2, float, float>,
-        (const void *)bicgstab3_kernel<NDOF, G3, 4, float, float>,
-        (const void *)bicgstab3_kernel<NDOF, G3, 1, float, float, true>,
-        (const void *)bicgstab3_kernel<NDOF, G3, 2, float, float, true>};
-    int best = 1 << 30;
-    for (const void *f : fns) {
-        int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kThreads, 0) != cudaSuccess) return 0;
-        if (per_sm < best) best = per_sm;
-    }
-    return best;
-}
-
 int krylov_blocks_fp32(int ndof, int num_sms, int cap)
 {
-    int per_sm = ndof == 3 ? coop_per_sm_fp32<3>() : coop_per_sm_fp32<4>();
+    int per_sm = ndof == 3 ? coop_single<3, float, float>() : coop_single<4, float, float>();
     if (cap > 0 && per_sm > cap) per_sm = cap;
     return per_sm * num_sms;
 }
@@ -1542,8 +1665,6 @@ cudaError_t krylov_solve(const KrylovCtx &c, const void *vals, bool fp32_vals, c
     if (fp32_vectors) {
         if (!fp32_vals) return cudaErrorInvalidValue;
         if (c.ndof == 3) return solve_t<3, float, float>(c, (const float *)vals, b, x, rtol, max_it);
-        if (c.lanes == 4) return solve_t<4, float, float, 4>(c, (const float *)vals, b, x, rtol, max_it);
-        if (c.lanes == 8) return solve_t<4, float, float, 8>(c, (const float *)vals, b, x, rtol, max_it);
         return solve_t<4, float, float>(c, (const float *)vals, b, x, rtol, max_it);
     }
     if (c.ndof == 3)
