@@ -41,6 +41,7 @@
 #include "gd_elem32.cuh"
 #include "gd_internal.cuh"
 #include "gd_net_fp64.cuh"
+#include "gd_rows.cuh"
 
 namespace gd {
 namespace {
@@ -51,31 +52,6 @@ constexpr double kTrialMargin = 1e-4;
 
 
 #include "gd_device_fp64.cuh"
-
-// Record of a quadrature point for the row mode, in doubles: every quantity pulled back to
-// the reference element and times J w.
-template <int DIM>
-struct Rec {
-    static constexpr int N2 = DIM * DIM, NS = DIM * (DIM + 1) / 2;
-    static constexpr int A = 0;                      // d P_ij / d H_kl, symmetric, packed upper triangle of (ij) x (kl)
-    static constexpr int B = A + N2 * (N2 + 1) / 2;  // d P_ij / d g_l [ij][l]
-    static constexpr int CV = B + N2 * DIM;          // c_d C^-1, packed symmetric
-    static constexpr int PE = CV + NS;               // dpsi_e/dF (undamaged, without J w) [ij]
-    static constexpr int P = PE + N2;                // stress [ij]
-    static constexpr int Y = P + N2;                 // flux [j]
-    static constexpr int FDK = Y + DIM;              // f_d' dkappa/dphi
-    static constexpr int BCK = FDK + 1;              // beta_d c_kappa
-    static constexpr int PP = BCK + 1;               // beta_d (1 - dkappa/dphi)
-    static constexpr int PEN = PP + 1;               // beta_d (phi - kappa)
-    static constexpr int SIZE = (PEN + 1) | 1;       // odd stride: one bank pair per point
-};
-// position of (r, c) in a packed symmetric N x N matrix (upper triangle by rows)
-template <int N>
-__device__ __forceinline__ int sym_pos(int r, int c)
-{
-    const int lo = r < c ? r : c, hi = r < c ? c : r;
-    return lo * N - lo * (lo - 1) / 2 + hi - lo;
-}
 
 // What a point keeps between its qp phases, in doubles (registers would halve the resident
 // warps)
@@ -101,7 +77,7 @@ struct Smem {
     __host__ __device__ static int net(int wmax) { return (int)(grp::buf_bytes(wmax) / 8); }
     __host__ __device__ static int total(int wmax)
     {
-        const int n = KW * net(wmax), r = NP * Rec<DIM>::SIZE;
+        const int n = KW * net(wmax), r = NP * rows::Rec<DIM>::SIZE;
         return U + ((n > r ? n : r) + 1) / 2 * 2;
     }
 };
@@ -111,85 +87,6 @@ __device__ __forceinline__ void cta_sync()
     if (KW == 1) __syncwarp();
     else __syncthreads();
 }
-
-constexpr double kNp = 0.5 * (1.0 + kGauss), kNm = 0.5 * (1.0 - kGauss);   // 1D shape functions at the Gauss points
-
-// out[b] = sum_q sum_l T[l][q] dN_b/dxi_l(q) (+ sum_q TN[q] N_b(q)), b and q numbered by
-// their axis bits (x lowest).  One axis at a time: the derivative's axis sums its two points,
-// the others mix them with (1 +- 1/sqrt 3) / 2.
-template <bool NPART>
-__device__ __forceinline__ void expand_rows(const double (&T)[2][4], const double *TN, double (&out)[4])
-{
-    // x derivative: S(y), then the y axis; y derivative: S(x), then the x axis
-    const double sx0 = T[0][0] + T[0][1], sx1 = T[0][2] + T[0][3];
-    const double sy0 = T[1][0] + T[1][2], sy1 = T[1][1] + T[1][3];
-    const double hp = 0.5 * kNp, hm = 0.5 * kNm;
-    const double qx0 = hp * sx0 + hm * sx1, qx1 = hm * sx0 + hp * sx1;       // by = 0, 1
-    const double qy0 = hp * sy0 + hm * sy1, qy1 = hm * sy0 + hp * sy1;       // bx = 0, 1
-    out[0] = -qx0 - qy0;
-    out[1] = qx0 - qy1;
-    out[2] = qy0 - qx1;
-    out[3] = qx1 + qy1;
-    if (NPART) {
-        const double a0 = kNp * TN[0] + kNm * TN[1], a1 = kNm * TN[0] + kNp * TN[1];
-        const double b0 = kNp * TN[2] + kNm * TN[3], b1 = kNm * TN[2] + kNp * TN[3];
-        out[0] += kNp * a0 + kNm * b0;
-        out[1] += kNp * a1 + kNm * b1;
-        out[2] += kNm * a0 + kNp * b0;
-        out[3] += kNm * a1 + kNp * b1;
-    }
-}
-template <bool NPART>
-__device__ __forceinline__ void expand_rows(const double (&T)[3][8], const double *TN, double (&out)[8])
-{
-    const double hp = 0.5 * kNp, hm = 0.5 * kNm;
-    double Q[3][4];                      // derivative along axis l; the other two axes (lower first)
-#pragma unroll
-    for (int l = 0; l < 3; ++l) {
-        const int u = l == 0 ? 1 : 0, v = l == 2 ? 1 : 2;
-        double s[4];
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const int q0 = ((m & 1) << u) | ((m >> 1) << v);
-            s[m] = T[l][q0] + T[l][q0 | (1 << l)];
-        }
-        const double a0 = hp * s[0] + hm * s[1], a1 = hm * s[0] + hp * s[1];
-        const double b0 = hp * s[2] + hm * s[3], b1 = hm * s[2] + hp * s[3];
-        Q[l][0] = kNp * a0 + kNm * b0;
-        Q[l][1] = kNp * a1 + kNm * b1;
-        Q[l][2] = kNm * a0 + kNp * b0;
-        Q[l][3] = kNm * a1 + kNp * b1;
-    }
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-        const int bx = b & 1, by = (b >> 1) & 1, bz = b >> 2;
-        const double x = Q[0][by | (bz << 1)], y = Q[1][bx | (bz << 1)], z = Q[2][bx | (by << 1)];
-        const double xy = (bx == by) ? x + y : x - y;        // sign of x times the sum
-        out[b] = (bx ? xy : -xy) + (bz ? z : -z);
-    }
-    if (NPART) {
-        double a[8], c[8];
-#pragma unroll
-        for (int q = 0; q < 8; q += 2) {
-            a[q] = kNp * TN[q] + kNm * TN[q + 1];
-            a[q + 1] = kNm * TN[q] + kNp * TN[q + 1];
-        }
-#pragma unroll
-        for (int z = 0; z < 8; z += 4)
-#pragma unroll
-            for (int x = 0; x < 2; ++x) {
-                c[z + x] = kNp * a[z + x] + kNm * a[z + x + 2];
-                c[z + x + 2] = kNm * a[z + x] + kNp * a[z + x + 2];
-            }
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            out[b] += kNp * c[b] + kNm * c[b + 4];
-            out[b + 4] += kNm * c[b] + kNp * c[b + 4];
-        }
-    }
-}
-// node with the axis bits l (x lowest): counter-clockwise numbering of each layer
-__device__ __forceinline__ int node_of_bits(int l) { return l ^ ((l >> 1) & 1); }
 
 // Local damage update (Eq. (dd_7_no_nn)) of the CTA's points p0 .. p0 + 3 that
 // belong to specimen sn: psi_e, phi, kappa_n at sIn[p 4 ..], results (kappa, loading, G',
@@ -417,7 +314,7 @@ __global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
 {
     using G_ = Geo<DIM>;
     using S_ = Smem<DIM, NP, KW>;
-    using R_ = Rec<DIM>;
+    using R_ = rows::Rec<DIM>;
     using P_ = State<DIM>;
     constexpr int NEN = G_::NEN, NQ = G_::NQ, NDOF = G_::NDOF, EL = S_::EL, N2 = DIM * DIM;
     extern __shared__ __align__(16) double smem[];
@@ -722,167 +619,20 @@ __global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
                 if (A.loading) A.loading[e_me * NQ + q] = loading ? 1 : 0;
                 if (o[4] > 0.5) atomicAdd(A.counters, 1);
             }
-            double *rec = sRec + pt * R_::SIZE;
-            const double Jw = valid ? st[P_::DET] : 0.0;
-            const bool dmg = kappa > m.kappa_d;
-            const double fd = dmg ? fx::exp_neg(m.eta_d * (kappa - m.kappa_d)) : 1.0;
-            const double fdp = dmg ? -m.eta_d * fd : 0.0;
-            const double ck = loading ? -o[2] / o[3] : 0.0;          // G' / (1 - G' dq/dkappa)
-            const double dkdphi = ck * m.qcoef / fd;                  // dq/dphi = qcoef / f_d
-            const double J = 1.0 + st[P_::X + 2], I1 = 3.0 + st[P_::X], ij = 1.0 / J;
-            const double *ps = st + P_::PS, *ph = st + P_::PH;
-            // F^-1 = cof(F)^T / J; pulled back to the reference element: F' = F Ji^T (F_iJ Ji_jJ),
-            // Fi'_ji = Ji_jJ F^-1_Ji
-            double Fp[DIM][DIM], Fi[DIM][DIM], G2[DIM][DIM], h[DIM], mv[DIM], b[DIM][DIM], Mj[DIM][DIM];
-            {
-                double Fv[DIM][DIM], F[DIM][DIM], Ji[DIM][DIM];
-#pragma unroll
-                for (int i = 0; i < DIM; ++i)
-#pragma unroll
-                    for (int j = 0; j < DIM; ++j) {
-                        F[i][j] = st[P_::F + i * DIM + j];
-                        Ji[i][j] = st[P_::JI + i * DIM + j];
-                    }
-                if constexpr (DIM == 2) {
-                    Fv[0][0] = F[1][1] * ij; Fv[0][1] = -F[0][1] * ij;
-                    Fv[1][0] = -F[1][0] * ij; Fv[1][1] = F[0][0] * ij;
-                } else {
-#pragma unroll
-                    for (int i = 0; i < DIM; ++i)
-#pragma unroll
-                        for (int j = 0; j < DIM; ++j) {
-                            const int i1 = (j + 1) % DIM, i2 = (j + 2) % DIM, j1 = (i + 1) % DIM, j2 = (i + 2) % DIM;
-                            Fv[i][j] = (F[i1][j1] * F[i2][j2] - F[i1][j2] * F[i2][j1]) * ij;
-                        }
-                }
-#pragma unroll
-                for (int i = 0; i < DIM; ++i)
-#pragma unroll
-                    for (int j = 0; j < DIM; ++j) {
-                        double s = 0.0, t = 0.0;
-#pragma unroll
-                        for (int K = 0; K < DIM; ++K) {
-                            s += F[i][K] * Ji[j][K];
-                            t += Ji[j][K] * Fv[K][i];
-                        }
-                        Fp[i][j] = s;
-                        Fi[j][i] = t;
-                    }
-                // F F^T and the metric (delta_JL pulled back)
-#pragma unroll
-                for (int i = 0; i < DIM; ++i)
-#pragma unroll
-                    for (int k = i; k < DIM; ++k) {
-                        double s = 0.0, t = 0.0;
-#pragma unroll
-                        for (int K = 0; K < DIM; ++K) {
-                            s += F[i][K] * F[k][K];
-                            t += Ji[i][K] * Ji[k][K];
-                        }
-                        b[i][k] = b[k][i] = s;
-                        Mj[i][k] = Mj[k][i] = t;
-                    }
-            }
-            // h = F^-T grad phi (= Fi'^T of the reference gradient), C^-1 grad phi pulled back
+            double F[DIM][DIM], Ji[DIM][DIM], gx[DIM];
 #pragma unroll
             for (int i = 0; i < DIM; ++i) {
-                double s = 0.0;
-#pragma unroll
-                for (int k = 0; k < DIM; ++k) s += Fi[k][i] * st[P_::GX + k];
-                h[i] = s;
-            }
-#pragma unroll
-            for (int j = 0; j < DIM; ++j) {
-                double s = 0.0;
-#pragma unroll
-                for (int i = 0; i < DIM; ++i) s += Fi[j][i] * h[i];
-                mv[j] = s;
-            }
-            // G^2 = dI2/dF pulled back; P = f_d dpsi_e/dF - c_d h (x) m
-            const double ps3J = ps[2] * J, cdw = m.c_d * Jw, fdw = fd * Jw;
-#pragma unroll
-            for (int i = 0; i < DIM; ++i)
+                gx[i] = st[P_::GX + i];
 #pragma unroll
                 for (int j = 0; j < DIM; ++j) {
-                    double s = I1 * Fp[i][j];
-#pragma unroll
-                    for (int k = 0; k < DIM; ++k) s -= b[i][k] * Fp[k][j];
-                    G2[i][j] = 2.0 * s;
-                    const double Pe = 2.0 * ps[0] * Fp[i][j] + ps[1] * G2[i][j] + ps3J * Fi[j][i];
-                    rec[R_::PE + i * DIM + j] = Pe;
-                    rec[R_::P + i * DIM + j] = fdw * Pe - cdw * h[i] * mv[j];
+                    F[i][j] = st[P_::F + i * DIM + j];
+                    Ji[i][j] = st[P_::JI + i * DIM + j];
                 }
-#pragma unroll
-            for (int j = 0; j < DIM; ++j) rec[R_::Y + j] = cdw * mv[j];
-            rec[R_::PEN] = m.beta_d * (st[P_::PHI] - kappa) * Jw;
-            if (A.tangent) {
-                rec[R_::FDK] = fdp * dkdphi * Jw;
-                rec[R_::BCK] = m.beta_d * ck * Jw;
-                rec[R_::PP] = m.beta_d * (1.0 - dkdphi) * Jw;
-                double hw[DIM];                                    // c_d J w h
-#pragma unroll
-                for (int i = 0; i < DIM; ++i) hw[i] = cdw * h[i];
-                double Cv[DIM][DIM], Sj[DIM][DIM];
-                const double g2w = 2.0 * fdw * ps[1], g1w = 2.0 * fdw * ps[0] + g2w * I1;
-#pragma unroll
-                for (int j = 0; j < DIM; ++j)
-#pragma unroll
-                    for (int l = j; l < DIM; ++l) {
-                        double ci = 0.0, c = 0.0;
-                        const double mm = Mj[j][l];
-#pragma unroll
-                        for (int i = 0; i < DIM; ++i) {
-                            ci += Fi[j][i] * Fi[l][i];             // C^-1
-                            c += Fp[i][j] * Fp[i][l];              // C
-                        }
-                        Cv[j][l] = Cv[l][j] = cdw * ci;
-                        rec[R_::CV + sym_pos<DIM>(j, l)] = cdw * ci;
-                        Mj[j][l] = Mj[l][j] = g2w * mm;
-                        Sj[j][l] = Sj[l][j] = g1w * mm - g2w * c;
-                    }
-                // d2 psi_e/dF2 with the kappa coupling, times f_d and J w:
-                //   sum_mn (f_d psi_mn + f_d' c_kappa psi_m psi_n) G^m G^n + f_d (psi_1 D2(I1) + psi_2 D2(I2) + psi_3 D2(J)),
-                //   G^1 = 2 F, G^2 = 2 (I1 F - F F^T F), G^3 = J F^-T,
-                //   D2(I1) = 2 d_ik d_JL,  D2(J) = J (F^-1_Ji F^-1_Lk - F^-1_Jk F^-1_Li),
-                //   D2(I2) = 2 [2 F_iJ F_kL - F_iL F_kJ + (I1 d_JL - C_JL) d_ik - d_JL b_ik];
-                // their products of first derivatives join the G^m G^n sum
-                const double ckw = fdp * ck * Jw, g3w = fdw * ps3J;
-                const double h11 = 4.0 * (fdw * ph[0] + ckw * ps[0] * ps[0]) + 2.0 * g2w;
-                const double h12 = 2.0 * (fdw * ph[1] + ckw * ps[0] * ps[1]);
-                const double h13 = 2.0 * (fdw * ph[2] + ckw * ps[0] * ps[2]) * J;
-                const double h22 = fdw * ph[3] + ckw * ps[1] * ps[1];
-                const double h23 = (fdw * ph[4] + ckw * ps[1] * ps[2]) * J;
-                const double h33 = (fdw * ph[5] + ckw * ps[2] * ps[2]) * J * J + g3w;
-                double V[DIM][DIM];                                // c_d J w h_k m_j - f_d psi_3 J J w F^-1_jk
-#pragma unroll
-                for (int k = 0; k < DIM; ++k)
-#pragma unroll
-                    for (int j = 0; j < DIM; ++j) V[k][j] = hw[k] * mv[j] - g3w * Fi[j][k];
-#pragma unroll
-                for (int i = 0; i < DIM; ++i)
-#pragma unroll
-                    for (int j = 0; j < DIM; ++j) {
-                        const int r = DIM * i + j;
-                        const double t1 = h11 * Fp[i][j] + h12 * G2[i][j] + h13 * Fi[j][i];
-                        const double t2 = h12 * Fp[i][j] + h22 * G2[i][j] + h23 * Fi[j][i];
-                        const double t3 = h13 * Fp[i][j] + h23 * G2[i][j] + h33 * Fi[j][i];
-#pragma unroll
-                        for (int c = r; c < N2; ++c) {
-                            const int k = c / DIM, l = c % DIM;
-                            double v = t1 * Fp[k][l] + t2 * G2[k][l] + t3 * Fi[l][k];
-                            if (i == k) v += Sj[j][l];
-                            v -= Mj[j][l] * b[i][k];
-                            v -= g2w * Fp[i][l] * Fp[k][j];
-                            v += Fi[l][i] * V[k][j];
-                            v += hw[i] * mv[l] * Fi[j][k];
-                            v += Cv[j][l] * (h[i] * h[k]);
-                            rec[R_::A + sym_pos<N2>(r, c)] = v;
-                        }
-#pragma unroll
-                        for (int l = 0; l < DIM; ++l)
-                            rec[R_::B + r * DIM + l] = -(cdw * mv[j] * Fi[l][i] + h[i] * Cv[j][l]);
-                    }
             }
+            const double fd = kappa > m.kappa_d ? fx::exp_neg(m.eta_d * (kappa - m.kappa_d)) : 1.0;
+            rows::point_record<double, DIM>(m, F, Ji, gx, st + P_::X, st[P_::PHI], valid ? st[P_::DET] : 0.0, st + P_::PS,
+                                            st + P_::PH, kappa, fd, loading, o[2], o[3], A.tangent != 0,
+                                            sRec + pt * R_::SIZE);
         }
         {
             const unsigned n_load = __ballot_sync(0xffffffffu, loading);
@@ -891,89 +641,8 @@ __global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
         cta_sync<KW>();
 
         // ================= row mode: element residual and tangent =================
-        {
-            constexpr int EPWR = 8 / NQ;                         // elements of a warp: HEX8 1, Q4 2
-            const int ee = lane / G_::ND, row = lane % G_::ND, a = row / NDOF, i = row % NDOF;
-            const int el_r = warp * EPWR + ee;
-            const int64_t e = e0 + el_r;
-            if (warp < NP / 8 && lane < EPWR * G_::ND && e < A.n_elems) {
-                const double *R0 = sRec + el_r * NQ * R_::SIZE;
-                const bool pr = i == DIM;                        // a phi row
-                double Rr = 0.0;
-#pragma unroll
-                for (int qq = 0; qq < NQ; ++qq) {
-                    const double *rq = R0 + qq * R_::SIZE, *c = sRef + (qq * NEN + a) * 4;
-                    const double *pj = rq + (pr ? R_::Y : R_::P + i * DIM);
-#pragma unroll
-                    for (int j = 0; j < DIM; ++j) Rr += c[j] * pj[j];
-                    if (pr) Rr += c[3] * rq[R_::PEN];
-                }
-                const int32_t na = __ldg(A.conn + e * NEN + a);
-                if (A.R) atomicAdd(A.R + (int64_t)na * NDOF + i, Rr);
-                if (A.tangent) {
-                    const int32_t rb = __ldg(A.rowptr + (int64_t)na * NDOF);
-                    const int64_t off = (int64_t)i * (__ldg(A.rowptr + (int64_t)na * NDOF + 1) - rb);
-                    const int32_t *sl = A.slot + (e * NEN + a) * NEN;
-                    double T[DIM][NQ], K[NEN];
-                    auto add = [&](int k) {
-#pragma unroll
-                        for (int l = 0; l < NEN; ++l) {
-                            const int64_t pos = (int64_t)__ldg(sl + node_of_bits(l)) + off + k;
-                            if (A.vals) atomicAdd(A.vals + pos, K[l]);
-                            else atomicAdd(A.vals32 + pos, (float)K[l]);
-                        }
-                    };
-#pragma unroll 1
-                    for (int k = 0; k < DIM; ++k) {
-                        // columns (b, u_k)
-                        int at[DIM][DIM];
-#pragma unroll
-                        for (int j = 0; j < DIM; ++j)
-#pragma unroll
-                            for (int l = 0; l < DIM; ++l)
-                                at[j][l] = pr ? R_::B + (DIM * k + l) * DIM + j
-                                              : R_::A + sym_pos<N2>(DIM * i + j, DIM * k + l);
-#pragma unroll
-                        for (int qq = 0; qq < NQ; ++qq) {
-                            const double *rq = R0 + qq * R_::SIZE, *c = sRef + (qq * NEN + a) * 4;
-#pragma unroll
-                            for (int l = 0; l < DIM; ++l) {
-                                double t = 0.0;
-#pragma unroll
-                                for (int j = 0; j < DIM; ++j) t += c[j] * rq[at[j][l]];
-                                T[l][qq] = t;
-                            }
-                            if (pr) {
-                                const double nb = c[3] * rq[R_::BCK];
-#pragma unroll
-                                for (int l = 0; l < DIM; ++l) T[l][qq] -= nb * rq[R_::PE + DIM * k + l];
-                            }
-                        }
-                        expand_rows<false>(T, nullptr, K);
-                        add(k);
-                    }
-                    // columns (b, phi)
-                    double TN[NQ];
-#pragma unroll
-                    for (int qq = 0; qq < NQ; ++qq) {
-                        const double *rq = R0 + qq * R_::SIZE, *c = sRef + (qq * NEN + a) * 4;
-                        double t = 0.0;
-#pragma unroll
-                        for (int l = 0; l < DIM; ++l) {
-                            double s = 0.0;
-#pragma unroll
-                            for (int j = 0; j < DIM; ++j)
-                                s += c[j] * rq[pr ? R_::CV + sym_pos<DIM>(j, l) : R_::B + (DIM * i + j) * DIM + l];
-                            T[l][qq] = s;
-                            t += c[l] * rq[R_::PE + (pr ? 0 : i) * DIM + l];
-                        }
-                        TN[qq] = pr ? c[3] * rq[R_::PP] : rq[R_::FDK] * t;
-                    }
-                    expand_rows<true>(T, TN, K);
-                    add(DIM);
-                }
-            }
-        }
+        if (warp < NP / 8)
+            rows::add_rows<double, DIM>(A, sRec + warp * 8 * R_::SIZE, sRef, e0 + warp * (8 / NQ), lane);
     }
 }
 

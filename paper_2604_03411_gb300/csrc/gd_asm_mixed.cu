@@ -125,26 +125,37 @@ __device__ void psi_net_unit(const DevNet &net, const float *x, float *out10, fl
     __syncwarp();
 }
 
+// floats of a warp's shared-memory scratch
+template <int DIM>
+__host__ __device__ constexpr int scratch_floats(int wmax)
+{
+    using G_ = Geo<DIM>;
+    return G_::EPW * G_::NEN * (DIM + G_::NDOF) + 32 * rows::Rec<DIM>::SIZE + 32 * 4 + 32 * 10 + 5 * wmax;
+}
+
 template <int DIM, int KW>
 __global__ void __launch_bounds__(32 * KW) asm_fp32_kernel(AsmArgs A)
 {
     using G_ = Geo<DIM>;
+    using R_ = rows::Rec<DIM>;
     constexpr int NEN = G_::NEN, NQ = G_::NQ, NDOF = G_::NDOF, EPW = G_::EPW;
     extern __shared__ float smem_f[];
-    float *smem = smem_f;
+    float *sRef = smem_f;                            // [NQ][NEN][4]
+    float *smem = smem_f + NQ * NEN * 4;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wmax = A.wmax;
     // per-warp scratch
-    const int scratch = EPW * NEN * (DIM + NDOF) + 32 * Q_REC + 32 * 4 + 32 * 10 + 5 * wmax + 2 * NQ * NEN * V_REC;
+    const int scratch = scratch_floats<DIM>(wmax);
     float *ws = smem + warp * scratch;
     float *sX = ws;                                  // [EPW][NEN][DIM]
     float *sD = sX + EPW * NEN * DIM;                // [EPW][NEN][NDOF]
-    float *sRec = sD + EPW * NEN * NDOF;             // [32][Q_REC]
-    float *sIn = sRec + 32 * Q_REC;                  // [32][4]: network input x (3), then kappa out
+    float *sRec = sD + EPW * NEN * NDOF;             // [32] records of the points
+    float *sIn = sRec + 32 * R_::SIZE;               // [32][4]: network input x (3), then kappa out
     float *sOut = sIn + 32 * 4;                      // [32][10]: N, grad, Hess / local-solve results
     float *sBuf = sOut + 32 * 10;                    // unit-mode buffers
-    float *sVec = sBuf + 5 * wmax;                   // [EPR*NQ*NEN][V_REC]
     const MatF m = to_f(A.mat);
+    ref_table<DIM>(sRef, threadIdx.x, 32 * KW);
+    __syncthreads();
 
     const int64_t n_batches = (A.n_elems + EPW - 1) / EPW;
     for (int64_t batch = (int64_t)blockIdx.x * KW + warp; batch < n_batches;
@@ -158,9 +169,9 @@ __global__ void __launch_bounds__(32 * KW) asm_fp32_kernel(AsmArgs A)
         const int64_t e_me = e0 + el;
         const bool valid = e_me < A.n_elems;
         const NcF nc = ncf(A.netc[valid ? spec_of(A, e_me) : 0]);
-        float *rec = sRec + lane * Q_REC;
-        float F[3][3], H[3][3], phi, g[3], x[3], Jdet;
-        qp_kinematics<DIM>(sX, sD, el, q, rec, F, H, phi, g, x, Jdet);
+        float F[DIM][DIM], Ji[DIM][DIM], gx[DIM], phi, x[3], det;
+        qp_kinematics<DIM>(sX, sD, sRef + q * NEN * 4, el, F, Ji, gx, phi, x, det);
+        const float Jdet = 1.0f + x[2];
         // network input (raw or isochoric map)
         float Tm[3][3], T2[3][6];   // dy/dx and d2y/dx2 of the iso map (raw: identity)
         {
@@ -250,28 +261,22 @@ __global__ void __launch_bounds__(32 * KW) asm_fp32_kernel(AsmArgs A)
                 if (o[4] > 0.5f) atomicAdd(A.counters, 1);
                 if (loading) atomicAdd(A.counters + 1, 1);
             }
-            stress_records(m, F, x, g, phi, Jdet, ps, ph, kappa, loading, o[2], o[3], valid, rec);
+            const float fd = kappa > m.kappa_d ? expf(-m.eta_d * (kappa - m.kappa_d)) : 1.0f;
+            rows::point_record<float, DIM>(m, F, Ji, gx, x, phi, valid ? det : 0.0f, ps, ph, kappa, fd, loading, o[2],
+                                           o[3], A.tangent != 0, sRec + lane * R_::SIZE);
         }
         __syncwarp();
 
         // ================= row mode: element residual and tangent =================
-        row_mode<DIM>(A, m, sRec, sVec, e0, lane);
+        for (int u = 0; u < 4; ++u) rows::add_rows<float, DIM>(A, sRec + u * 8 * R_::SIZE, sRef, e0 + u * (8 / NQ), lane);
+        __syncwarp();
     }
-}
-
-template <int DIM>
-size_t smem_bytes(int wmax)
-{
-    using G_ = Geo<DIM>;
-    size_t scratch = G_::EPW * G_::NEN * (DIM + G_::NDOF) + 32 * Q_REC + 32 * 4 + 32 * 10 + 5 * wmax +
-                     2 * G_::NQ * G_::NEN * V_REC;
-    return scratch * sizeof(float);          // per warp
 }
 
 template <int DIM, int KW>
 cudaError_t launch_kw(const AsmArgs &a, int num_sms, const AsmTune &t, cudaStream_t s)
 {
-    size_t sm = smem_bytes<DIM>(a.wmax) * KW;
+    const size_t sm = sizeof(float) * (Geo<DIM>::NQ * Geo<DIM>::NEN * 4 + (size_t)scratch_floats<DIM>(a.wmax) * KW);
     int dev = 0, optin = 0;
     cudaError_t e0 = cudaGetDevice(&dev);
     if (e0 == cudaSuccess) e0 = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);

@@ -29,6 +29,11 @@
 // kernel (gd_elem32.cuh); the loading/unloading decision, the history and the residual
 // accumulation are FP64.
 //
+// Bound by instruction latency at two CTAs (8 warps) per SM; measured on 2,097,152 HEX8
+// points, widths 64, split operands, tangent: 10.0 -> 4.3 ms with unit loops free of
+// branches, sigmoids kept in tensor memory between the rounds instead of recomputed, and the
+// rows of gd_rows.cuh (18,816 points: 156 -> 104 us per call).
+//
 // Paper passages: Sec. 3.1f (kinematics, residual), Sec. 2.2f and Sec. 3.2f Eq.
 // (dd_7_no_nn) (local update, KKT), Sec. 3.2f (monolithic tangent), Sec. 4.1f, Sec. 4.2f
 // Eqs. (dd_0), (dd_1), (Gq_NN), (dd_7).
@@ -128,6 +133,19 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16])
+{
+    uint32_t r[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(v[i]);
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};" ::"r"(
+            r[0]),
+        "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]),
+        "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // ---------------------------------------------------------------- operand packing
@@ -235,41 +253,68 @@ __device__ __forceinline__ void slot_fill(Shared &S, const TcArgs &T, int src_of
     S.slot_pending = true;
 }
 
+// 16 operand columns from j0 on of this thread's row: high parts into tile t0 (and, with
+// split operands, residuals into t1)
+template <bool SPLIT>
+__device__ __forceinline__ void st_row16(uint8_t *t0, uint8_t *t1, int row, int j0, int wp, const float (&v)[16])
+{
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float a[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) a[i] = v[8 * h + i];
+        st_row8(t0, row, j0 / 8 + h, wp, a);
+        if (SPLIT) st_row8_lo(t1, row, j0 / 8 + h, wp, a);
+    }
+}
+
 // ---------------------------------------------------------------- energy network
+// The per-unit vectors are padded to wp with zeros, whose products vanish, so the unit loops
+// have no branches and 16 units are in flight at a time (a test per unit made every unit a
+// serial chain of about 150 cycles).
 // Layer 1 of the energy network for this thread's point; writes the operand rows of
 // one round.  Plain: round 0 = (s1, sg1 W1[:,0]), round 1 = (sg1 W1[:,1], sg1 W1[:,2])
 // into tiles 0 and 1; split: round r = column r (r = 0: s1, r = 1..3: sg1 W1[:,r-1]),
-// high part into tile 0 and residual into tile 1.
+// high part into tile 0 and residual into tile 1.  Round 0 leaves sg1 in tensor-memory columns
+// [3 wp, 4 wp), which the last round's product overwrites after every round has read it.
 template <bool SPLIT>
-__device__ __forceinline__ void energy_l1(const float *e32, int w, int wp, const float (&y)[3], int round, uint8_t *t0,
-                                          uint8_t *t1, int row)
+__device__ __forceinline__ void energy_l1(const float4 *E1, int wp, const float (&y)[3], int round, uint8_t *t0,
+                                          uint8_t *t1, int row, uint32_t sg_base)
 {
-    const float *W1 = e32, *b1 = e32 + 3 * w;
-    for (int j8 = 0; j8 < wp / 8; ++j8) {
-        float a[8], b[8];
+    for (int j0 = 0; j0 < wp; j0 += 16) {
+        float sg[16], a[16];
+        if (round == 0) {
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-            const int j = j8 * 8 + jj;
-            float va = 0.0f, vb = 0.0f;
-            if (j < w) {
-                const float w0 = W1[3 * j], w1 = W1[3 * j + 1], w2 = W1[3 * j + 2];
-                const float h = b1[j] + w0 * y[0] + w1 * y[1] + w2 * y[2];
-                float sp, sg;
-                sp_sig_fast(h, sp, sg);
-                if (!SPLIT) {
-                    va = round == 0 ? sp : sg * w1;
-                    vb = round == 0 ? sg * w0 : sg * w2;
-                } else {
-                    va = round == 0 ? sp : sg * (round == 1 ? w0 : round == 2 ? w1 : w2);
-                }
+            for (int i = 0; i < 16; ++i) {
+                const float4 w = E1[j0 + i];
+                sp_sig_fast(w.w + w.x * y[0] + w.y * y[1] + w.z * y[2], a[i], sg[i]);
             }
-            a[jj] = va;
-            b[jj] = vb;
+            tmem_st16(sg_base + (uint32_t)j0, sg);
+        } else {
+            tmem_ld16(sg_base + (uint32_t)j0, sg);
+            tmem_wait_ld();
         }
-        st_row8(t0, row, j8, wp, a);
-        if (SPLIT) st_row8_lo(t1, row, j8, wp, a);
-        else st_row8(t1, row, j8, wp, b);
+        if (SPLIT) {
+            if (round > 0)
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const float4 w = E1[j0 + i];
+                    a[i] = sg[i] * (round == 1 ? w.x : round == 2 ? w.y : w.z);
+                }
+            st_row16<true>(t0, t1, row, j0, wp, a);
+        } else {
+            float b[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const float4 w = E1[j0 + i];
+                if (round > 0) a[i] = sg[i] * w.y;
+                b[i] = sg[i] * (round == 0 ? w.x : w.z);
+            }
+            st_row16<false>(t0, t0, row, j0, wp, a);
+            st_row16<false>(t1, t1, row, j0, wp, b);
+        }
     }
+    if (round == 0) tmem_wait_st();
 }
 
 // Value, gradient and Hessian (sym6 order) of the energy network at y for every point
@@ -281,10 +326,9 @@ template <bool SPLIT>
 __device__ void energy_net_tc(Shared &S, const TcArgs &T, const float (&y)[3], float (&out)[10], int tid, int warp)
 {
     const TcLayout &L = T.L;
-    const int w = L.we, wp = L.wpe;
-    const float *e32 = reinterpret_cast<const float *>(S.blob + T.s_e32);
-    const float *W1 = e32, *b1 = e32 + 3 * w, *A2 = e32 + 4 * w, *b2 = e32 + 7 * w, *w3 = e32 + 8 * w,
-                *a3 = e32 + 9 * w;
+    const int wp = L.wpe;
+    const float4 *E1 = reinterpret_cast<const float4 *>(S.blob + T.s_e32), *E2 = E1 + wp;     // W1 b1, A2 b2
+    const float *w3 = reinterpret_cast<const float *>(E2 + wp), *a3 = w3 + wp;
     uint8_t *t0 = S.tiles, *t1 = S.tiles + T.tile_bytes;
     const uint32_t a0 = saddr(t0), a1 = saddr(t1), bw = saddr(S.blob), br = saddr(S.blob + T.s_slot);
     const uint32_t lane_base = S.tbase + ((uint32_t)(warp * 32) << 16);
@@ -292,7 +336,8 @@ __device__ void energy_net_tc(Shared &S, const TcArgs &T, const float (&y)[3], f
     // ---- forward columns: type t lands in tensor-memory columns [t wp, (t+1) wp)
     for (int r = 0; r < ROUNDS; ++r) {
         if (r > 0) wait_mma(S, T);           // the previous round's product has read the tiles
-        energy_l1<SPLIT>(e32, w, wp, y, r, t0, t1, tid);
+        energy_l1<SPLIT>(E1, wp, y, r, t0, t1, tid, lane_base + (uint32_t)(3 * wp));
+        tc_before();
         fence_async_smem();
         __syncthreads();
         if (tid == 0) {
@@ -321,38 +366,27 @@ __device__ void energy_net_tc(Shared &S, const TcArgs &T, const float (&y)[3], f
         float u[16];
 #pragma unroll
         for (int kk = 0; kk < 16; ++kk) {
-            const int k = k0 + kk;
-            u[kk] = 0.0f;
-            if (k < w) {
-                const float c0 = A2[3 * k], c1 = A2[3 * k + 1], c2 = A2[3 * k + 2];
-                const float h = hS[kk] + b2[k] + c0 * y[0] + c1 * y[1] + c2 * y[2];
-                const float ga = g0[kk] + c0, gb = g1[kk] + c1, gc = g2[kk] + c2;
-                float spv, sg;
-                sp_sig_fast(h, spv, sg);
-                const float wk = w3[k];
-                const float e2 = wk * sg * (1.0f - sg);
-                acc[0] += wk * spv;
-                acc[1] += wk * sg * ga;
-                acc[2] += wk * sg * gb;
-                acc[3] += wk * sg * gc;
-                acc[4] += e2 * ga * ga;
-                acc[5] += e2 * ga * gb;
-                acc[6] += e2 * ga * gc;
-                acc[7] += e2 * gb * gb;
-                acc[8] += e2 * gb * gc;
-                acc[9] += e2 * gc * gc;
-                u[kk] = wk * sg;
-            }
+            const float4 c = E2[k0 + kk];
+            const float h = hS[kk] + c.w + c.x * y[0] + c.y * y[1] + c.z * y[2];
+            const float ga = g0[kk] + c.x, gb = g1[kk] + c.y, gc = g2[kk] + c.z;
+            float spv, sg;
+            sp_sig_fast(h, spv, sg);
+            const float wk = w3[k0 + kk], us = wk * sg;
+            const float e2 = us * (1.0f - sg), ea = e2 * ga, eb = e2 * gb;
+            acc[0] += wk * spv;
+            acc[1] += us * ga;
+            acc[2] += us * gb;
+            acc[3] += us * gc;
+            acc[4] += ea * ga;
+            acc[5] += ea * gb;
+            acc[6] += ea * gc;
+            acc[7] += eb * gb;
+            acc[8] += eb * gc;
+            acc[9] += e2 * gc * gc;
+            u[kk] = us;
         }
         // reverse operand u = w3 o sg2 (the tiles are free: the last forward product is done)
-#pragma unroll
-        for (int h8 = 0; h8 < 2; ++h8) {
-            float v8[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) v8[i] = u[h8 * 8 + i];
-            st_row8(t0, tid, k0 / 8 + h8, wp, v8);
-            if (SPLIT) st_row8_lo(t1, tid, k0 / 8 + h8, wp, v8);
-        }
+        st_row16<SPLIT>(t0, t1, tid, k0, wp, u);
     }
     // ---- reverse column v = W2^T u into columns [0, wp) (W2^T in the weight slot)
     slot_wait(S, T);
@@ -374,20 +408,16 @@ __device__ void energy_net_tc(Shared &S, const TcArgs &T, const float (&y)[3], f
         tmem_wait_ld();
 #pragma unroll
         for (int jj = 0; jj < 16; ++jj) {
-            const int j = j0 + jj;
-            if (j < w) {
-                const float w0 = W1[3 * j], w1 = W1[3 * j + 1], w2 = W1[3 * j + 2];
-                const float h = b1[j] + w0 * y[0] + w1 * y[1] + w2 * y[2];
-                float spv, sg;
-                sp_sig_fast(h, spv, sg);
-                const float c = v[jj] * sg * (1.0f - sg);
-                acc[4] += c * w0 * w0;
-                acc[5] += c * w0 * w1;
-                acc[6] += c * w0 * w2;
-                acc[7] += c * w1 * w1;
-                acc[8] += c * w1 * w2;
-                acc[9] += c * w2 * w2;
-            }
+            const float4 w = E1[j0 + jj];
+            float spv, sg;
+            sp_sig_fast(w.w + w.x * y[0] + w.y * y[1] + w.z * y[2], spv, sg);
+            const float c = v[jj] * sg * (1.0f - sg), cx = c * w.x, cy = c * w.y;
+            acc[4] += cx * w.x;
+            acc[5] += cx * w.y;
+            acc[6] += cx * w.z;
+            acc[7] += cy * w.y;
+            acc[8] += cy * w.z;
+            acc[9] += c * w.z * w.z;
         }
     }
     tc_before();
@@ -402,36 +432,31 @@ __device__ void energy_net_tc(Shared &S, const TcArgs &T, const float (&y)[3], f
 // ---------------------------------------------------------------- yield network
 // Layer 1 of the yield network at q: s1 = sp(V1 q + c1) and sg1 V1.  Plain: both into
 // tiles 0 and 1; split: round 0 = s1, round 1 = sg1 V1 (high part into tile 0,
-// residual into tile 1).
+// residual into tile 1), kept in tensor-memory columns [2 wp, 3 wp) from round 0 on.
 template <bool SPLIT>
-__device__ __forceinline__ void yield_l1(const float *y32, int w, int wp, float q, int round, uint8_t *t0, uint8_t *t1,
-                                         int row)
+__device__ __forceinline__ void yield_l1(const float2 *Y1, int wp, float q, int round, uint8_t *t0, uint8_t *t1,
+                                         int row, uint32_t keep)
 {
-    const float *V1 = y32, *c1 = y32 + w;
-    for (int j8 = 0; j8 < wp / 8; ++j8) {
-        float a[8], b[8];
+    for (int j0 = 0; j0 < wp; j0 += 16) {
+        float a[16], b[16];
+        if (round == 0) {
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-            const int j = j8 * 8 + jj;
-            float va = 0.0f, vb = 0.0f;
-            if (j < w) {
-                const float v1 = V1[j];
-                float sp, sg;
-                sp_sig_fast(c1[j] + v1 * q, sp, sg);
-                if (!SPLIT) {
-                    va = sp;
-                    vb = sg * v1;
-                } else {
-                    va = round == 0 ? sp : sg * v1;
-                }
+            for (int i = 0; i < 16; ++i) {
+                const float2 v = Y1[j0 + i];
+                float sg;
+                sp_sig_fast(v.y + v.x * q, a[i], sg);
+                b[i] = sg * v.x;
             }
-            a[jj] = va;
-            b[jj] = vb;
+            if (SPLIT) tmem_st16(keep + (uint32_t)j0, b);
+            st_row16<SPLIT>(t0, t1, row, j0, wp, a);
+            if (!SPLIT) st_row16<false>(t1, t1, row, j0, wp, b);
+        } else {
+            tmem_ld16(keep + (uint32_t)j0, b);
+            tmem_wait_ld();
+            st_row16<SPLIT>(t0, t1, row, j0, wp, b);
         }
-        st_row8(t0, row, j8, wp, a);
-        if (SPLIT) st_row8_lo(t1, row, j8, wp, a);
-        else st_row8(t1, row, j8, wp, b);
     }
+    if (SPLIT && round == 0) tmem_wait_st();
 }
 
 // G(q) = s (N_k(q) - N_k(0)) and G'(q) for the points with `need` (CTA-uniform call;
@@ -441,16 +466,20 @@ __device__ void yield_tc(Shared &S, const TcArgs &T, const NcF &nc, float q, boo
                          int warp)
 {
     const TcLayout &L = T.L;
-    const int w = L.wy, wp = L.wpy;
-    const float *y32 = reinterpret_cast<const float *>(S.blob + T.s_y32);
-    const float *B2 = y32 + 2 * w, *c2 = y32 + 3 * w, *v3 = y32 + 4 * w, *b3 = y32 + 5 * w;
+    const int wp = L.wpy;
+    const float2 *Y1 = reinterpret_cast<const float2 *>(S.blob + T.s_y32);            // V1 c1
+    const float4 *Y2 = reinterpret_cast<const float4 *>(Y1 + wp);                     // B2 c2 v3
+    const float *b3 = reinterpret_cast<const float *>(Y2 + wp);
+    const uint32_t lane_base = S.tbase + ((uint32_t)(warp * 32) << 16);
+    const bool any = __any_sync(0xffffffffu, need);          // a warp's rows are written together
     uint8_t *t0 = S.tiles, *t1 = S.tiles + T.tile_bytes;
     const uint32_t a0 = saddr(t0), a1 = saddr(t1), bv = saddr(S.blob + T.s_slot);
     constexpr int ROUNDS = SPLIT ? 2 : 1;
     slot_wait(S, T);                     // V2 in the weight slot
     for (int r = 0; r < ROUNDS; ++r) {
         if (r > 0) wait_mma(S, T);
-        if (need) yield_l1<SPLIT>(y32, w, wp, q, r, t0, t1, tid);
+        if (any) yield_l1<SPLIT>(Y1, wp, q, r, t0, t1, tid, lane_base + (uint32_t)(2 * wp));
+        tc_before();
         fence_async_smem();
         __syncthreads();
         if (tid == 0) {
@@ -467,8 +496,7 @@ __device__ void yield_tc(Shared &S, const TcArgs &T, const NcF &nc, float q, boo
     wait_mma(S, T);
     tc_after();
     float n0 = 0.0f, n1 = 0.0f;
-    if (__any_sync(0xffffffffu, need)) {
-        const uint32_t lane_base = S.tbase + ((uint32_t)(warp * 32) << 16);
+    if (any) {
         for (int k0 = 0; k0 < wp; k0 += 16) {
             float hS[16], hT[16];
             tmem_ld16(lane_base + (uint32_t)k0, hS);
@@ -476,14 +504,11 @@ __device__ void yield_tc(Shared &S, const TcArgs &T, const NcF &nc, float q, boo
             tmem_wait_ld();
 #pragma unroll
             for (int kk = 0; kk < 16; ++kk) {
-                const int k = k0 + kk;
-                if (k < w) {
-                    const float bk = B2[k];
-                    float spv, sg;
-                    sp_sig_fast(hS[kk] + c2[k] + bk * q, spv, sg);
-                    n0 += v3[k] * spv;
-                    n1 += v3[k] * sg * (hT[kk] + bk);
-                }
+                const float4 c = Y2[k0 + kk];
+                float spv, sg;
+                sp_sig_fast(hS[kk] + c.y + c.x * q, spv, sg);
+                n0 += c.z * spv;
+                n1 += c.z * sg * (hT[kk] + c.x);
             }
         }
     }
@@ -497,7 +522,8 @@ template <int DIM, bool SPLIT>
 __global__ void __launch_bounds__(kTcThreads, 1) asm_tc_kernel(AsmArgs A, TcArgs T)
 {
     using G_ = Geo<DIM>;
-    constexpr int NEN = G_::NEN, NQ = G_::NQ, NDOF = G_::NDOF, EPW = G_::EPW, EPR = G_::EPR;
+    using R_ = rows::Rec<DIM>;
+    constexpr int NEN = G_::NEN, NQ = G_::NQ, NDOF = G_::NDOF, EPW = G_::EPW;
     extern __shared__ __align__(1024) uint8_t tc_smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     Shared S;
@@ -512,11 +538,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) asm_tc_kernel(AsmArgs A, TcArgs
     float *ws = reinterpret_cast<float *>(tc_smem + T.warp_off) + warp * T.warp_floats;
     float *sX = ws;                                  // [EPW][NEN][DIM]
     float *sD = sX + EPW * NEN * DIM;                // [EPW][NEN][NDOF]
-    float *sRec = sD + EPW * NEN * NDOF;             // [32][Q_REC]
-    float *sVec = reinterpret_cast<float *>(S.tiles) + warp * (EPR * NQ * NEN * V_REC);   // row mode (tiles reused)
+    float *sRef = reinterpret_cast<float *>(tc_smem + T.warp_off) + 4 * T.warp_floats;      // [NQ][NEN][4]
+    float *sRec = reinterpret_cast<float *>(S.tiles) + warp * (32 * R_::SIZE);   // records (the tiles' place)
     const MatF m = to_f(A.mat);
     const NcF nc = ncf(A.netc[0]);
 
+    ref_table<DIM>(sRef, tid, kTcThreads);
     if (tid == 0) {
         mbar_init(S.bar, 1);
         mbar_init(S.bar + 1, 1);
@@ -561,12 +588,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) asm_tc_kernel(AsmArgs A, TcArgs
         const int el = lane / NQ, q = lane % NQ;
         const int64_t e_me = e0 + el;
         const bool valid = e_me < A.n_elems;
-        float *rec = sRec + lane * Q_REC;
-        float F[3][3], H[3][3], phi, g[3], x[3], Jdet;
-        qp_kinematics<DIM>(sX, sD, el, q, rec, F, H, phi, g, x, Jdet);
+        float F[DIM][DIM], Ji[DIM][DIM], gx[DIM], phi, x[3], det;
+        qp_kinematics<DIM>(sX, sD, sRef + q * NEN * 4, el, F, Ji, gx, phi, x, det);
+        const float Jdet = 1.0f + x[2];
         float Tm[3][3], T2[3][6], y[3];
         input_map(m, x, Jdet, Tm, T2, y);
-        // every warp has left the previous batch's row mode (its vectors share the tiles)
+        // every warp has left the previous batch's row mode (its records share the tiles)
         if (__syncthreads_or(!S.ok)) break;
         // ================= energy network (tensor cores) =================
         float o10[10];
@@ -675,19 +702,29 @@ __global__ void __launch_bounds__(kTcThreads, 1) asm_tc_kernel(AsmArgs A, TcArgs
         if (__syncthreads_or(!S.ok)) break;
         // ================= qp mode: history, stress and records =================
         if (valid) {
-            atomicAdd(A.counters + 2, n_eval);
             if (A.kappa_new)
                 A.kappa_new[e_me * NQ + q] = frozen ? __ldg(A.kappa_fixed + e_me * NQ + q)
                                              : loading ? fmax(kn_d, (double)kappa) : kn_d;
             if (A.loading) A.loading[e_me * NQ + q] = loading ? 1 : 0;
             if (fail) atomicAdd(A.counters, 1);
-            if (loading) atomicAdd(A.counters + 1, 1);
         }
-        stress_records(m, F, x, g, phi, Jdet, ps, ph, kappa, loading, Gp, dr, valid, rec);
-        // every warp is done with the tiles (the last product completed) before the row
-        // mode writes its vectors over them
-        __syncthreads();
-        row_mode<DIM>(A, m, sRec, sVec, e0, lane);
+        {
+            const int n = __reduce_add_sync(0xffffffffu, valid ? n_eval : 0);
+            const unsigned ld = __ballot_sync(0xffffffffu, valid && loading);
+            if (lane == 0) {
+                if (n) atomicAdd(A.counters + 2, n);
+                if (ld) atomicAdd(A.counters + 1, __popc(ld));
+            }
+        }
+        // the records take the tiles' place (the last product completed before the
+        // __syncthreads_or above)
+        const float fd = kappa > m.kappa_d ? expf(-m.eta_d * (kappa - m.kappa_d)) : 1.0f;
+        rows::point_record<float, DIM>(m, F, Ji, gx, x, phi, valid ? det : 0.0f, ps, ph, kappa, fd, loading, Gp, dr,
+                                       A.tangent != 0, sRec + lane * R_::SIZE);
+        __syncwarp();
+        for (int u = 0; u < 4; ++u)
+            rows::add_rows<float, DIM>(A, sRec + u * 8 * R_::SIZE, sRef, e0 + u * (8 / NQ), lane);
+        __syncwarp();
     }
     slot_wait(S, T);                     // no copy into shared memory outlives the CTA
     tc_before();
@@ -717,29 +754,32 @@ __global__ void tc_blob_kernel(const float *pe, int we, const float *py, int wy,
                     *w3 = b2 + we, *a3 = w3 + we;
         put(L.off_w2f, L.wpe, we, W2, false);
         put(L.off_w2r, L.wpe, we, W2, true);
-        float *e = reinterpret_cast<float *>(blob + L.off_e32);
-        for (int i = t0; i < 3 * we; i += stride) e[i] = W1[i];
-        for (int i = t0; i < we; i += stride) e[3 * we + i] = b1[i];
-        for (int i = t0; i < 3 * we; i += stride) e[4 * we + i] = A2[i];
+        // padded units stay zero (the blob is cleared first)
+        float *e = reinterpret_cast<float *>(blob + L.off_e32), *e2 = e + 4 * L.wpe, *e3 = e2 + 4 * L.wpe;
         for (int i = t0; i < we; i += stride) {
-            e[7 * we + i] = b2[i];
-            e[8 * we + i] = w3[i];
+            for (int c = 0; c < 3; ++c) {
+                e[4 * i + c] = W1[3 * i + c];
+                e2[4 * i + c] = A2[3 * i + c];
+            }
+            e[4 * i + 3] = b1[i];
+            e2[4 * i + 3] = b2[i];
+            e3[i] = w3[i];
         }
-        for (int i = t0; i < 3; i += stride) e[9 * we + i] = a3[i];
+        for (int i = t0; i < 3; i += stride) e3[L.wpe + i] = a3[i];
     }
     if (wy > 0) {
         const float *V1 = py, *c1 = V1 + wy, *V2 = c1 + wy, *B2 = V2 + wy * wy, *c2 = B2 + wy, *v3 = c2 + wy,
                     *b3 = v3 + wy;
         put(L.off_v2f, L.wpy, wy, V2, false);
-        float *f = reinterpret_cast<float *>(blob + L.off_y32);
+        float *f = reinterpret_cast<float *>(blob + L.off_y32), *f2 = f + 2 * L.wpy;
         for (int i = t0; i < wy; i += stride) {
-            f[i] = V1[i];
-            f[wy + i] = c1[i];
-            f[2 * wy + i] = B2[i];
-            f[3 * wy + i] = c2[i];
-            f[4 * wy + i] = v3[i];
+            f[2 * i] = V1[i];
+            f[2 * i + 1] = c1[i];
+            f2[4 * i] = B2[i];
+            f2[4 * i + 1] = c2[i];
+            f2[4 * i + 2] = v3[i];
         }
-        if (t0 == 0) f[5 * wy] = b3[0];
+        if (t0 == 0) f2[4 * L.wpy] = b3[0];
     }
 }
 
@@ -764,9 +804,9 @@ TcLayout tc_layout(int we, int wy, bool split)
     L.off_v2f = off;
     off += parts * 2 * L.wpy * L.wpy;
     L.off_e32 = off;
-    off += ((9 * we + 3) * 4 + 15) / 16 * 16;
+    off += (9 * L.wpe + 4) * 4;
     L.off_y32 = off;
-    off += ((5 * wy + 1) * 4 + 15) / 16 * 16;
+    off += (6 * L.wpy + 4) * 4;
     L.bytes = off;
     return L;
 }
@@ -791,8 +831,10 @@ cudaError_t launch_tc_t(const AsmArgs &a, const TcLaunch &c, cudaStream_t s)
     T.tol_r = SPLIT ? 4e-5f : 4e-3f;
     T.tol_br = SPLIT ? 2e-5f : 2e-3f;
     const int wpmax = c.L.wpe > c.L.wpy ? c.L.wpe : c.L.wpy;
-    // tensor memory: four energy columns of width wp (or two yield columns), a power of two >= 32
-    int need_cols = 4 * c.L.wpe > 2 * c.L.wpy ? 4 * c.L.wpe : 2 * c.L.wpy;
+    // tensor memory: four energy columns of width wp (or two yield columns and, split, the kept
+    // operand), a power of two >= 32
+    const int ycols = (SPLIT ? 3 : 2) * c.L.wpy;
+    const int need_cols = 4 * c.L.wpe > ycols ? 4 * c.L.wpe : ycols;
     int ncols = 32;
     while (ncols < need_cols) ncols *= 2;
     T.ncols = ncols;
@@ -811,17 +853,17 @@ cudaError_t launch_tc_t(const AsmArgs &a, const TcLaunch &c, cudaStream_t s)
     T.s_slot = T.fwd_bytes;
     T.s_e32 = T.s_slot + T.slot_bytes;
     T.s_y32 = T.s_e32 + (c.L.off_y32 - c.L.off_e32);
-    // shared memory: weights | two operand tiles (also the row-mode vectors) | per-warp scratch | barriers
+    // shared memory: weights | two operand tiles (then the points' records) | per-warp nodes | reference table | barriers
     size_t off = ((size_t)(T.s_e32 + T.vec_bytes) + 1023) / 1024 * 1024;
     T.tiles_off = (int)off;
     T.tile_bytes = 128 * (wpmax > 0 ? wpmax : 16) * 2;
-    const size_t vec_bytes = (size_t)4 * G_::EPR * G_::NQ * G_::NEN * V_REC * sizeof(float);
+    const size_t rec_bytes = (size_t)128 * rows::Rec<DIM>::SIZE * sizeof(float);
     size_t tiles = 2 * (size_t)T.tile_bytes;
-    if (tiles < vec_bytes) tiles = vec_bytes;
+    if (tiles < rec_bytes) tiles = rec_bytes;
     off += (tiles + 1023) / 1024 * 1024;
     T.warp_off = (int)off;
-    T.warp_floats = G_::EPW * G_::NEN * (DIM + G_::NDOF) + 32 * Q_REC;
-    off += (size_t)4 * T.warp_floats * sizeof(float);
+    T.warp_floats = G_::EPW * G_::NEN * (DIM + G_::NDOF);
+    off += (size_t)(4 * T.warp_floats + G_::NQ * G_::NEN * 4) * sizeof(float);
     off = (off + 15) / 16 * 16;
     T.bar_off = (int)off;
     off += 32;

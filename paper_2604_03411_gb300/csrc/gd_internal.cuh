@@ -104,7 +104,8 @@ struct Checkpoint {
 // blob that every CTA copies into shared memory: the layer-2 tiles of both networks
 // in the canonical K-major BF16 layout (energy W2 for the forward columns, W2^T for
 // the reverse column, yield V2; with split operands each tile is followed by its
-// residual tile), then FP32 vectors (energy W1 b1 A2 b2 w3 a3, yield V1 c1 B2 c2 v3 b3).
+// residual tile), then FP32 vectors per unit, padded with zeros to the tile width (energy
+// (W1 b1) and (A2 b2) as float4, w3, a3; yield (V1 c1) as float2, (B2 c2 v3 0) as float4, b3).
 struct TcLayout {
     int we = 0, wy = 0;          // widths (0: no network)
     int wpe = 0, wpy = 0;        // widths padded to 16
