@@ -90,6 +90,7 @@ struct AdjArgs {
     const NetConst *netc;
     MatConst mat;
     int mode;
+    int split;                 // shares (warps) per batch of 32 points; the launcher sets it
 };
 
 // a stored state of the load path (for the adjoint's recomputation)
