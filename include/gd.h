@@ -149,7 +149,9 @@ typedef struct gd_options {
                                   preconditioner M^-1 = D^-1 + P (P^T K P)^-1 P^T (D the
                                   node-block diagonal, P constants and rigid rotations on
                                   aggregates of the node graph); default 1536, at most 3072,
-                                  0 = node-block Jacobi only.  The preconditioner changes the
+                                  0 = node-block Jacobi only.  Systems of at most min(coarse,
+                                  1024) dofs take every free dof as a coarse unknown and
+                                  M^-1 = (P^T K P)^-1 alone.  The preconditioner changes the
                                   iteration count, not the solution.  A batch with a coarse
                                   level (aggregates never span two specimens) solves its
                                   union system in one recurrence instead of per-specimen

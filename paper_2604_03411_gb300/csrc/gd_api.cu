@@ -292,6 +292,14 @@ gd_status norms(gd::Handle &H, const double *R, NormPair &out)
 // that computed it.  kind: the Newton tangent, its transpose (adjoint), or a
 // caller's matrix (always recomputed, and not kept).
 constexpr int kCoarseReuse = 8;
+// Systems of up to kCoarseFull dofs take all of them as coarse unknowns, so that M^-1 is the
+// FP32 inverse of a recent matrix of the path.  It is recomputed when a solve needs more
+// iterations than an inversion is worth.  Measured (gd_solve, inversion included, and load
+// paths with gradient of 10 steps): 243 dofs 744 -> 304 us and 48 -> 27 ms, 504 dofs 832 -> 593
+// us and 55 -> 29 ms (429 dofs), 864 dofs in 3D 1,526 -> 1,119 us.  The inversion grows by
+// 16 rows at a time and its share of a single solve passes the saved iterations near 1,000 dofs.
+constexpr int kCoarseFull = 1024;
+constexpr int kFullIters = 16;
 enum MatKind { kTangent = 0, kTransposed = 1, kCallerMatrix = 2 };
 
 // FP64-vector GMRES(gmres_m) on `vals` (the handle's precision: FP64 values, or FP32
@@ -398,7 +406,7 @@ gd_status krylov(gd::Handle &H, const void *vals, const double *b, double *x, in
             H.coarse_rate = rate;
         } else {
             ++H.coarse_age;
-            if (rate < 0.7 * H.coarse_rate) H.coarse_age = -1;
+            if (H.coarse.full ? iters > kFullIters : rate < 0.7 * H.coarse_rate) H.coarse_age = -1;
         }
     }
     if (kout[2] != 0.0 && !(kout[2] != 2.0 && std::isfinite(rel) && rel <= std::max(accept, rtol))) {
@@ -1866,6 +1874,9 @@ static gd_status create_impl(int32_t n_spec, const gd_mesh *meshes, const gd_icn
         std::vector<int32_t> agg, coff;
         std::vector<float> Pc;
         int target = (int)std::max<int64_t>(4, (NN * C.nm + o.coarse - 1) / o.coarse);
+        // small systems: one aggregate per node (its basis: the node's free dofs)
+        C.full = n_dofs <= std::min<int64_t>(o.coarse, kCoarseFull);
+        if (C.full) target = 1;
         int32_t na = 0;
         for (int tries = 0; tries < 8; ++tries) {
             na = gd::coarse_aggregate(NN, ndof, H.h_rowptr, H.h_colidx, target, agg);

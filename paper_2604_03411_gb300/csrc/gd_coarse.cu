@@ -12,7 +12,9 @@
 // these columns, the Galerkin coarse matrix Ac = P^T A P is assembled from the
 // current tangent and inverted densely, and the preconditioner becomes
 //   M^-1 = D^-1 + P Ac^-1 P^T      (D: node-block diagonal of A),
-// the additive two-level Schwarz form.  The paper solves every Newton system by
+// the additive two-level Schwarz form.  Small systems (at most 1,024 dofs) take one
+// aggregate per node: the coarse unknowns are then all free dofs and M^-1 is Ac^-1
+// alone, the FP32 inverse of a recent matrix of the path.  The paper solves every Newton system by
 // a sparse LU factorisation (Sec. 3.2); this preconditioner only changes how
 // fast the iterative replacement converges, not what it converges to.
 //
@@ -553,7 +555,9 @@ cudaError_t coarse_setup(const CoarseSpace &cs, int ndof, int64_t n_nodes, const
     int ncv = nc;
     int *st = cs.status;
     void *args[] = {(void *)&Ac, (void *)&X, (void *)&ncv, (void *)&st};
-    return cudaLaunchCooperativeKernel(fn, dim3(num_sms), dim3(kGjThreads), args, smem, s);
+    // a panel of rows per CTA at least: CTAs without rows only lengthen the barriers
+    const int np = (nc + kGjRows - 1) / kGjRows;
+    return cudaLaunchCooperativeKernel(fn, dim3(np < num_sms ? np : num_sms), dim3(kGjThreads), args, smem, s);
 }
 
 }  // namespace gd

@@ -169,6 +169,7 @@ struct CoarseSpace {
     int nm = 0;                   // basis slots per aggregate: ndof constants + rotations (4 in 2D, 7 in 3D)
     int n_agg = 0;
     int nc = 0;                   // coarse unknowns (the kept basis columns of all aggregates)
+    bool full = false;            // one aggregate per node: the coarse unknowns are all free dofs
     int32_t *agg = nullptr;       // [n_nodes] aggregate of every node
     int32_t *coff = nullptr;      // [n_agg + 1] first coarse unknown of every aggregate
     int32_t *node_co = nullptr;   // [n_nodes] 8 x first coarse unknown + count of the node's aggregate

@@ -27,7 +27,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kCluster = 16;          // CTAs of the largest cluster
-constexpr int kClusterWant = 16;      // systems that want up to this many CTAs run on one cluster
+constexpr int kClusterWant = 32;      // systems that want up to this many CTAs run on one cluster
 
 template <class V, class T>
 struct KArgs {
@@ -58,6 +58,7 @@ struct KArgs {
     const float *c_X32;
     T *c_rc, *c_cc;
     const int *c_status;
+    int c_full;               // 1: the coarse unknowns are all free dofs: M^-1 = P Ac^-1 P^T alone
     int c_xs;                 // 1: each CTA keeps its rows of the inverse in shared memory
     int cluster;              // 1: the grid is one cluster (its hardware barrier serves as the grid's)
 };
@@ -513,6 +514,10 @@ __global__ void __launch_bounds__(kThreads, std::is_same<T, float>::value ? 4 : 
     // the product reads them.  Skipped when the inversion reported a zero pivot.
     bool co = false;
     if constexpr (CO) co = __ldcg(A.c_status) == 0;
+    // With every free dof a coarse unknown Ac^-1 is the inverse itself (to FP32) and the
+    // node-block part is left out.
+    bool jac = true;
+    if constexpr (CO) jac = !(co && A.c_full);
     T *rc0 = nullptr, *rc1 = nullptr, *cc = nullptr;
     if constexpr (CO) {
         rc0 = A.c_rc;
@@ -646,7 +651,7 @@ __global__ void __launch_bounds__(kThreads, std::is_same<T, float>::value ? 4 : 
             const int32_t row = nd * NDOF + sub;
             const bool fx = own ? A.fixed[row] != 0 : true;
             const T bv = (own && !fx) ? (T)A.b[row] : T(0);
-            const T yv = node_apply<NDOF, T>(A.binv, nd, node_ok, sub, nbase, bv, fx);
+            const T yv = jac ? node_apply<NDOF, T>(A.binv, nd, node_ok, sub, nbase, bv, fx) : T(0);
             if (co) restrict_node(ps, nd, node_ok, bv, rc0);
             if (own) {
                 r[row] = bv;
@@ -720,7 +725,7 @@ __global__ void __launch_bounds__(kThreads, std::is_same<T, float>::value ? 4 : 
                         v[row] = vn;
                         s1.add(rh[row], vn);
                     }
-                    const T yv = node_apply<NDOF, T>(A.binv, nd, node_ok, sub, nbase, vn, fx);
+                    const T yv = jac ? node_apply<NDOF, T>(A.binv, nd, node_ok, sub, nbase, vn, fx) : T(0);
                     if (co) restrict_node(ps, nd, node_ok, vn, rc0);
                     if (own) y[row] = yv;
                 }
@@ -801,7 +806,7 @@ __global__ void __launch_bounds__(kThreads, std::is_same<T, float>::value ? 4 : 
                         prhr.add(rh[row], rn);
                         prr.add(rn, rn);
                     }
-                    const T wn = node_apply<NDOF, T>(A.binv, nd, node_ok, sub, nbase, rn, fx);
+                    const T wn = jac ? node_apply<NDOF, T>(A.binv, nd, node_ok, sub, nbase, rn, fx) : T(0);
                     if (co) restrict_node(ps, nd, node_ok, rn, rc1);
                     if (own) wv[row] = wn;
                 }
@@ -877,7 +882,7 @@ __global__ void __launch_bounds__(kThreads, std::is_same<T, float>::value ? 4 : 
         const int32_t row = nd * NDOF + sub;
         const bool fx = own ? A.fixed[row] != 0 : true;
         const T xv = own ? xt[row] : T(0);
-        const T xo = node_apply<NDOF, T>(A.binv, nd, node_ok, sub, nbase, xv, fx);
+        const T xo = jac ? node_apply<NDOF, T>(A.binv, nd, node_ok, sub, nbase, xv, fx) : T(0);
         if (co) restrict_node(ps, nd, node_ok, xv, rc0);
         if (own) A.x_out[row] = (double)xo;
     }
@@ -1480,6 +1485,7 @@ cudaError_t solve_t(const KrylovCtx &c, const V *vals, const double *b, double *
         A.c_rc = (T *)cs.rc;
         A.c_cc = (T *)cs.cc;
         A.c_status = cs.status;
+        A.c_full = cs.full;
     }
     // the grid-wide accumulators (2 parities x 5 slots) start at zero
     e = cudaMemsetAsync(c.red, 0, 10 * sizeof(double), c.stream);
@@ -1511,7 +1517,9 @@ cudaError_t solve_t(const KrylovCtx &c, const V *vals, const double *b, double *
         if (want < blocks) blocks = (int)want;
         // Where the CTAs of one cluster suffice the grid is that cluster: its barrier is hardware,
         // the cooperative one an atomic counter in L2 (load path with gradient of the 8x8
-        // square, 7 barriers per iteration on 11 CTAs: 57.4 -> 54.5 ms).
+        // square, 7 barriers per iteration on 11 CTAs: 57.4 -> 54.5 ms).  A system that wants up
+        // to 32 CTAs does two rounds of its coarse rows on 16 (about 1 us more per application)
+        // and saves as much on each of the seven barriers.
         if (want <= kClusterWant && c.blocks >= kCluster) {
             A.cluster = 1;
             blocks = want <= 8 ? 8 : kCluster;
