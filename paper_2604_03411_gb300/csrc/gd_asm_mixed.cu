@@ -9,14 +9,19 @@
 // switches between three lane mappings:
 //   qp mode    lane = quadrature point: kinematics, invariants, energy chain,
 //              stress and the per-point records of the tangent;
-//   unit mode  lane = network unit, one point at a time: both ICNN layers of the
-//              energy network (value, gradient by forward tangents, Hessian by
-//              one reverse sweep through layer 2) and every yield-network
-//              evaluation of the local damage solve, so the per-point iteration
-//              counts cost no divergence;
+//   unit mode  lane = network unit, four points of an element at a time: both ICNN
+//              layers of the energy network (value, gradient by forward tangents,
+//              Hessian by one reverse sweep through layer 2) and every yield-network
+//              evaluation of the local damage solve, whose points iterate together;
 //   row mode   lane = element row (node a, dof i): the row of the consistent
 //              tangent and of the residual, accumulated over the points of one
 //              element and scattered into CSR through the slot map.
+//
+// Instruction fetches bound the kernel (10 of 14 cycles per issued instruction with 190 KB of
+// code, 16 warps per SM in different modes), so each network is in the code once, loops over
+// units and rows stay loops, and the three kinds of yield evaluation share one call.
+// Measured (96 specimens, 690,000 Q4 points, widths 16 to 32, GB300): one point at a time
+// 3.37 ms; four at a time with three copies 3.29, with one copy and loops 1.84.
 //
 // Paper passages: Sec. 3.1f (F, phi_q, grad phi_q, element residual, Table
 // kernel_inputs), Sec. 2.1f (P, Y vector, Y), Sec. 2.2f and Sec. 3.2f Eq. (dd_7_no_nn)
@@ -32,96 +37,158 @@ namespace {
 
 using namespace e32;
 
-// Energy network in unit mode for one point: value, gradient and Hessian of
+// Energy network in unit mode for four points of one element: value, gradient and Hessian of
 // N(x) (Sec. 4.2f ICNN).  Layer 1 and the gradient columns of layer 2 are
 // forward tangents; the second derivative uses the identity
 //   d2N/dx2 = sum_k w3_k sp''(h2_k) g_k g_k^T + sum_j v_j sp''(h1_j) W1_j W1_j^T,
 //   g_k = dh2_k/dx,  v = W2^T (w3 o sp'(h2)),
 // so layer 2 costs 4 forward columns and 1 reverse column per point.
-// Every lane returns the full result.
-__device__ void psi_net_unit(const DevNet &net, const float *x, float *out10, float *buf, int lane)
+// in: [4][4] inputs, out: [4][10] results (shared memory).
+__device__ __forceinline__ void psi_net_unit4(const DevNet &net, const float *in, float *out, float *buf, int lane)
 {
+    constexpr unsigned kAll = 0xffffffffu;
     const int w = net.width;
     const float *W1 = net.pf, *b1 = W1 + 3 * w, *W2 = b1 + w, *A2 = W2 + w * w, *b2 = A2 + 3 * w, *w3 = b2 + w,
                  *a3 = w3 + w;
-    float *sS = buf, *sD0 = buf + w, *sD1 = buf + 2 * w, *sD2 = buf + 3 * w, *sU = buf + 4 * w;
-    float e1[2], W1r[2][3];
+    float4 *sZ = reinterpret_cast<float4 *>(buf);         // [w][kNP]: value, three tangents
+    PVec *sU = reinterpret_cast<PVec *>(buf + 16 * w);        // [w]
+    PVec *sE = sU + w;                                       // [w] sp'' of layer 1 (own units)
+    float x[kNP][3];
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        int j = lane + 32 * t;
-        e1[t] = 0.0f;
-        W1r[t][0] = W1r[t][1] = W1r[t][2] = 0.0f;
+    for (int p = 0; p < kNP; ++p)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) x[p][i] = in[p * 4 + i];
+#pragma unroll 1
+    for (int t = 0; t < kUnits; ++t) {
+        const int j = lane + 32 * t;
         if (j < w) {
-            float a0 = __ldg(W1 + 3 * j), a1 = __ldg(W1 + 3 * j + 1), a2 = __ldg(W1 + 3 * j + 2);
-            float h = __ldg(b1 + j) + a0 * x[0] + a1 * x[1] + a2 * x[2];
-            float sg, spv;
-            sp_sig(h, spv, sg);
-            sS[j] = spv;
-            sD0[j] = sg * a0;
-            sD1[j] = sg * a1;
-            sD2[j] = sg * a2;
-            e1[t] = sg * (1.0f - sg);
-            W1r[t][0] = a0; W1r[t][1] = a1; W1r[t][2] = a2;
-        }
-    }
-    __syncwarp();
-    float acc[10];
+            const float a0 = __ldg(W1 + 3 * j), a1 = __ldg(W1 + 3 * j + 1), a2 = __ldg(W1 + 3 * j + 2), b = __ldg(b1 + j);
+            PVec e1;
 #pragma unroll
-    for (int c = 0; c < 10; ++c) acc[c] = 0.0f;
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        int k = lane + 32 * t;
-        if (k < w) {
-            float h = __ldg(b2 + k), g0 = __ldg(A2 + 3 * k), g1 = __ldg(A2 + 3 * k + 1), g2 = __ldg(A2 + 3 * k + 2);
-            h += g0 * x[0] + g1 * x[1] + g2 * x[2];
-            const float *col = net.W2Tf + k;     // W2[k][j] = W2T[j*w + k]
-            for (int j = 0; j < w; ++j) {
-                float wkj = __ldg(col + j * w);
-                h += wkj * sS[j];
-                g0 += wkj * sD0[j];
-                g1 += wkj * sD1[j];
-                g2 += wkj * sD2[j];
+            for (int p = 0; p < kNP; ++p) {
+                float sg, spv;
+                sp_sig(b + a0 * x[p][0] + a1 * x[p][1] + a2 * x[p][2], spv, sg);
+                sZ[j * kNP + p] = make_float4(spv, sg * a0, sg * a1, sg * a2);
+                e1.v[p] = sg * (1.0f - sg);
             }
-            float sg, spv;
-            sp_sig(h, spv, sg);
-            const float wk = __ldg(w3 + k);
-            float e2 = wk * sg * (1.0f - sg);
-            acc[0] += wk * spv;
-            acc[1] += wk * sg * g0;
-            acc[2] += wk * sg * g1;
-            acc[3] += wk * sg * g2;
-            acc[4] += e2 * g0 * g0;
-            acc[5] += e2 * g0 * g1;
-            acc[6] += e2 * g0 * g2;
-            acc[7] += e2 * g1 * g1;
-            acc[8] += e2 * g1 * g2;
-            acc[9] += e2 * g2 * g2;
-            sU[k] = wk * sg;
+            sE[j] = e1;
         }
     }
     __syncwarp();
+    float acc[kNP][10];
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        int j = lane + 32 * t;
-        if (j < w) {
-            float v = 0.0f;
-            const float *row = W2 + j;          // W2[k][j] at k*w + j
-            for (int k = 0; k < w; ++k) v += __ldg(row + k * w) * sU[k];
-            float c = v * e1[t];
-            acc[4] += c * W1r[t][0] * W1r[t][0];
-            acc[5] += c * W1r[t][0] * W1r[t][1];
-            acc[6] += c * W1r[t][0] * W1r[t][2];
-            acc[7] += c * W1r[t][1] * W1r[t][1];
-            acc[8] += c * W1r[t][1] * W1r[t][2];
-            acc[9] += c * W1r[t][2] * W1r[t][2];
+    for (int p = 0; p < kNP; ++p)
+#pragma unroll
+        for (int c = 0; c < 10; ++c) acc[p][c] = 0.0f;
+#pragma unroll 1
+    for (int t = 0; t < kUnits; ++t) {
+        const int k = lane + 32 * t;
+        if (k < w) {
+            const float c0 = __ldg(A2 + 3 * k), c1 = __ldg(A2 + 3 * k + 1), c2 = __ldg(A2 + 3 * k + 2),
+                        bk = __ldg(b2 + k), wk = __ldg(w3 + k);
+            float h[kNP], g0[kNP], g1[kNP], g2[kNP];
+#pragma unroll
+            for (int p = 0; p < kNP; ++p) {
+                h[p] = bk + c0 * x[p][0] + c1 * x[p][1] + c2 * x[p][2];
+                g0[p] = c0;
+                g1[p] = c1;
+                g2[p] = c2;
+            }
+            const float *col = net.W2Tf + k;     // W2[k][j] = W2T[j*w + k]
+#pragma unroll 2
+            for (int j = 0; j < w; ++j) {
+                const float wkj = __ldg(col + j * w);
+#pragma unroll
+                for (int p = 0; p < kNP; ++p) {
+                    const float4 z = sZ[j * kNP + p];
+                    h[p] += wkj * z.x;
+                    g0[p] += wkj * z.y;
+                    g1[p] += wkj * z.z;
+                    g2[p] += wkj * z.w;
+                }
+            }
+            PVec u;
+#pragma unroll
+            for (int p = 0; p < kNP; ++p) {
+                float sg, spv;
+                sp_sig(h[p], spv, sg);
+                const float e2 = wk * sg * (1.0f - sg);
+                u.v[p] = wk * sg;
+                acc[p][0] += wk * spv;
+                acc[p][1] += wk * sg * g0[p];
+                acc[p][2] += wk * sg * g1[p];
+                acc[p][3] += wk * sg * g2[p];
+                acc[p][4] += e2 * g0[p] * g0[p];
+                acc[p][5] += e2 * g0[p] * g1[p];
+                acc[p][6] += e2 * g0[p] * g2[p];
+                acc[p][7] += e2 * g1[p] * g1[p];
+                acc[p][8] += e2 * g1[p] * g2[p];
+                acc[p][9] += e2 * g2[p] * g2[p];
+            }
+            sU[k] = u;
         }
     }
+    __syncwarp();
+#pragma unroll 1
+    for (int t = 0; t < kUnits; ++t) {
+        const int j = lane + 32 * t;
+        if (j < w) {
+            float v[kNP];
 #pragma unroll
-    for (int c = 0; c < 10; ++c) out10[c] = warp_sum(acc[c]);
-    out10[0] += __ldg(a3) * x[0] + __ldg(a3 + 1) * x[1] + __ldg(a3 + 2) * x[2];
-    out10[1] += __ldg(a3);
-    out10[2] += __ldg(a3 + 1);
-    out10[3] += __ldg(a3 + 2);
+            for (int p = 0; p < kNP; ++p) v[p] = 0.0f;
+            const float *row = W2 + j;          // W2[k][j] at k*w + j
+#pragma unroll 4
+            for (int k = 0; k < w; ++k) {
+                const float wkj = __ldg(row + k * w);
+                const PVec u = sU[k];
+#pragma unroll
+                for (int p = 0; p < kNP; ++p) v[p] += wkj * u.v[p];
+            }
+            const float a0 = __ldg(W1 + 3 * j), a1 = __ldg(W1 + 3 * j + 1), a2 = __ldg(W1 + 3 * j + 2);
+            const PVec e1 = sE[j];
+#pragma unroll
+            for (int p = 0; p < kNP; ++p) {
+                const float c = v[p] * e1.v[p];
+                acc[p][4] += c * a0 * a0;
+                acc[p][5] += c * a0 * a1;
+                acc[p][6] += c * a0 * a2;
+                acc[p][7] += c * a1 * a1;
+                acc[p][8] += c * a1 * a2;
+                acc[p][9] += c * a2 * a2;
+            }
+        }
+    }
+    // Sums over the units.  Each exchange halves the values a lane holds (4 points x 10, 2 x 10,
+    // 10, 5): 45 exchanges for the four points where a butterfly per value takes 200.  The eight
+    // lanes 8 p .. 8 p + 7 end with point p, the upper four of them with values 5..9.
+    float r2[2][10], r1[10], rv[5];
+    const bool h4 = lane & 16, h3 = lane & 8;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int c = 0; c < 10; ++c)
+            r2[i][c] = (h4 ? acc[2 + i][c] : acc[i][c]) + __shfl_xor_sync(kAll, h4 ? acc[i][c] : acc[2 + i][c], 16);
+#pragma unroll
+    for (int c = 0; c < 10; ++c) r1[c] = (h3 ? r2[1][c] : r2[0][c]) + __shfl_xor_sync(kAll, h3 ? r2[0][c] : r2[1][c], 8);
+    const bool up = lane & 4;
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+        rv[c] = (up ? r1[5 + c] : r1[c]) + __shfl_xor_sync(kAll, up ? r1[c] : r1[5 + c], 4);
+        rv[c] += __shfl_xor_sync(kAll, rv[c], 2);
+        rv[c] += __shfl_xor_sync(kAll, rv[c], 1);
+    }
+    if ((lane & 3) == 0) {
+        const int p = lane >> 3;
+        if (!up) {
+            const float s0 = __ldg(a3), s1 = __ldg(a3 + 1), s2 = __ldg(a3 + 2);
+            rv[0] += s0 * in[p * 4] + s1 * in[p * 4 + 1] + s2 * in[p * 4 + 2];
+            rv[1] += s0;
+            rv[2] += s1;
+            rv[3] += s2;
+        }
+#pragma unroll
+        for (int c = 0; c < 5; ++c) out[p * 10 + (up ? 5 : 0) + c] = rv[c];
+    }
     __syncwarp();
 }
 
@@ -130,11 +197,12 @@ template <int DIM>
 __host__ __device__ constexpr int scratch_floats(int wmax)
 {
     using G_ = Geo<DIM>;
-    return G_::EPW * G_::NEN * (DIM + G_::NDOF) + 32 * rows::Rec<DIM>::SIZE + 32 * 4 + 32 * 10 + 5 * wmax;
+    const int rec = 32 * rows::Rec<DIM>::SIZE, unit = unit_floats(wmax);
+    return G_::EPW * G_::NEN * (DIM + G_::NDOF) + (rec > unit ? rec : unit) + 32 * 4 + 32 * 10;
 }
 
 template <int DIM, int KW>
-__global__ void __launch_bounds__(32 * KW) asm_fp32_kernel(AsmArgs A)
+__global__ void __launch_bounds__(32 * KW, (DIM == 2 ? 16 : 12) / KW) asm_fp32_kernel(AsmArgs A)
 {
     using G_ = Geo<DIM>;
     using R_ = rows::Rec<DIM>;
@@ -149,14 +217,15 @@ __global__ void __launch_bounds__(32 * KW) asm_fp32_kernel(AsmArgs A)
     float *ws = smem + warp * scratch;
     float *sX = ws;                                  // [EPW][NEN][DIM]
     float *sD = sX + EPW * NEN * DIM;                // [EPW][NEN][NDOF]
-    float *sRec = sD + EPW * NEN * NDOF;             // [32] records of the points
-    float *sIn = sRec + 32 * R_::SIZE;               // [32][4]: network input x (3), then kappa out
+    float *sIn = sD + EPW * NEN * NDOF;              // [32][4]: network input x (3), then kappa out
     float *sOut = sIn + 32 * 4;                      // [32][10]: N, grad, Hess / local-solve results
-    float *sBuf = sOut + 32 * 10;                    // unit-mode buffers
+    float *sBuf = sOut + 32 * 10;                    // unit-mode buffers, then
+    float *sRec = sBuf;                              // [32] records of the points
     const MatF m = to_f(A.mat);
     ref_table<DIM>(sRef, threadIdx.x, 32 * KW);
     __syncthreads();
 
+    int evals = 0, n_loading = 0;        // the lane's share of the counters
     const int64_t n_batches = (A.n_elems + EPW - 1) / EPW;
     for (int64_t batch = (int64_t)blockIdx.x * KW + warp; batch < n_batches;
          batch += (int64_t)gridDim.x * KW) {
@@ -185,13 +254,11 @@ __global__ void __launch_bounds__(32 * KW) asm_fp32_kernel(AsmArgs A)
 
         // ================= unit mode: energy network =================
         if (m.energy != GD_ENERGY_NEO_HOOKE) {
-            for (int p = 0; p < 32; ++p) {
+#pragma unroll 1
+            for (int p = 0; p < 32; p += 4) {
                 if (e0 + p / NQ >= A.n_elems) break;
-                float y[3] = {sIn[p * 4], sIn[p * 4 + 1], sIn[p * 4 + 2]}, out[10];
-                psi_net_unit(psi_of(A, spec_of(A, e0 + p / NQ)), y, out, sBuf, lane);
-                if (lane == 0)
-#pragma unroll
-                    for (int c = 0; c < 10; ++c) sOut[p * 10 + c] = out[c];
+                const DevNet &net = psi_of(A, spec_of(A, e0 + p / NQ));
+                psi_net_unit4(net, sIn + p * 4, sOut + p * 10, sBuf, lane);
             }
         }
         __syncwarp();
@@ -215,33 +282,29 @@ __global__ void __launch_bounds__(32 * KW) asm_fp32_kernel(AsmArgs A)
             o[4] = 0.0f;
             o[5] = 0.0f;
         } else
-        for (int p = 0; p < 32; ++p) {
-            if (e0 + p / NQ >= A.n_elems) break;
+#pragma unroll 1
+        for (int p4 = 0; p4 < 32; p4 += 4) {
+            if (e0 + p4 / NQ >= A.n_elems) break;
+            const int p = p4 + (lane >> 3);                 // the lane's point
             const float ppe = sIn[p * 4], pphi = sIn[p * 4 + 1], kn = sIn[p * 4 + 2];
-            const int sp = spec_of(A, e0 + p / NQ);
+            const int sp = spec_of(A, e0 + p4 / NQ);
             const DevNet &yn = yld_of(A, sp);
             const NcF ncp = ncf(A.netc[sp]);
             const double kn_d = __ldg(A.kappa_n + e0 * NQ + p);
-            float r, dr, Gp;
-            int n_eval = 1;
-            r_slope(yn, m, ncp, ppe, pphi, kn, r, dr, Gp, sBuf, lane);
-            // loading/unloading decided in FP64: Phi_d(kappa_n) = G(q(kappa_n)) - kappa_n > 0
-            const double phi_trial = (double)(r + kn) - kn_d;
-            float kappa = kn, fail = 0.0f, loading = 0.0f;
-            if (phi_trial > 0.0) {
-                loading = 1.0f;
-                const float kg = A.kappa_guess ? (float)__ldg(A.kappa_guess + e0 * NQ + p) : kn;
-                if (!bracketed_newton(yn, m, ncp, ppe, pphi, kn, kg, kappa, r, dr, Gp, n_eval, sBuf, lane)) fail = 1.0f;
-            }
-            if (lane == 0) {
+            const float kg = A.kappa_guess ? (float)__ldg(A.kappa_guess + e0 * NQ + p) : kn;
+            float kappa, dr, Gp;
+            bool loading;
+            int n_eval;
+            const bool ok = local_update4(yn, m, ncp, ppe, pphi, kn, kn_d, kg, kappa, loading, dr, Gp, n_eval, sBuf, lane);
+            if ((lane & 7) == 0) {
                 float *o = sOut + p * 10;
-                if (e0 + p / NQ < A.n_elems) atomicAdd(A.counters + 2, n_eval);
+                evals += n_eval;
                 o[0] = kappa;
-                o[5] = loading > 0.5f ? 0.0f : 1.0f;   // elastic: keep the FP64 history exactly
-                o[1] = loading;
+                o[1] = loading ? 1.0f : 0.0f;
                 o[2] = Gp;
                 o[3] = dr;
-                o[4] = fail;
+                o[4] = ok ? 0.0f : 1.0f;
+                o[5] = loading ? 0.0f : 1.0f;   // elastic: keep the FP64 history exactly
             }
         }
         __syncwarp();
@@ -259,7 +322,7 @@ __global__ void __launch_bounds__(32 * KW) asm_fp32_kernel(AsmArgs A)
                 }
                 if (A.loading) A.loading[e_me * NQ + q] = loading ? 1 : 0;
                 if (o[4] > 0.5f) atomicAdd(A.counters, 1);
-                if (loading) atomicAdd(A.counters + 1, 1);
+                if (loading) ++n_loading;
             }
             const float fd = kappa > m.kappa_d ? expf(-m.eta_d * (kappa - m.kappa_d)) : 1.0f;
             rows::point_record<float, DIM>(m, F, Ji, gx, x, phi, valid ? det : 0.0f, ps, ph, kappa, fd, loading, o[2],
@@ -268,8 +331,15 @@ __global__ void __launch_bounds__(32 * KW) asm_fp32_kernel(AsmArgs A)
         __syncwarp();
 
         // ================= row mode: element residual and tangent =================
+#pragma unroll 1
         for (int u = 0; u < 4; ++u) rows::add_rows<float, DIM>(A, sRec + u * 8 * R_::SIZE, sRef, e0 + u * (8 / NQ), lane);
         __syncwarp();
+    }
+    evals = __reduce_add_sync(0xffffffffu, evals);
+    n_loading = __reduce_add_sync(0xffffffffu, n_loading);
+    if (lane == 0) {
+        if (evals) atomicAdd(A.counters + 2, evals);
+        if (n_loading) atomicAdd(A.counters + 1, n_loading);
     }
 }
 

@@ -119,118 +119,192 @@ __device__ __forceinline__ int sym6(int i, int j)
     return a == 0 ? b : (a == 1 ? 2 + b : 5);
 }
 
-// Yield network value and slope in unit mode: G(q) = s (N_k(q) - N_k(0)),
-// G' = s N_k'(q) (Eq. (Gq_NN)); width 0 is the identity G(q) = q.
-static __device__ void yield_unit(const DevNet &net, const NcF &nc, float q, float &G, float &Gp, float *buf, int lane)
+// Unit mode evaluates the networks of kNP points of one element at once (lane = network unit,
+// up to two units per lane), so that a weight load serves four points and four independent
+// chains hide each other's latency.  (Two groups of 16 lanes for narrow networks were slower:
+// the second copy of the code cost more in instruction fetches than half-empty warps, 2.23
+// against 1.84 ms on 96 specimens of widths 16 to 32.)
+constexpr int kNP = 4;
+constexpr int kUnits = 2;                     // units per lane
+struct alignas(16) PVec {
+    float v[kNP];
+};
+// floats of a warp's unit-mode buffer
+__host__ __device__ constexpr int unit_floats(int wmax) { return 24 * wmax; }
+
+// Yield network value and slope of four points in unit mode: G(q) = s (N_k(q) - N_k(0)),
+// G' = s N_k'(q) (Eq. (Gq_NN)).  Lane l holds the argument of point l / 8 and receives
+// its G and G'.  Every lane calls it.
+static __device__ __forceinline__ void yield_unit4(const DevNet &net, const NcF &nc, float q, float &G, float &Gp,
+                                                   float *buf, int lane)
 {
+    constexpr unsigned kAll = 0xffffffffu;
     const int w = net.width;
-    if (w == 0) {
-        G = q;
-        Gp = 1.0f;
-        return;
-    }
     const float *V1 = net.pf, *c1 = V1 + w, *V2 = c1 + w, *B2 = V2 + w * w, *c2 = B2 + w, *v3 = c2 + w,
                  *b3 = v3 + w;
-    float *sS = buf, *sT = buf + w;
+    PVec *sS = reinterpret_cast<PVec *>(buf), *sT = sS + w;
+    float qp[kNP];
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        int j = lane + 32 * t;
+    for (int p = 0; p < kNP; ++p) qp[p] = __shfl_sync(kAll, q, 8 * p);
+#pragma unroll 1
+    for (int t = 0; t < kUnits; ++t) {
+        const int j = lane + 32 * t;
         if (j < w) {
-            float a = __ldg(V1 + j);
-            float h = __ldg(c1 + j) + a * q;
-            float spv, sg;
-            sp_sig(h, spv, sg);
-            sS[j] = spv;
-            sT[j] = sg * a;
+            const float a = __ldg(V1 + j), b = __ldg(c1 + j);
+            PVec s, d;
+#pragma unroll
+            for (int p = 0; p < kNP; ++p) {
+                float sg;
+                sp_sig(b + a * qp[p], s.v[p], sg);
+                d.v[p] = sg * a;
+            }
+            sS[j] = s;
+            sT[j] = d;
         }
     }
     __syncwarp();
-    float n0 = 0.0f, n1 = 0.0f;
+    float n0[kNP], n1[kNP];
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        int k = lane + 32 * t;
+    for (int p = 0; p < kNP; ++p) n0[p] = n1[p] = 0.0f;
+#pragma unroll 1
+    for (int t = 0; t < kUnits; ++t) {
+        const int k = lane + 32 * t;
         if (k < w) {
-            float g = __ldg(B2 + k);
-            float h = __ldg(c2 + k) + g * q;
-            const float *col = net.W2Tf + k;
-            for (int j = 0; j < w; ++j) {
-                float wkj = __ldg(col + j * w);
-                h += wkj * sS[j];
-                g += wkj * sT[j];
+            const float bk = __ldg(B2 + k), ck = __ldg(c2 + k), vk = __ldg(v3 + k);
+            float h[kNP], d[kNP];
+#pragma unroll
+            for (int p = 0; p < kNP; ++p) {
+                h[p] = ck + bk * qp[p];
+                d[p] = bk;
             }
-            float vk = __ldg(v3 + k);
-            float spv, sg;
-            sp_sig(h, spv, sg);
-            n0 += vk * spv;
-            n1 += vk * sg * g;
+            const float *col = net.W2Tf + k;
+#pragma unroll 2
+            for (int j = 0; j < w; ++j) {
+                const float wkj = __ldg(col + j * w);
+                const PVec s = sS[j], e = sT[j];
+#pragma unroll
+                for (int p = 0; p < kNP; ++p) {
+                    h[p] += wkj * s.v[p];
+                    d[p] += wkj * e.v[p];
+                }
+            }
+#pragma unroll
+            for (int p = 0; p < kNP; ++p) {
+                float spv, sg;
+                sp_sig(h[p], spv, sg);
+                n0[p] += vk * spv;
+                n1[p] += vk * sg * d[p];
+            }
         }
     }
-    n0 = warp_sum(n0);
-    n1 = warp_sum(n1);
-    float b = __ldg(b3);
-    G = nc.y_s * (n0 + b * q - nc.y_N0);
-    Gp = nc.y_s * (n1 + b);
+    // the eight lanes of a point end with its two sums
+    float a2[2], d2[2];
+    const bool h4 = lane & 16, h3 = lane & 8;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        a2[i] = (h4 ? n0[2 + i] : n0[i]) + __shfl_xor_sync(kAll, h4 ? n0[i] : n0[2 + i], 16);
+        d2[i] = (h4 ? n1[2 + i] : n1[i]) + __shfl_xor_sync(kAll, h4 ? n1[i] : n1[2 + i], 16);
+    }
+    float a = (h3 ? a2[1] : a2[0]) + __shfl_xor_sync(kAll, h3 ? a2[0] : a2[1], 8);
+    float d = (h3 ? d2[1] : d2[0]) + __shfl_xor_sync(kAll, h3 ? d2[0] : d2[1], 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(kAll, a, o);
+        d += __shfl_xor_sync(kAll, d, o);
+    }
+    const float b = __ldg(b3);
+    G = nc.y_s * (a + b * q - nc.y_N0);
+    Gp = nc.y_s * (d + b);
     __syncwarp();
 }
 
-// r(kappa) = G(q(kappa)) - kappa and dr/dkappa (Eq. (potential_function)),
-// q = psi_e + qcoef (phi - kappa) / f_d(kappa) (Eq. (ostwald_potential)).
-__device__ __forceinline__ void r_slope(const DevNet &yld, const MatF &m, const NcF &nc, float pe, float phi,
-                                        float kappa, float &r, float &dr, float &Gp, float *buf, int lane)
+// r(kappa) = G(q(kappa)) - kappa and dr/dkappa (Eq. (potential_function)) of four points,
+// q = psi_e + qcoef (phi - kappa) / f_d(kappa) (Eq. (ostwald_potential)); lane l holds
+// point l / 8.  Width 0 is the identity G(q) = q.
+__device__ __forceinline__ void r_slope4(const DevNet &yld, const MatF &m, const NcF &nc, float pe, float phi,
+                                         float kappa, float &r, float &dr, float &Gp, float *buf, int lane)
 {
-    bool dmg = kappa > m.kappa_d;
-    float f = dmg ? expf(-m.eta_d * (kappa - m.kappa_d)) : 1.0f;
-    float q = pe + m.qcoef * (phi - kappa) / f;
-    float dq = m.qcoef * (-1.0f / f + (dmg ? (phi - kappa) * m.eta_d / f : 0.0f));
+    const bool dmg = kappa > m.kappa_d;
+    const float f = dmg ? expf(-m.eta_d * (kappa - m.kappa_d)) : 1.0f;
+    const float q = pe + m.qcoef * (phi - kappa) / f;
+    const float dq = m.qcoef * (-1.0f / f + (dmg ? (phi - kappa) * m.eta_d / f : 0.0f));
     float G;
-    yield_unit(yld, nc, q, G, Gp, buf, lane);
+    if (yld.width == 0) {
+        G = q;
+        Gp = 1.0f;
+    } else {
+        yield_unit4(yld, nc, q, G, Gp, buf, lane);
+    }
     r = G - kappa;
     dr = Gp * dq - 1.0f;
 }
 
-// Local damage update in unit mode (Eq. (dd_7_no_nn)): the smallest root above
-// kappa_n of r(kappa) = G(q(kappa)) - kappa, entered with kappa = kappa_n and (r, dr,
-// Gp) evaluated there (r > 0: the point is loading) and a warm start kg (used when
-// above kappa_n).  On return kappa is the root to |r| <= 2e-6 max(1, kappa) (or a
-// bracket of 4 FP32 ulps), r, dr and Gp are evaluated there, n_eval counts the
-// evaluations; false when local_max iterations did not reach it.  Every lane takes
-// the same path (r and dr are warp-reduced).
-// step_test: also stop when the next Newton correction |r / r'| is within the tolerance
-// and either the root is bracketed within 1e-2 relative or the iteration is converging
-// from one side (the last step a Newton step at least twice as long).  For a starting
-// point that FP64 refines: near full damage r' grows like 1 / f_d and |r| cannot get
-// below its FP32 rounding; far past the root, where f_d underflows, r' is huge, so a
-// wide bracket never qualifies.
-__device__ __forceinline__ bool bracketed_newton(const DevNet &yn, const MatF &m, const NcF &ncp, float pe, float phi,
-                                                 float kn, float kg, float &kappa, float &r, float &dr, float &Gp,
-                                                 int &n_eval, float *buf, int lane, bool step_test = false)
+// Local damage update of four points in unit mode (Eq. (dd_7_no_nn)), lane l holding point
+// l / 8.  The trial value decides loading in FP64 (Phi_d(kappa_n) = G(q(kappa_n)) - kappa_n >
+// 0 with the FP64 kappa_n kn_d); a loading point's kappa is the smallest root above kappa_n of
+// r(kappa) = G(q(kappa)) - kappa, searched from the warm start kg when that lies above
+// kappa_n, to |r| <= 2e-6 max(1, kappa) (or a bracket of 4 FP32 ulps).  On return r' = dr and
+// G' = Gp are those at kappa, n_eval counts the point's evaluations; false when local_max
+// iterations did not reach the root.  The points iterate together until the last one is
+// done, a finished point keeps its values; trial, warm start and iterations share one
+// evaluation in the code (three inlined copies cost instruction fetches).
+__device__ __forceinline__ bool local_update4(const DevNet &yn, const MatF &m, const NcF &ncp, float pe, float phi,
+                                              float kn, double kn_d, float kg, float &kappa, bool &loading,
+                                              float &dr, float &Gp, int &n_eval, float *buf, int lane)
 {
     // Newton iteration on r(kappa) = G(q(kappa)) - kappa from kappa_n (r > 0 there)
     // or from the warm-start guess, bracketing lazily: lo keeps the last point with
     // r > 0; once a point with r <= 0 is met it becomes hi and the iteration turns
     // into the safeguarded Newton-bisection on [lo, hi].  Before that, a step that
     // is not a forward Newton step (slope >= 0) probes ahead geometrically.
-    if (kg > kn && isfinite(kg)) {
-        kappa = kg;
-        r_slope(yn, m, ncp, pe, phi, kappa, r, dr, Gp, buf, lane);
+    constexpr unsigned kAll = 0xffffffffu;
+    float r = 0.0f, lo = kn, hi = kn, dx_prev = 1.0e30f, dx = 1.0e30f;
+    bool have_hi = false, ok = true, todo = true;
+    kappa = kn;
+    loading = false;
+    dr = -1.0f;
+    Gp = 0.0f;
+    n_eval = 0;
+    int it = -2;                      // -2 trial, -1 warm start, then the iterations done
+#pragma unroll 1
+    while (__any_sync(kAll, todo)) {
+        float r1, dr1, G1;
+        r_slope4(yn, m, ncp, pe, phi, kappa, r1, dr1, G1, buf, lane);
+        if (!todo) continue;
+        r = r1;
+        dr = dr1;
+        Gp = G1;
         ++n_eval;
-    }
-    float lo = kn, hi = kn;
-    bool have_hi = false;
-    if (r > 0.0f) lo = kappa;
-    else {
-        hi = kappa;
-        have_hi = true;
-    }
-    float dx_prev = have_hi ? hi - lo : 1.0e30f, dx = dx_prev;
-    bool took_newton = false;
-    int it;
-    for (it = 0; it < m.local_max; ++it) {
+        if (it == -2) {
+            loading = (double)(r + kn) - kn_d > 0.0;
+            if (!loading) {
+                todo = false;
+                continue;
+            }
+            it = -1;
+            if (kg > kn && isfinite(kg)) {
+                kappa = kg;
+                continue;             // evaluate the warm start
+            }
+        }
+        if (r > 0.0f) {
+            lo = kappa;
+        } else {
+            hi = kappa;
+            have_hi = true;
+            if (it == -1) dx_prev = dx = hi - lo;
+        }
+        ++it;
         const float scale = fabsf(kappa) > 1.0f ? fabsf(kappa) : 1.0f;
-        if (fabsf(r) <= 2e-6f * scale || (have_hi && (hi - lo) <= 4.0f * kEpsF * scale)) break;
-        if (step_test && fabsf(r) <= 2e-6f * scale * fabsf(dr) &&
-            (have_hi ? (hi - lo) <= 1e-2f * scale : (took_newton && fabsf(2.0f * r) <= fabsf(dx * dr))))
-            break;
+        if (it >= m.local_max) {
+            ok = false;
+            todo = false;
+            continue;
+        }
+        if (fabsf(r) <= 2e-6f * scale || (have_hi && (hi - lo) <= 4.0f * kEpsF * scale)) {
+            todo = false;
+            continue;
+        }
         const float newton = kappa - r / dr;
         bool take;
         if (have_hi) {
@@ -241,7 +315,6 @@ __device__ __forceinline__ bool bracketed_newton(const DevNet &yn, const MatF &m
             take = dr < 0.0f && newton > lo && (newton - kappa) <= cap;
         }
         dx_prev = dx;
-        took_newton = take;
         if (take) {
             dx = kappa - newton;
             kappa = newton;
@@ -253,16 +326,8 @@ __device__ __forceinline__ bool bracketed_newton(const DevNet &yn, const MatF &m
             dx = step;
             kappa = lo + step;
         }
-        r_slope(yn, m, ncp, pe, phi, kappa, r, dr, Gp, buf, lane);
-        ++n_eval;
-        if (r > 0.0f) {
-            lo = kappa;
-        } else {
-            hi = kappa;
-            have_hi = true;
-        }
     }
-    return it < m.local_max;
+    return ok;
 }
 
 // element nodes of a warp's batch into shared memory (lane = (element, node)).
