@@ -318,7 +318,7 @@ __device__ __forceinline__ void energy_l1(const float4 *E1, int wp, const float 
 }
 
 // Value, gradient and Hessian (sym6 order) of the energy network at y for every point
-// of the CTA (out10, as psi_net_unit of the CUDA-core kernel):
+// of the CTA (out10, as psi_net_unit4 of the CUDA-core kernel):
 //   d2N/dy2 = sum_k w3_k sp''(h2_k) g_k g_k^T + sum_j v_j sp''(h1_j) W1_j W1_j^T,
 //   v = W2^T (w3 o sp'(h2)).
 // CTA-uniform control flow; returns with the tensor memory free for the next product.

@@ -50,13 +50,6 @@ __device__ __forceinline__ MatF to_f(const MatConst &m)
     return r;
 }
 
-__device__ __forceinline__ float softplus(float v) { return fmaxf(v, 0.0f) + log1pf(expf(-fabsf(v))); }
-__device__ __forceinline__ float sigm(float v)
-{
-    float e = expf(-fabsf(v));
-    float r = 1.0f / (1.0f + e);
-    return v >= 0.0f ? r : e * r;
-}
 // softplus(v) and its derivative sigmoid(v) from one exponential
 __device__ __forceinline__ void sp_sig(float v, float &sp, float &sg)
 {
@@ -65,13 +58,6 @@ __device__ __forceinline__ void sp_sig(float v, float &sp, float &sg)
     const float r = 1.0f / (1.0f + e);
     sg = v >= 0.0f ? r : e * r;
 }
-__device__ __forceinline__ float warp_sum(float v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 template <int DIM>
 struct Geo {
     static constexpr int NEN = DIM == 2 ? 4 : 8;
