@@ -53,6 +53,17 @@ constexpr double kTrialMargin = 1e-4;
 
 #include "gd_device_fp64.cuh"
 
+// the normalising constants of this kernel's own evaluation
+__device__ __forceinline__ NetConst own_consts(const NetConst &c)
+{
+    NetConst r = c;
+    r.psi_N0 = c.psi_N0_own;
+    r.psi_n = c.psi_n_own;
+    r.y_N0 = c.y_N0_own;
+    r.y_s = c.y_s_own;
+    return r;
+}
+
 // What a point keeps between its qp phases, in doubles (registers would halve the resident
 // warps)
 template <int DIM>
@@ -103,7 +114,7 @@ __device__ __forceinline__ int local_update(const AsmArgs &A, const e32::MatF &m
     const int64_t e_p = e0 + p / NQ;
     const bool need = e_p < A.n_elems && spec_of(A, e_p < A.n_elems ? e_p : A.n_elems - 1) == sn;
     const DevNet &yn = yld_of(A, sn);
-    const NetConst nc = A.netc[sn];
+    const NetConst nc = own_consts(A.netc[sn]);
     const e32::NcF nf = e32::ncf(nc);
     const int local_max = A.mat.local_max;
     const double pe = sIn[p * 4], phi = sIn[p * 4 + 1], kn = sIn[p * 4 + 2];
@@ -511,7 +522,7 @@ __global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
                 ph[5] = (m.lambda_e + m.mu_e - m.lambda_e * L) / (J * J);
             } else {
                 const double *o = sOut + pt * 10;
-                const NetConst nc = A.netc[valid ? spec_of(A, e_me) : 0];
+                const NetConst nc = own_consts(A.netc[valid ? spec_of(A, e_me) : 0]);
 #pragma unroll
                 for (int i = 0; i < 3; ++i) ps[i] = o[1 + i];
 #pragma unroll
@@ -702,24 +713,38 @@ cudaError_t launch_assemble_fp64(int dim, const AsmArgs &a, int num_sms, cudaStr
 }
 
 // ---------------------------------------------------------------------------
-// network constants: N(0), n (S(C=I) = 0), N_k(0), s = 1/N_k'(0)  (Sec. 4.2)
+// network constants: N(0), n (S(C=I) = 0), N_k(0), s = 1/N_k'(0)  (Sec. 4.2), by the FP64
+// functions and by the element kernel's.  Two roundings of N(0) would leave psi_e and G near
+// +-1e-16 at a point without strain, and half of those above zero: "loading".
 // ---------------------------------------------------------------------------
 namespace {
 __global__ void prep_nets_kernel(DevNet psi, DevNet yld, int energy, NetConst *out)
 {
-    __shared__ double buf[5 * kMaxWidth];
+    __shared__ __align__(16) double buf[grp::buf_bytes(kMaxWidth) / sizeof(double)];
+    __shared__ double sY[grp::kPts * 4], sO[grp::kPts * 10];
     const int lane = threadIdx.x;
+    const bool need = lane < grp::kLanes;            // one point
     NetConst nc;
     nc.psi_N0 = 0.0;
     nc.psi_n = 0.0;
     nc.y_N0 = 0.0;
     nc.y_s = 1.0;
+    nc.psi_N0_own = nc.psi_n_own = nc.y_N0_own = 0.0;
+    nc.y_s_own = 1.0;
     if (energy != GD_ENERGY_NEO_HOOKE && psi.width > 0) {
         double x0[3] = {0.0, 0.0, 0.0}, o[10];
         psi_net_unit(psi, x0, o, buf, lane);
         nc.psi_N0 = o[0];
         // dI1/dC = I, dI2/dC = 2 I, dJ/dC = I/2 at C = I (raw); dI1G/dC = dI2G/dC = 0 (Eq. (dd_1))
         nc.psi_n = (energy == GD_ENERGY_ICNN_RAW) ? 2.0 * o[1] + 4.0 * o[2] + o[3] : o[3];
+        if (lane < grp::kPts * 4) sY[lane] = 0.0;
+        __syncwarp();
+        grp::energy(psi, sY, sO, reinterpret_cast<unsigned char *>(buf), lane, need, false);
+        // (weights that are not finite leave no trace in the fixed-point copies)
+        nc.psi_N0_own = isfinite(nc.psi_N0) ? sO[0] : nc.psi_N0;
+        nc.psi_n_own = !isfinite(nc.psi_n) ? nc.psi_n
+                       : (energy == GD_ENERGY_ICNN_RAW) ? 2.0 * sO[1] + 4.0 * sO[2] + sO[3] : sO[3];
+        __syncwarp();
     }
     if (yld.width > 0) {
         NetConst unit;
@@ -729,6 +754,9 @@ __global__ void prep_nets_kernel(DevNet psi, DevNet yld, int energy, NetConst *o
         yield_unit(yld, unit, 0.0, G, Gp, buf, lane);   // raw N_k(0), N_k'(0)
         nc.y_N0 = G;
         nc.y_s = 1.0 / Gp;
+        const double2 n = grp::yield<true>(yld.p, yld.fx, yld.width, 0.0, reinterpret_cast<unsigned char *>(buf), lane, need);
+        nc.y_N0_own = isfinite(G) ? __shfl_sync(0xffffffffu, n.x, 0) : G;
+        nc.y_s_own = isfinite(Gp) ? 1.0 / __shfl_sync(0xffffffffu, n.y, 0) : nc.y_s;
     }
     if (lane == 0) *out = nc;
 }

@@ -19,6 +19,10 @@ constexpr int kMaxWidth = 64;   // widest supported ICNN layer
 // S(C = I) = 0; yield: N_k(0) and s = 1 / N_k'(0) so that G(0) = 0, G'(0) = 1.
 struct NetConst {
     double psi_N0, psi_n, y_N0, y_s;
+    // the same constants as the FP64 element kernel's own evaluation of the networks gives them
+    // (it rounds otherwise than the FP64 functions, and a point without strain must come out
+    // with psi_e = 0 and G = 0 exactly)
+    double psi_N0_own, psi_n_own, y_N0_own, y_s_own;
 };
 
 // One ICNN on the device: packed parameters (gd_icnn layout) plus a

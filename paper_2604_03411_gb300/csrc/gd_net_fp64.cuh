@@ -22,7 +22,7 @@ constexpr int kOut = 16 / kLanes;          // a lane's outputs of a 16-wide chun
 
 // shared-memory bytes of a warp's network buffers for width w: operands [w][kPts][4], one
 // 64-bit word [w][kPts] per unit, reverse operands [w][kPts]
-__host__ __device__ inline size_t buf_bytes(int w) { return (size_t)w * kPts * (4 + 1 + 1) * 8; }
+__host__ __device__ constexpr size_t buf_bytes(int w) { return (size_t)w * kPts * (4 + 1 + 1) * 8; }
 
 template <class T>
 __device__ __forceinline__ T sum_lanes(T v)
@@ -90,7 +90,9 @@ __device__ __forceinline__ void chunk_product(const int2 *__restrict__ W, int wp
 }
 
 // Energy network N(y) with gradient and (hess) Hessian in sym6 order, for the points with
-// need: y at sY[pt 4 ..], results to sO[pt 10 ..].  Same identities as psi_net_unit:
+// need: y at sY[pt 4 ..], results to sO[pt 10 ..].  N(y) is the same to the last bit wherever this
+// is compiled in (explicit fma in its sum): the normalising constants rely on it, as they do
+// for both forms of yield.  Same identities as psi_net_unit:
 //   d2N/dy2 = sum_k w3_k sp''(h2_k) g_k g_k^T + sum_j v_j sp''(h1_j) W1_j W1_j^T,
 //   v = W2^T (w3 o sp'(h2)).
 __device__ __forceinline__ void energy(const DevNet &net, const double *sY, double *sO, unsigned char *buf, int lane,
@@ -149,7 +151,7 @@ __device__ __forceinline__ void energy(const DevNet &net, const double *sY, doub
                 fx::softplus_sigmoid(h, s, g);
                 const i64 uq = fx::mulhi_s(__ldg(fn.w3 + k), g);              // units of 2^(ew3 - 60)
                 const double u = fx::to_double(uq, ew3 - 60);
-                acc[0] += __ldg(w3 + k) * (hi_word(h) >= 0x40500000 ? h : fx::to_double(s, -57));
+                acc[0] = fma(__ldg(w3 + k), hi_word(h) >= 0x40500000 ? h : fx::to_double(s, -57), acc[0]);
                 acc[1] += u * g0;
                 acc[2] += u * g1;
                 acc[3] += u * g2;
@@ -247,7 +249,7 @@ static __device__ __noinline__ double2 yield(const double *p, const unsigned cha
                 const double h = fx::to_double(V[i][0], er + ep) + fma(b, q, __ldg(c2 + k));
                 i64 s, g;
                 fx::softplus_sigmoid(h, s, g);
-                n0 += __ldg(v3 + k) * (hi_word(h) >= 0x40500000 ? h : fx::to_double(s, -57));
+                n0 = fma(__ldg(v3 + k), hi_word(h) >= 0x40500000 ? h : fx::to_double(s, -57), n0);
                 if (SLOPE)
                     n1 += fx::to_double(fx::mulhi_s(__ldg(fn.w3 + k), g), ew3 - 60) *
                           (fx::to_double(V[i][NC - 1], er + ew1) + b);
