@@ -50,9 +50,6 @@ namespace {
 // decided by the FP32 evaluation; closer ones by an FP64 evaluation
 constexpr double kTrialMargin = 1e-4;
 
-
-#include "gd_device_fp64.cuh"
-
 // the normalising constants of this kernel's own evaluation
 __device__ __forceinline__ NetConst own_consts(const NetConst &c)
 {
@@ -754,7 +751,8 @@ __global__ void prep_nets_kernel(DevNet psi, DevNet yld, int energy, NetConst *o
         yield_unit(yld, unit, 0.0, G, Gp, buf, lane);   // raw N_k(0), N_k'(0)
         nc.y_N0 = G;
         nc.y_s = 1.0 / Gp;
-        const double2 n = grp::yield<true>(yld.p, yld.fx, yld.width, 0.0, reinterpret_cast<unsigned char *>(buf), lane, need);
+        const double2 n = grp::yield<true>(yld.p, yld.W2T, yld.fx, yld.width, 0.0, reinterpret_cast<unsigned char *>(buf), lane,
+                                                  need);
         nc.y_N0_own = isfinite(G) ? __shfl_sync(0xffffffffu, n.x, 0) : G;
         nc.y_s_own = isfinite(Gp) ? 1.0 / __shfl_sync(0xffffffffu, n.y, 0) : nc.y_s;
     }

@@ -5,8 +5,18 @@
 // layer's units are FP64; activations and the layer products are 64-bit fixed point
 // (gd_fixed.cuh).  The FP32 evaluations of the local solve use the same mapping.
 // Every function is called by the whole warp; `need` marks the points that take part (all
-// lanes of a point agree) and net is the same for all of them.
+// lanes of a point agree) and net is the same for all of them.  Points whose argument is not
+// finite (far past the root of the local solve f_d underflows and q is infinite) take the FP64
+// functions of gd_device_fp64.cuh, one after the other with a lane per unit.
 #pragma once
+
+#include "gd_internal.cuh"
+
+namespace gd {
+namespace {
+#include "gd_device_fp64.cuh"
+}
+}  // namespace gd
 
 #include "gd_elem32.cuh"
 #include "gd_fixed.cuh"
@@ -38,6 +48,55 @@ __device__ __forceinline__ int max_lanes(int v)
     return v;
 }
 __device__ __forceinline__ int hi_word(double v) { return __double2hiint(v); }
+
+// bit p: point p of the warp takes the FP64 functions (all lanes of a point agree on `take`)
+__device__ __forceinline__ unsigned points_of(bool take)
+{
+    const unsigned b = __ballot_sync(0xffffffffu, take);
+    return (b & 1u) | (b >> 7 & 2u) | (b >> 14 & 4u) | (b >> 21 & 8u);
+}
+static_assert(kLanes == 8, "points_of");
+// The networks of the points in `mask` by the FP64 functions (p, W2T: the network's parameters
+// and transposed W2).  Out of line: few points come here.
+static __device__ __noinline__ void energy_fp64(const double *p, double *W2T, int w, const double *sY, double *sO,
+                                                double *buf, int lane, unsigned mask, bool hess)
+{
+    DevNet net;
+    net.p = const_cast<double *>(p);
+    net.W2T = W2T;
+    net.width = w;
+    for (int pt = 0; pt < kPts; ++pt) {
+        if (!(mask >> pt & 1u)) continue;
+        double o[10];
+        psi_net_unit(net, sY + pt * 4, o, buf, lane, hess);
+        if (lane < 10) {
+            double v = 0.0;
+#pragma unroll
+            for (int c = 0; c < 10; ++c)
+                if (c == lane) v = o[c];
+            sO[pt * 10 + lane] = lane < 4 || hess ? v : 0.0;
+        }
+    }
+    __syncwarp();
+}
+static __device__ __noinline__ double2 yield_fp64(const double *p, double *W2T, int w, double q, double2 r, double *buf,
+                                                  int lane, unsigned mask)
+{
+    DevNet net;
+    net.p = const_cast<double *>(p);
+    net.W2T = W2T;
+    net.width = w;
+    NetConst unit;
+    unit.y_N0 = 0.0;
+    unit.y_s = 1.0;
+    for (int pt = 0; pt < kPts; ++pt) {
+        if (!(mask >> pt & 1u)) continue;
+        double N, Np;
+        yield_unit(net, unit, __shfl_sync(0xffffffffu, q, pt * kLanes), N, Np, buf, lane);
+        if (lane / kLanes == pt) r = make_double2(N, Np);
+    }
+    return r;
+}
 
 // NC column products of a 16-wide output chunk: V[i][c] = sum_j W(k_i, j) z_c(j) in units of
 // 2^-56 (times the operand and row scales), k_i = c0 + 8 i + sub.  Three multiply-adds per
@@ -105,8 +164,8 @@ __device__ __forceinline__ void energy(const DevNet &net, const double *sY, doub
     i64 *sE = reinterpret_cast<i64 *>(z + w * kPts * 4);        // [w][kPts]: h1, then sp''(h1)
     int2 *su = reinterpret_cast<int2 *>(sE + w * kPts);         // [w][kPts]
     double y0 = sY[pt * 4], y1 = sY[pt * 4 + 1], y2 = sY[pt * 4 + 2];
-    const bool bad = !(isfinite(y0) && isfinite(y1) && isfinite(y2));
-    if (bad || !need) y0 = y1 = y2 = 0.0;
+    const unsigned far = points_of(need && !(isfinite(y0) && isfinite(y1) && isfinite(y2)));
+    if ((far >> pt & 1u) || !need) y0 = y1 = y2 = 0.0;
     // layer 1: pre-activations and the point's operand scale
     int hm = 0;
     for (int j = sub; j < w; j += kLanes) {
@@ -192,24 +251,21 @@ __device__ __forceinline__ void energy(const DevNet &net, const double *sY, doub
         if (c < 4 || hess) acc[c] = sum_lanes(acc[c]);
     if (sub == 0 && need) {
         double *o = sO + pt * 10;
-        const double nan = __longlong_as_double(0x7ff8000000000000LL);
         o[0] = acc[0] + __ldg(a3) * y0 + __ldg(a3 + 1) * y1 + __ldg(a3 + 2) * y2;
         o[1] = acc[1] + __ldg(a3);
         o[2] = acc[2] + __ldg(a3 + 1);
         o[3] = acc[3] + __ldg(a3 + 2);
 #pragma unroll
         for (int c = 4; c < 10; ++c) o[c] = hess ? acc[c] : 0.0;
-        if (bad)
-#pragma unroll
-            for (int c = 0; c < 10; ++c) o[c] = nan;
     }
     __syncwarp();
+    if (far) energy_fp64(net.p, net.W2T, w, sY, sO, reinterpret_cast<double *>(buf), lane, far, hess);
 }
 
-// Yield network N_k(q) and, with SLOPE, N_k'(q) (parameters p and fixed-point copy fxp of a
-// network of width w > 0).  Every lane of a point returns the same values.
+// Yield network N_k(q) and, with SLOPE, N_k'(q) (parameters p, transposed W2T and fixed-point
+// copy fxp of a network of width w > 0).  Every lane of a point returns the same values.
 template <bool SLOPE>
-static __device__ __noinline__ double2 yield(const double *p, const unsigned char *fxp, int w, double q,
+static __device__ __noinline__ double2 yield(const double *p, double *W2T, const unsigned char *fxp, int w, double q,
                                              unsigned char *buf, int lane, bool need)
 {
     constexpr int NC = SLOPE ? 2 : 1;
@@ -218,8 +274,9 @@ static __device__ __noinline__ double2 yield(const double *p, const unsigned cha
     const fx::Net fn = fx::net_of(fxp, w);
     int2 *z = reinterpret_cast<int2 *>(buf);                       // [w][kPts][NC]
     i64 *sE = reinterpret_cast<i64 *>(z + w * kPts * NC);
-    const bool bad = !isfinite(q);
-    if (bad || !need) q = 0.0;
+    const double q_in = q;
+    const unsigned far = points_of(need && !isfinite(q));
+    if (!need || !isfinite(q)) q = 0.0;
     int hm = 0;
     for (int j = sub; j < w; j += kLanes) {
         const double h = fma(__ldg(V1 + j), q, __ldg(c1 + j));
@@ -256,11 +313,11 @@ static __device__ __noinline__ double2 yield(const double *p, const unsigned cha
             }
         }
     }
-    const double b = __ldg(b3), nan = __longlong_as_double(0x7ff8000000000000LL);
+    const double b = __ldg(b3);
     double2 r = make_double2(sum_lanes(n0) + b * q, 0.0);
     if (SLOPE) r.y = sum_lanes(n1) + b;
-    if (bad) r = make_double2(nan, nan);
     __syncwarp();
+    if (far) r = yield_fp64(p, W2T, w, q_in, r, reinterpret_cast<double *>(buf), lane, far);
     return r;
 }
 
@@ -277,7 +334,7 @@ __device__ __forceinline__ void residual(const MatConst &m, const DevNet &yld, c
     // G(q) = s (N_k(q) - N_k(0)) (Eq. (Gq_NN)); width 0 is the identity G(q) = q
     double G = q, Gs = 1.0;
     if (yld.width > 0) {
-        const double2 n = yield<SLOPE>(yld.p, yld.fx, yld.width, q, buf, lane, need);
+        const double2 n = yield<SLOPE>(yld.p, yld.W2T, yld.fx, yld.width, q, buf, lane, need);
         G = nc.y_s * (n.x - nc.y_N0);
         Gs = nc.y_s * n.y;
     }
