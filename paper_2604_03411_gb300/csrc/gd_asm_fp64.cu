@@ -46,9 +46,11 @@
 namespace gd {
 namespace {
 
-// trial yield values farther than this (relative to max(1, kappa_n)) from zero are
-// decided by the FP32 evaluation; closer ones by an FP64 evaluation
-constexpr double kTrialMargin = 1e-4;
+// Trial yield values farther than this (relative to max(1, kappa_n)), and than what FP32 may be
+// off by, from zero are decided by the FP32 evaluation; closer ones by an FP64 evaluation.  The
+// FP32 network's relative error is a few 1e-7 (two sums of up to 64 positive terms), of
+// N(0) / N'(0) where the network hardly depends on q and of q's terms near full damage.
+constexpr double kTrialMargin = 1e-4, kTrialRel = 2e-6;
 
 // the normalising constants of this kernel's own evaluation
 __device__ __forceinline__ NetConst own_consts(const NetConst &c)
@@ -121,11 +123,11 @@ __device__ __forceinline__ int local_update(const AsmArgs &A, const e32::MatF &m
     int n_eval = 0;
     // Trial Phi_d(kappa_n): the FP32 network decides points clearly off the yield
     // surface, an FP64 evaluation the others.
-    float r32, dr32, Gp32;
-    grp::residual32(mf, yn, nf, pef, phf, knf, r32, dr32, Gp32, nbuf, lane);
+    float r32, dr32, Gp32, mag;
+    grp::residual32(mf, yn, nf, pef, phf, knf, r32, dr32, Gp32, mag, nbuf, lane);
     const double scale_n = fabs(kn) > 1.0 ? fabs(kn) : 1.0;
     bool load = need && r32 > 0.0f;
-    const bool close = need && !(fabs((double)r32) > kTrialMargin * scale_n);
+    const bool close = need && !(fabs((double)r32) > kTrialMargin * scale_n + kTrialRel * (double)mag);
     if (__any_sync(kAll, close)) {
         double rt, drt, gt;
         grp::residual<true>(A.mat, yn, nc, pe, phi, kn, rt, drt, gt, nbuf, lane, close);
@@ -198,7 +200,7 @@ __device__ __forceinline__ int local_update(const AsmArgs &A, const e32::MatF &m
             }
             if (!__any_sync(kAll, run)) break;
             float re, dre, ge;
-            grp::residual32(mf, yn, nf, pef, phf, k32, re, dre, ge, nbuf, lane);
+            grp::residual32(mf, yn, nf, pef, phf, k32, re, dre, ge, mag, nbuf, lane);
             if (run) {
                 r32 = re;
                 dr32 = dre;
