@@ -25,11 +25,15 @@
 //    closed form of every (a, b) pair.
 //  - The networks run in 64-bit fixed point (gd_fixed.cuh).
 // Measured (GB300, gd_assemble with tangent; before: FP64 networks one point at a time with
-// a lane per unit, closed-form rows): 140,400 points of HEX8, both widths 64, 33.6 -> 5.75 ms;
-// 159,744 of Q4, widths 32, 10.2 -> 2.4 ms; 256 of Q4, widths 16 and 8, 1.21 -> 0.085 ms;
-// residual alone of 32,640 HEX8 points, widths 24 and 40, 3.53 -> 0.50 ms.  16 warps per SM
-// (128 registers, the points' state in shared memory) against 8 with 255 registers: 7.5 ->
-// 5.75 ms on the first; instruction latency is the leading stall, the FP64 pipe 30 % busy.
+// a lane per unit, closed-form rows): 140,400 points of HEX8, both widths 64, 33.6 -> 5.83 ms;
+// 159,744 of Q4, widths 32, 10.2 -> 2.60 ms; 256 of Q4, widths 16 and 8, 1.21 -> 0.088 ms;
+// residual alone of 32,640 HEX8 points, widths 24 and 40, 3.53 -> 0.53 ms.  (Without the
+// trust in the fixed-point sums being checked and with one scale for all first-layer and
+// one for all output weights: 5.70, 2.52, 0.085 and 0.51 ms.)  Built for 16 warps per SM: 128
+// registers, with 180-340 bytes of spills in 2D and 560-990 in 3D, the points' state in shared
+// memory.  Width-64 HEX8 networks need 64 KB per CTA of four warps, so that 12 warps are
+// resident there (8 with 255 registers: 7.5 ms where 12 took 5.75).  Instruction latency is the
+// leading stall, the FP64 pipe 30 % busy.
 //
 // Paper passages: Sec. 3.1 (F, phi_q, grad phi_q, element residual, Table
 // kernel_inputs), Sec. 2.1 (P, Y vector, Y), Sec. 2.2 and Sec. 3.2 Eq. (dd_7_no_nn)
@@ -113,6 +117,7 @@ __device__ __forceinline__ int local_update(const AsmArgs &A, const e32::MatF &m
     const int64_t e_p = e0 + p / NQ;
     const bool need = e_p < A.n_elems && spec_of(A, e_p < A.n_elems ? e_p : A.n_elems - 1) == sn;
     const DevNet &yn = yld_of(A, sn);
+    const int yp = grp::path_of(yn);
     const NetConst nc = own_consts(A.netc[sn]);
     const e32::NcF nf = e32::ncf(nc);
     const int local_max = A.mat.local_max;
@@ -130,7 +135,7 @@ __device__ __forceinline__ int local_update(const AsmArgs &A, const e32::MatF &m
     const bool close = need && !(fabs((double)r32) > kTrialMargin * scale_n + kTrialRel * (double)mag);
     if (__any_sync(kAll, close)) {
         double rt, drt, gt;
-        grp::residual<true>(A.mat, yn, nc, pe, phi, kn, rt, drt, gt, nbuf, lane, close);
+        grp::residual<true>(A.mat, yn, yp, nc, pe, phi, kn, rt, drt, gt, nbuf, lane, close);
         if (close) {
             ++n_eval;
             r = rt;
@@ -223,11 +228,11 @@ __device__ __forceinline__ int local_update(const AsmArgs &A, const e32::MatF &m
     if (__any_sync(kAll, polish)) {
         const double sc = fabs((double)k32) > 1.0 ? fabs((double)k32) : 1.0;
         double r0, d0, g0;
-        grp::residual<false>(A.mat, yn, nc, pe, phi, (double)k32, r0, d0, g0, nbuf, lane, polish);
+        grp::residual<false>(A.mat, yn, yp, nc, pe, phi, (double)k32, r0, d0, g0, nbuf, lane, polish);
         if (polish) ++n_eval;
         polish = polish && fabs(r0) <= 1e-4 * sc;
         const double k1 = polish ? (double)k32 - r0 / (double)dr32 : kn;
-        grp::residual<true>(A.mat, yn, nc, pe, phi, k1, r0, d0, g0, nbuf, lane, polish);
+        grp::residual<true>(A.mat, yn, yp, nc, pe, phi, k1, r0, d0, g0, nbuf, lane, polish);
         if (polish) {
             ++n_eval;
             r = r0;
@@ -251,7 +256,7 @@ __device__ __forceinline__ int local_update(const AsmArgs &A, const e32::MatF &m
         int it = 0;
         while (__any_sync(kAll, run)) {
             double re, dre, ge;
-            grp::residual<true>(A.mat, yn, nc, pe, phi, kappa, re, dre, ge, nbuf, lane, run);
+            grp::residual<true>(A.mat, yn, yp, nc, pe, phi, kappa, re, dre, ge, nbuf, lane, run);
             if (run) {
                 ++n_eval;
                 r = re;
@@ -343,6 +348,7 @@ __global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
         sRef[t * 4 + 3] = N;
     }
     const int64_t e_last = A.n_elems - 1;
+    const int psi_path = m.energy != GD_ENERGY_NEO_HOOKE && !A.psi_tab ? grp::path_of(A.psi) : 0;
 
     const int64_t n_batches = (A.n_elems + EL - 1) / EL;
     for (int64_t batch = blockIdx.x; batch < n_batches; batch += gridDim.x) {
@@ -500,8 +506,11 @@ __global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
                 specimens(p0, s0, s1);
                 const int64_t e_p = e0 + (p0 + lane / grp::kLanes) / NQ;
                 const int sp = e_p <= e_last ? spec_of(A, e_p) : -1;
-                for (int sn = s0; sn <= s1; ++sn)
-                    grp::energy(psi_of(A, sn), sIn + p0 * 4, sOut + p0 * 10, nbuf, lane, sp == sn, A.tangent != 0);
+                for (int sn = s0; sn <= s1; ++sn) {
+                    const DevNet &net = psi_of(A, sn);
+                    grp::energy(net, A.psi_tab ? grp::path_of(net) : psi_path, sIn + p0 * 4, sOut + p0 * 10, nbuf, lane,
+                                sp == sn, A.tangent != 0);
+                }
             }
         }
         cta_sync<KW>();
@@ -738,11 +747,9 @@ __global__ void prep_nets_kernel(DevNet psi, DevNet yld, int energy, NetConst *o
         nc.psi_n = (energy == GD_ENERGY_ICNN_RAW) ? 2.0 * o[1] + 4.0 * o[2] + o[3] : o[3];
         if (lane < grp::kPts * 4) sY[lane] = 0.0;
         __syncwarp();
-        grp::energy(psi, sY, sO, reinterpret_cast<unsigned char *>(buf), lane, need, false);
-        // (weights that are not finite leave no trace in the fixed-point copies)
-        nc.psi_N0_own = isfinite(nc.psi_N0) ? sO[0] : nc.psi_N0;
-        nc.psi_n_own = !isfinite(nc.psi_n) ? nc.psi_n
-                       : (energy == GD_ENERGY_ICNN_RAW) ? 2.0 * sO[1] + 4.0 * sO[2] + sO[3] : sO[3];
+        grp::energy(psi, grp::path_of(psi), sY, sO, reinterpret_cast<unsigned char *>(buf), lane, need, false);
+        nc.psi_N0_own = sO[0];
+        nc.psi_n_own = (energy == GD_ENERGY_ICNN_RAW) ? 2.0 * sO[1] + 4.0 * sO[2] + sO[3] : sO[3];
         __syncwarp();
     }
     if (yld.width > 0) {
@@ -753,10 +760,10 @@ __global__ void prep_nets_kernel(DevNet psi, DevNet yld, int energy, NetConst *o
         yield_unit(yld, unit, 0.0, G, Gp, buf, lane);   // raw N_k(0), N_k'(0)
         nc.y_N0 = G;
         nc.y_s = 1.0 / Gp;
-        const double2 n = grp::yield<true>(yld.p, yld.W2T, yld.fx, yld.width, 0.0, reinterpret_cast<unsigned char *>(buf), lane,
-                                                  need);
-        nc.y_N0_own = isfinite(G) ? __shfl_sync(0xffffffffu, n.x, 0) : G;
-        nc.y_s_own = isfinite(Gp) ? 1.0 / __shfl_sync(0xffffffffu, n.y, 0) : nc.y_s;
+        const double2 n = grp::yield<true>(yld.p, yld.W2T, yld.fx, yld.width, grp::path_of(yld), 0.0,
+                                             reinterpret_cast<unsigned char *>(buf), lane, need);
+        nc.y_N0_own = __shfl_sync(0xffffffffu, n.x, 0);
+        nc.y_s_own = 1.0 / __shfl_sync(0xffffffffu, n.y, 0);
     }
     if (lane == 0) *out = nc;
 }
@@ -795,8 +802,12 @@ cudaError_t launch_net_to_float(const DevNet &net, cudaStream_t s)
 }
 
 namespace {
-// fixed-point copies of one network (layout of fx::Net): each weight row and column set is
-// scaled by the power of two above its largest magnitude
+// a bias below this: the units are likely to reach the tail of softplus (h < -3.47), and points of
+// such a network are evaluated with it at once
+constexpr double kTailBias = -3.0;
+
+// fixed-point copies of one network (layout of fx::Net): each row of W2 and W2^T, each column of
+// W1 and each output weight is scaled by the power of two above its largest magnitude
 __global__ void net_fixed_kernel(DevNet net)
 {
     using namespace fx;
@@ -804,13 +815,28 @@ __global__ void net_fixed_kernel(DevNet net)
     const double *W1 = net.p, *W2 = W1 + w * n_in + w, *w3 = W2 + w * w + w * n_in + w;
     const Net f = net_of(net.fx, w);
     int *e = const_cast<int *>(f.e);
-    for (int t = t0; t < 2 * w + 2; t += nt) {
+    for (int t = t0; t < 3 * w + 3; t += nt) {
         double m = 0.0;
         if (t < w) for (int j = 0; j < w; ++j) m = fmax(m, fabs(W2[t * w + j]));
         else if (t < 2 * w) for (int k = 0; k < w; ++k) m = fmax(m, fabs(W2[k * w + t - w]));
-        else if (t == 2 * w) for (int i = 0; i < w * n_in; ++i) m = fmax(m, fabs(W1[i]));
-        else for (int k = 0; k < w; ++k) m = fmax(m, fabs(w3[k]));
-        e[t] = bound_exp(m);
+        else if (t < 3 * w) m = fabs(w3[t - 2 * w]);
+        else if (t - 3 * w < n_in) for (int j = 0; j < w; ++j) m = fmax(m, fabs(W1[j * n_in + t - 3 * w]));
+        e[t] = m == 0.0 ? kZero : bound_exp(m);
+    }
+    __syncthreads();
+    int path = kPlain;
+    for (int t = t0; t < net.n_params; t += nt)
+        if (!isfinite(net.p[t])) path = kFp64;
+    for (int t = t0; t < 3 * w + 3; t += nt)
+        if (e[t] > kLargest) path = kFp64;
+    for (int t = t0; t < w; t += nt)
+        if (path == kPlain && (net.p[w * n_in + t] < kTailBias || w3[t - w] < kTailBias)) path = kTails;
+    const bool fp64 = __syncthreads_or(path == kFp64), tails = __syncthreads_or(path == kTails);
+    if (t0 == 0) e[3 * w + kPath] = fp64 ? kFp64 : tails ? kTails : kPlain;
+    if (t0 < 3) {
+        int m = kZero;
+        for (int k = 0; k < w; ++k) m = max(m, e[t0 * w + k]);
+        e[3 * w + kRows + t0] = m;
     }
     __syncthreads();
     for (int t = t0; t < w * wp; t += nt) {
@@ -823,8 +849,8 @@ __global__ void net_fixed_kernel(DevNet net)
     for (int j = t0; j < w; j += nt) {
         double v[3] = {0.0, 0.0, 0.0};
         for (int c = 0; c < n_in && c < 3; ++c) v[c] = W1[j * n_in + c];
-        for (int c = 0; c < 4; ++c) const_cast<i64 *>(f.W1)[4 * j + c] = c < 3 ? from_double(v[c], 62 - e[2 * w]) : 0;
-        const_cast<i64 *>(f.w3)[j] = from_double(w3[j], 62 - e[2 * w + 1]);
+        for (int c = 0; c < 4; ++c) const_cast<i64 *>(f.W1)[4 * j + c] = c < 3 ? from_double(v[c], 62 - e[3 * w + c]) : 0;
+        const_cast<i64 *>(f.w3)[j] = from_double(w3[j], 62 - e[2 * w + j]);
         double *ww = const_cast<double *>(f.WW) + 6 * j;
         ww[0] = v[0] * v[0]; ww[1] = v[0] * v[1]; ww[2] = v[0] * v[2];
         ww[3] = v[1] * v[1]; ww[4] = v[1] * v[2]; ww[5] = v[2] * v[2];
