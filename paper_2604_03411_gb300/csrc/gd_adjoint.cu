@@ -332,23 +332,18 @@ __global__ void __launch_bounds__(32) adjoint_kernel(AdjArgs A)
                 ps[2] += -m.mu_e * nc.psi_n + m.lambda_e * 2.0 * t * dt;
             }
         }
-        const double kn = valid ? __ldg(A.kappa_prev + e_me * NQ + q) : 0.0;
         const double kc = valid ? __ldg(A.kappa_cur + e_me * NQ + q) : 0.0;
         Q[3] = pe;
         Q[4] = phi;
-        Q[5] = kn;
         Q[6] = kc;
         __syncwarp();
-        // ---- unit mode: the forward loading decision and G, G' at kappa_n ----
+        // ---- unit mode: G, G' at kappa_n ----
         for (int p = p0; p < p1; ++p) {
             if (e0 + p / NQ >= A.n_elems) break;
-            const double ppe = sQ[p * 16 + 3], pphi = sQ[p * 16 + 4], pkn = sQ[p * 16 + 5], pkc = sQ[p * 16 + 6];
+            const double ppe = sQ[p * 16 + 3], pphi = sQ[p * 16 + 4], pkc = sQ[p * 16 + 6];
             double r, dr, Gp;
-            r_slope(A.mat, A.yld, nc, ppe, pphi, pkn, r, dr, Gp, sBuf, lane);
-            const double loading = r > 0.0 ? 1.0 : 0.0;
             r_slope(A.mat, A.yld, nc, ppe, pphi, pkc, r, dr, Gp, sBuf, lane);
             if (lane == 0) {
-                sOut[p * 10 + 4] = loading;
                 sOut[p * 10 + 5] = Gp;
                 sOut[p * 10 + 6] = dr;
                 sOut[p * 10 + 7] = r + pkc;     // G(q(kappa_n))
@@ -357,7 +352,10 @@ __global__ void __launch_bounds__(32) adjoint_kernel(AdjArgs A)
         __syncwarp();
         // ---- qp mode: coupling coefficients ----
         const double *o = sOut + lane * 10;
-        const bool loading = o[4] > 0.5;
+        // the branch of the transposed tangent: a decision taken anew could differ from the element
+        // kernel's where Phi_d(kappa_{n-1}) is at its rounding (a held load), and the gradient would
+        // mix both branches
+        const bool loading = valid && __ldg(A.loading + e_me * NQ + q) != 0;
         const double Gp = o[5], rp = o[6], Gn = o[7];
         const bool dmg = kc > m.kappa_d;
         const double fd = dmg ? exp(-m.eta_d * (kc - m.kappa_d)) : 1.0;

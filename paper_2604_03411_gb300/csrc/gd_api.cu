@@ -2461,7 +2461,7 @@ gd_status gd_backward(gd_handle *h, const double *dL_dreaction, double *dL_dthet
             A.conn = H.conn;
             A.X = H.X;
             A.dofs = d_c;
-            A.kappa_prev = k_p;
+            A.loading = H.loading2;
             A.kappa_cur = k_c;
             A.w = nullptr;
             A.kbar = H.kbar;

@@ -82,7 +82,7 @@ struct AdjArgs {
     const int32_t *conn;
     const double *X;
     const double *dofs;        // d_n
-    const double *kappa_prev;  // kappa_{n-1}
+    const int8_t *loading;     // branch of every point in the tangent that is transposed
     const double *kappa_cur;   // kappa_n
     const double *w;           // nodal adjoint weights (mode 1)
     const double *kbar;        // dL/dkappa_n
