@@ -472,6 +472,10 @@ __device__ void yield_tc(Shared &S, const TcArgs &T, const NcF &nc, float q, boo
     const float *b3 = reinterpret_cast<const float *>(Y2 + wp);
     const uint32_t lane_base = S.tbase + ((uint32_t)(warp * 32) << 16);
     const bool any = __any_sync(0xffffffffu, need);          // a warp's rows are written together
+    // The padded units' weights are zero, and zero times an infinite q (f_d underflows) is NaN: a
+    // large finite q keeps the sign of the result.  (Split operands make NaN of it by themselves:
+    // the residual of an infinite operand is inf - inf.)
+    if (!SPLIT && isinf(q)) q = copysignf(1.0e30f, q);
     uint8_t *t0 = S.tiles, *t1 = S.tiles + T.tile_bytes;
     const uint32_t a0 = saddr(t0), a1 = saddr(t1), bv = saddr(S.blob + T.s_slot);
     constexpr int ROUNDS = SPLIT ? 2 : 1;
