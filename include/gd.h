@@ -396,12 +396,13 @@ typedef struct gd_tune_report {
     double asm_ms[3];            /* element-kernel pass (tangent) with 2, 4, 8 warps; -1: does
                                     not fit in shared memory                                    */
     double krylov_us[4];         /* Krylov iteration time with 1..4 CTAs per SM; -1: not
-                                    co-resident                                                 */
-    int32_t krylov_up;           /* node groups per lane in the Krylov products (1, 2 or 4)     */
-    double krylov_us_up[3];      /* iteration time with 1, 2, 4 node groups at the chosen grid  */
+                                    co-resident, or (systems that fill fewer CTAs) the same
+                                    launch as with fewer                                        */
+    int32_t krylov_up;           /* node groups per lane in the Krylov products (1, 2 or 4; 3D: 1) */
+    double krylov_us_up[3];      /* iteration time with 1, 2, 4 node groups at the chosen grid;
+                                    -1: not timed (3D)                                          */
     int32_t krylov_lanes;        /* lanes per node of the products of 3D solves (8)             */
-    double krylov_us_lanes[3];   /* iteration time with 32, 8, 4 lanes per node; -1: not timed
-                                    (the mapping is fixed at 8; GD_MIXED 3D solves report it)   */
+    double krylov_us_lanes[3];   /* -1: the mapping is fixed                                    */
 } gd_tune_report;
 
 /* Times the element kernel (one tangent pass at the committed state) for each CTA

@@ -2137,6 +2137,7 @@ gd_status gd_autotune(gd_handle *h, gd_tune_report *rep)
     ++H.launches;
     const int keep_grid32 = H.krylov_grid32;
     int kpick32 = H.krylov_cpsm32;
+    int last_ctas = 0;
     for (int cap = 1; cap <= 4; ++cap) {
         // the solve timed here runs with FP32 vectors in GD_MIXED: tune that grid
         const int grid = fp32 ? gd::krylov_blocks_fp32(H.ndof, H.num_sms, cap)
@@ -2144,6 +2145,10 @@ gd_status gd_autotune(gd_handle *h, gd_tune_report *rep)
         if (grid != cap * H.num_sms) continue;       // not co-resident at this width
         if ((size_t)grid > (size_t)4 * H.num_sms) continue;
         if (grid > H.red_blocks) continue;           // beyond the reduction buffers
+        // small systems launch the CTAs that they fill: the same launch as with fewer per SM
+        const int ctas = gd::krylov_launch_ctas(H.ndof, H.n_nodes, H.coarse.nc, grid, fp32);
+        if (ctas == last_ctas) continue;
+        last_ctas = ctas;
         if (fp32) H.krylov_grid32 = grid;
         else H.krylov_grid = grid;
         double tmin = 1e300;
@@ -2175,12 +2180,13 @@ gd_status gd_autotune(gd_handle *h, gd_tune_report *rep)
         if (H.krylov_grid < 1) H.krylov_grid = keep_grid;
         r.krylov_ctas_per_sm = kpick;
     }
-    // node groups per product round at the chosen grid (the two-level kernel: 1 or 2)
+    // node groups per product round at the chosen grid (the two-level kernel: 1 or 2; 4 x 4 blocks
+    // always take one)
     const int ups[3] = {1, 2, 4};
     double ubest = 1e300;
     int upick = H.krylov_up;
     for (double &v : r.krylov_us_up) v = -1.0;
-    for (int ui = 0; ui < (H.coarse.nc > 0 ? 2 : 3) && st == GD_OK; ++ui) {
+    for (int ui = 0; ui < (H.ndof == 4 ? 0 : H.coarse.nc > 0 ? 2 : 3) && st == GD_OK; ++ui) {
         H.krylov_up = ups[ui];
         double tmin = 1e300;
         for (int rep_i = 0; rep_i < 2; ++rep_i) {
@@ -2202,7 +2208,6 @@ gd_status gd_autotune(gd_handle *h, gd_tune_report *rep)
     // 3D solves have one mapping (eight lanes per node in the products)
     for (double &v : r.krylov_us_lanes) v = -1.0;
     r.krylov_lanes = 8;
-    if (st == GD_OK && H.ndof == 4 && fp32) r.krylov_us_lanes[1] = ubest;
     std::swap(H.vals, H.vals_trial);
     H.opt.krylov_max = keep_max;
     if (st) return st;

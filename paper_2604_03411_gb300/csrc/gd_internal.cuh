@@ -429,6 +429,8 @@ cudaError_t krylov_solve_batch(const KrylovCtx &c, const BatchKrylov &L, const v
                                const double *b, double *x, int max_it, bool fp32_vectors);
 // cooperative grid of the Krylov kernels: SMs x co-resident CTAs per SM (at most cap)
 int krylov_blocks(int ndof, bool fp32_vals, int num_sms, int cap = 2);
+// CTAs that a single-system solve launches on a co-resident grid of up to `blocks`
+int krylov_launch_ctas(int ndof, int64_t n_nodes, int nc, int blocks, bool fp32_vectors);
 // the same for the single-system kernels with FP32 vectors (built for four CTAs per SM)
 int krylov_blocks_fp32(int ndof, int num_sms, int cap = 4);
 // Solves K x = b on the free dofs; the result and statistics land in x and c.out.

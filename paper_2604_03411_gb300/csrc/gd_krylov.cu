@@ -1422,6 +1422,28 @@ __global__ void block_inverse_kernel(int64_t n_nodes, const int32_t *rowptr, con
     }
 }
 
+// CTAs of a single-system solve on a co-resident grid of up to `blocks` (npw: nodes per warp, nc:
+// coarse unknowns).  Small systems take fewer CTAs than that: one per four node groups (one
+// warp per SM quarter), or per eight coarse rows (one round of the coarse solve).  A
+// 243-dof system with 87 coarse unknowns on 304 CTAs spent 60 us per iteration on
+// barriers among CTAs without rows.
+// Where the CTAs of one cluster suffice the grid is that cluster: its barrier is hardware,
+// the cooperative one an atomic counter in L2.  A system that wants up to 32 CTAs does two
+// rounds of its coarse rows on 16 (about 1 us more per application) and saves as much on each
+// of the seven barriers.  Measured (gd_solve, cooperative -> cluster): 200 coarse unknowns, 243
+// dofs 759 -> 654 us, 320 in 3D 1,130 -> 1,069, 510 1,024 -> 980, 864 in 3D 1,269 -> 1,133, 972
+// 1,252 -> 1,266, 1,953 1,583 -> 1,617; the full inverse (few iterations), 48 dofs 125 -> 123, 108
+// 272 -> 262, 243 273 -> 272.  A limit of 64: 429 dofs with the full inverse 448 -> 483 us.
+int launch_ctas(int64_t n_nodes, int npw, int nc, int blocks, bool &cluster)
+{
+    int64_t want = ((n_nodes + npw - 1) / npw + 3) / 4;
+    if ((nc + 7) / 8 > want) want = (nc + 7) / 8;
+    if (want < 1) want = 1;
+    cluster = want <= kClusterWant && blocks >= kCluster;
+    if (cluster) return want <= 8 ? 8 : kCluster;
+    return want < blocks ? (int)want : blocks;
+}
+
 // G: lanes per node of the FP32-vector kernels in 2D (otherwise one lane per row)
 template <int NDOF, class V, class T, int G = (NDOF == 3 ? 8 : 4)>
 cudaError_t solve_t(const KrylovCtx &c, const V *vals, const double *b, double *x, double rtol, int max_it)
@@ -1504,27 +1526,9 @@ cudaError_t solve_t(const KrylovCtx &c, const V *vals, const double *b, double *
              : up == 4 ? (const void *)bicgstab3_kernel<NDOF, G, 4, V, T>
                        : (const void *)bicgstab3_kernel<NDOF, G, 2, V, T>;
     using M = RowMap<NDOF, G, T>;
-    // Small systems take fewer CTAs than the co-resident grid: one per four node groups (one
-    // warp per SM quarter), or per eight coarse rows (one round of the coarse solve).  A
-    // 243-dof system with 87 coarse unknowns on 304 CTAs spent 60 us per iteration on
-    // barriers among CTAs without rows.
-    int blocks = c.blocks;
-    {
-        const int64_t groups = (c.n_nodes + M::NPW - 1) / M::NPW;
-        int64_t want = (groups + 3) / 4;
-        if (co && (c.coarse->nc + 7) / 8 > want) want = (c.coarse->nc + 7) / 8;
-        if (want < 1) want = 1;
-        if (want < blocks) blocks = (int)want;
-        // Where the CTAs of one cluster suffice the grid is that cluster: its barrier is hardware,
-        // the cooperative one an atomic counter in L2 (load path with gradient of the 8x8
-        // square, 7 barriers per iteration on 11 CTAs: 57.4 -> 54.5 ms).  A system that wants up
-        // to 32 CTAs does two rounds of its coarse rows on 16 (about 1 us more per application)
-        // and saves as much on each of the seven barriers.
-        if (want <= kClusterWant && c.blocks >= kCluster) {
-            A.cluster = 1;
-            blocks = want <= 8 ? 8 : kCluster;
-        }
-    }
+    bool cluster = false;
+    int blocks = launch_ctas(c.n_nodes, M::NPW, co ? c.coarse->nc : 0, c.blocks, cluster);
+    A.cluster = cluster;
     // Shared-memory copy of each block's rows (3 dofs per node): column lists and, when they
     // fit, values, for as long as the grid stays co-resident with that shared memory.
     // The products then wait on the gathered x alone instead of the chain
@@ -1685,6 +1689,14 @@ __global__ void narrow_kernel(const double *in, float *out, int64_t n)
 }
 
 }  // namespace
+
+int krylov_launch_ctas(int ndof, int64_t n_nodes, int nc, int blocks, bool fp32_vectors)
+{
+    const int npw = ndof == 3 ? (fp32_vectors ? RowMap<3, 8, float>::NPW : RowMap<3, 8, double>::NPW)
+                              : (fp32_vectors ? RowMap<4, 4, float>::NPW : RowMap<4, 4, double>::NPW);
+    bool cluster = false;
+    return launch_ctas(n_nodes, npw, nc, blocks, cluster);
+}
 
 int krylov_blocks_fp32(int ndof, int num_sms, int cap)
 {
