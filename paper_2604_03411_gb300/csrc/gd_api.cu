@@ -294,11 +294,15 @@ gd_status norms(gd::Handle &H, const double *R, NormPair &out)
 constexpr int kCoarseReuse = 8;
 // Systems of up to kCoarseFull dofs take all of them as coarse unknowns, so that M^-1 is the
 // FP32 inverse of a recent matrix of the path.  It is recomputed when a solve needs more
-// iterations than an inversion is worth.  Measured (gd_solve, inversion included, and load
-// paths with gradient of 10 steps): 243 dofs 744 -> 304 us and 48 -> 27 ms, 504 dofs 832 -> 593
-// us and 55 -> 29 ms (429 dofs), 864 dofs in 3D 1,526 -> 1,119 us.  The inversion grows by
-// 16 rows at a time and its share of a single solve passes the saved iterations near 1,000 dofs.
+// iterations than an inversion is worth.  Measured, without -> with: gd_solve, its inversion
+// included, 48 dofs 349 -> 126 us, 243 695 -> 274, 510 1,043 -> 509, 864 in 3D 1,431 -> 858, 972 975 ->
+// 1,061, 1,071 1,125 -> 1,323; load paths of 12 steps with gradient, 48 dofs 36 -> 23 ms, 243 55 ->
+// 28, 510 68 -> 32, 864 in 3D 71 -> 51, 972 63 -> 41, 1,071 76 -> 45.  A single solve is worth the larger
+// inversion up to about 900 dofs, a path beyond; the line lies between.
 constexpr int kCoarseFull = 1024;
+// Iterations of a solve with a reused inverse after which it is recomputed.  Load paths of 12 steps
+// with gradient, 4 / 16 / 64: 48 dofs 22.6 / 23.9 / 23.9 ms, 243 26.5 / 27.9 / 27.9, 320 in 3D 39.3 /
+// 41.6 / 43.2, 972 45.3 / 42.0 / 42.0.
 constexpr int kFullIters = 16;
 enum MatKind { kTangent = 0, kTransposed = 1, kCallerMatrix = 2 };
 

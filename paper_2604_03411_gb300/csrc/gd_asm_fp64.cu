@@ -16,13 +16,9 @@
 // The FP64 pipe bounds the kernel (1.7 lanes per clock and SM), so the design spends as few
 // FP64 operations as it can:
 //  - The point's tangent is formed once per point as the derivative D of (P, Y vector, -Y)
-//    with respect to (grad u, grad phi, phi), both gradients pulled back to the reference
-//    element and weighted by J w, and a row of the element matrix is
-//    K_(a,i),(b,k) = sum_q sum_jl dN_a/dxi_j D_(ij),(kl) dN_b/dxi_l: 3 multiply-adds per
-//    entry of D and row, and the sum over the points and dN_b/dxi_l factorised over the axes
-//    (their values are products of (1 +- 1/sqrt 3) / 2): 20 instead of 64 operations per
-//    derivative and column.  About 100 operations per row and point, against 700 for the
-//    closed form of every (a, b) pair.
+//    with respect to (grad u, grad phi, phi) in reference coordinates, and the element rows
+//    are built from it (gd_rows.cuh): about 100 operations per row and point, against 700 for
+//    the closed form of every (a, b) pair.
 //  - The networks run in 64-bit fixed point (gd_fixed.cuh).
 // Measured (GB300, gd_assemble with tangent; before: FP64 networks one point at a time with
 // a lane per unit, closed-form rows): 140,400 points of HEX8, both widths 64, 33.6 -> 5.83 ms;
@@ -95,12 +91,6 @@ struct Smem {
         return U + ((n > r ? n : r) + 1) / 2 * 2;
     }
 };
-template <int KW>
-__device__ __forceinline__ void cta_sync()
-{
-    if (KW == 1) __syncwarp();
-    else __syncthreads();
-}
 
 // Local damage update (Eq. (dd_7_no_nn)) of the CTA's points p0 .. p0 + 3 that
 // belong to specimen sn: psi_e, phi, kappa_n at sIn[p 4 ..], results (kappa, loading, G',
@@ -331,7 +321,7 @@ __global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
     using S_ = Smem<DIM, NP, KW>;
     using R_ = rows::Rec<DIM>;
     using P_ = State<DIM>;
-    constexpr int NEN = G_::NEN, NQ = G_::NQ, NDOF = G_::NDOF, EL = S_::EL, N2 = DIM * DIM;
+    constexpr int NEN = G_::NEN, NQ = G_::NQ, NDOF = G_::NDOF, EL = S_::EL;
     extern __shared__ __align__(16) double smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double *sX = smem + S_::X, *sD = smem + S_::D, *sRef = smem + S_::REF, *sIn = smem + S_::IN, *sOut = smem + S_::OUT;
@@ -353,7 +343,7 @@ __global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
     const int64_t n_batches = (A.n_elems + EL - 1) / EL;
     for (int64_t batch = blockIdx.x; batch < n_batches; batch += gridDim.x) {
         const int64_t e0 = batch * EL;
-        cta_sync<KW>();
+        __syncthreads();
         for (int t = threadIdx.x; t < EL * NEN; t += 32 * KW) {
             const int64_t e = e0 + t / NEN;
             if (e < A.n_elems) {
@@ -371,7 +361,7 @@ __global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
                 for (int c = 0; c < NDOF; ++c) sD[t * NDOF + c] = 0.0;
             }
         }
-        cta_sync<KW>();
+        __syncthreads();
 
         // ================= qp mode: kinematics and invariants =================
         // the threads that hold the points move on by one warp per batch, so that the SM's
@@ -485,7 +475,7 @@ __global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
             sIn[pt * 4 + 1] = y[1];
             sIn[pt * 4 + 2] = y[2];
         }
-        cta_sync<KW>();
+        __syncthreads();
 
         // ================= net mode: energy network =================
         // (points of different specimens take turns: a round's networks are uniform)
@@ -513,7 +503,7 @@ __global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
                 }
             }
         }
-        cta_sync<KW>();
+        __syncthreads();
 
         // ================= qp mode: energy derivatives wrt (I1-3, I2-3, J-1) =================
         if (qp) {
@@ -599,7 +589,7 @@ __global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
             sIn[pt * 4 + 1] = st[P_::PHI];
             sIn[pt * 4 + 2] = valid ? __ldg(A.kappa_n + e_me * NQ + q) : 0.0;
         }
-        cta_sync<KW>();
+        __syncthreads();
 
         // ================= net mode: local damage update =================
         if (A.kappa_fixed) {
@@ -625,7 +615,7 @@ __global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
             n_eval = __reduce_add_sync(0xffffffffu, n_eval);
             if (lane == 0 && n_eval) atomicAdd(A.counters + 2, n_eval);
         }
-        cta_sync<KW>();
+        __syncthreads();
 
         // ================= qp mode: stress and the point's tangent =================
         bool loading = false;
@@ -657,7 +647,7 @@ __global__ void __launch_bounds__(32 * KW, 16 / KW) asm_fp64_kernel(AsmArgs A)
             const unsigned n_load = __ballot_sync(0xffffffffu, loading);
             if (lane == 0 && n_load) atomicAdd(A.counters + 1, __popc(n_load));
         }
-        cta_sync<KW>();
+        __syncthreads();
 
         // ================= row mode: element residual and tangent =================
         if (warp < NP / 8)

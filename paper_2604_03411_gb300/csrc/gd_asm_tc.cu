@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) asm_tc_kernel(AsmArgs A, TcArgs
 {
     using G_ = Geo<DIM>;
     using R_ = rows::Rec<DIM>;
-    constexpr int NEN = G_::NEN, NQ = G_::NQ, NDOF = G_::NDOF, EPW = G_::EPW;
+    constexpr int NEN = G_::NEN, NQ = G_::NQ, EPW = G_::EPW;
     extern __shared__ __align__(1024) uint8_t tc_smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     Shared S;

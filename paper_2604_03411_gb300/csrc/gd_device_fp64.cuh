@@ -1,5 +1,5 @@
 // gd_device_fp64.cuh -- FP64 device building blocks shared by the element
-// kernel and the adjoint kernel: shape functions, the per-point record layout,
+// kernel and the adjoint kernel: shape functions,
 // the energy and yield networks in unit mode (lane = network unit) and the
 // local-update residual.  Included inside an anonymous namespace of each
 // translation unit.
@@ -34,9 +34,7 @@ struct Geo {
     static constexpr int NEN = DIM == 2 ? 4 : 8;
     static constexpr int NQ = NEN;
     static constexpr int NDOF = DIM + 1;
-    static constexpr int ND = NEN * NDOF;
     static constexpr int EPW = 32 / NQ;         // elements per batch
-    static constexpr int EPR = 32 / ND;         // elements per row pass (Q4: 2, HEX8: 1)
 };
 
 // sign of node a along reference axis k (HEX8 ordering; Q4 uses the first four)
@@ -68,35 +66,6 @@ __device__ __forceinline__ void ref_shape(int a, const double *xi, double &N, do
         dN[k] = v;
     }
 }
-
-// ---- per-point record (row-mode inputs), doubles ----
-enum : int {
-    Q_JW = 0,
-    Q_JINV = 1,      // 9: dxi_k/dX_J at [k*3+J]
-    Q_F = 10,        // 9
-    Q_P = 19,        // 9: total first Piola-Kirchhoff stress
-    Q_M = 28,        // 3: C^-1 grad phi
-    Q_H = 31,        // 3: F^-T grad phi
-    Q_I1 = 34,
-    Q_B = 35,        // 9: F F^T
-    Q_FINV = 44,     // 9: F^-1
-    Q_HS = 53,       // 6: f_d psi_mn (11 12 13 22 23 33)
-    Q_G1 = 59,       // f_d psi_1
-    Q_G2 = 60,       // f_d psi_2
-    Q_G3J = 61,      // f_d psi_3 J
-    Q_PS1 = 62,      // psi_1 (undamaged)
-    Q_PS2 = 63,
-    Q_PS3J = 64,     // psi_3 J
-    Q_CK = 65,       // f_d' c_kappa
-    Q_BCK = 66,      // beta_d c_kappa
-    Q_FDK = 67,      // f_d' dkappa/dphi
-    Q_PP = 68,       // beta_d (1 - dkappa/dphi)
-    Q_PEN = 69,      // beta_d (phi - kappa)
-    Q_J = 70,        // det F
-    Q_REC = 71
-};
-// ---- per (point, node) vector record ----
-enum : int { V_N = 0, V_NN = 3, V_F = 4, V_G2 = 7, V_NT = 10, V_PN = 13, V_MN = 16, V_REC = 17 };
 
 __device__ __forceinline__ int sym6(int i, int j)
 {

@@ -63,9 +63,7 @@ struct Geo {
     static constexpr int NEN = DIM == 2 ? 4 : 8;
     static constexpr int NQ = NEN;
     static constexpr int NDOF = DIM + 1;
-    static constexpr int ND = NEN * NDOF;
     static constexpr int EPW = 32 / NQ;         // elements per batch
-    static constexpr int EPR = 32 / ND;         // elements per row pass (Q4: 2, HEX8: 1)
 };
 
 // sign of node a along reference axis k (HEX8 ordering; Q4 uses the first four)
