@@ -21,11 +21,11 @@
 //    the closed form of every (a, b) pair.
 //  - The networks run in 64-bit fixed point (gd_fixed.cuh).
 // Measured (GB300, gd_assemble with tangent; before: FP64 networks one point at a time with
-// a lane per unit, closed-form rows): 140,400 points of HEX8, both widths 64, 33.6 -> 5.83 ms;
-// 159,744 of Q4, widths 32, 10.2 -> 2.60 ms; 256 of Q4, widths 16 and 8, 1.21 -> 0.088 ms;
-// residual alone of 32,640 HEX8 points, widths 24 and 40, 3.53 -> 0.53 ms.  (Without the
+// a lane per unit, closed-form rows): 140,400 points of HEX8, both widths 64, 33.6 -> 5.75 ms;
+// 159,744 of Q4, widths 32, 10.2 -> 2.55 ms; 256 of Q4, widths 16 and 8, 1.21 -> 0.087 ms;
+// residual alone of 32,640 HEX8 points, widths 24 and 40, 3.53 -> 0.52 ms.  (Without the
 // trust in the fixed-point sums being checked and with one scale for all first-layer and
-// one for all output weights: 5.70, 2.52, 0.085 and 0.51 ms.)  Built for 16 warps per SM: 128
+// one for all output weights: 2 to 3 % less.)  Built for 16 warps per SM: 128
 // registers, with 180-340 bytes of spills in 2D and 560-990 in 3D, the points' state in shared
 // memory.  Width-64 HEX8 networks need 64 KB per CTA of four warps, so that 12 warps are
 // resident there (8 with 255 registers: 7.5 ms where 12 took 5.75).  Instruction latency is the
@@ -48,9 +48,10 @@ namespace {
 
 // Trial yield values farther than this (relative to max(1, kappa_n)), and than what FP32 may be
 // off by, from zero are decided by the FP32 evaluation; closer ones by an FP64 evaluation.  The
-// FP32 network's relative error is a few 1e-7 (two sums of up to 64 positive terms), of
-// N(0) / N'(0) where the network hardly depends on q and of q's terms near full damage.
-constexpr double kTrialMargin = 1e-4, kTrialRel = 2e-6;
+// FP32 network's relative error is a few 1e-7 (two sums of up to 64 positive terms) and __expf's, up to
+// 1.4e-7 |h| (8e-6 at h = -57), of N(0) / N'(0) where the network hardly depends on q, and of q's
+// terms near full damage.
+constexpr double kTrialMargin = 1e-4, kTrialRel = 8e-6;
 
 // the normalising constants of this kernel's own evaluation
 __device__ __forceinline__ NetConst own_consts(const NetConst &c)
@@ -138,7 +139,7 @@ __device__ __forceinline__ int local_update(const AsmArgs &A, const e32::MatF &m
     }
     // The root in FP32 (the lazily bracketed Newton iteration of the mixed kernels, from the
     // warm start), then FP64: one value-only evaluation and a Newton step with the FP32 slope
-    // (its relative error, ~1e-7, times a correction of ~1e-6 leaves ~1e-13), then one full
+    // (its relative error, ~1e-6, times a correction of ~1e-6 leaves ~1e-12), then one full
     // evaluation and a last Newton step; the slope and G' of that evaluation feed the tangent
     // (they change by ~1e-12 relative over the last step).  Where the FP32 root is not close
     // enough, the FP64 bracketed iteration takes over from it.  Both iterations also stop on

@@ -459,24 +459,24 @@ __device__ __forceinline__ void residual(const MatConst &m, const DevNet &yld, i
     }
 }
 
-// Softplus and sigmoid to FP32 relative accuracy (below 5e-7), for the FP32 part of the local solve.
-// The trial decision rests on G = (N_k(q) - N_k(0)) / N_k'(0), which amplifies an absolute error
-// wherever the units are in the flat part of softplus: the logarithm of the rounded 1 + e moved G
-// by 4e-3 with biases of -10.  log1p(e) / e for 0 <= e <= 1 is a minimax polynomial (Lawson's
-// iteration on the Chebyshev basis, 3e-8), which with the approximate reciprocal costs less
-// than log1pf and a division (notched plate, 159,744 points: 2,595 us with those).
+// Softplus and sigmoid for the FP32 part of the local solve, with relative errors of a few 1e-7 plus
+// those of __expf (1.2 |v| units in the last place).  The trial decision rests on G = (N_k(q) -
+// N_k(0)) / N_k'(0), which amplifies an absolute error wherever the units are in the flat part of
+// softplus: the logarithm of the rounded 1 + e moved G by 4e-3 with biases of -10.  log1p(e) / e for
+// 0 <= e <= 1 is a minimax polynomial (Lawson's iteration on the Chebyshev basis, 1.9e-7).
+// (A pass over the notched plate, 159,744 points: expf, log1pf and a division 5 % more, expf and one
+// more term here 1.5 %.)
 __device__ __forceinline__ void sp_sig_start(float v, float &sp, float &sg)
 {
-    const float e = expf(-fabsf(v)), r = __fdividef(1.0f, 1.0f + e);
-    float p = 0.00523268804f;
-    p = fmaf(p, e, -0.0295052137f);
-    p = fmaf(p, e, 0.0782259107f);
-    p = fmaf(p, e, -0.136632428f);
-    p = fmaf(p, e, 0.191060051f);
-    p = fmaf(p, e, -0.24842982f);
-    p = fmaf(p, e, 0.333190978f);
-    p = fmaf(p, e, -0.499994934f);
-    p = fmaf(p, e, 0.99999994f);
+    const float e = __expf(-fabsf(v)), r = __fdividef(1.0f, 1.0f + e);
+    float p = -0.0085391989f;
+    p = fmaf(p, e, 0.0440895967f);
+    p = fmaf(p, e, -0.107681662f);
+    p = fmaf(p, e, 0.177452385f);
+    p = fmaf(p, e, -0.244954616f);
+    p = fmaf(p, e, 0.332754791f);
+    p = fmaf(p, e, -0.499974042f);
+    p = fmaf(p, e, 0.999999821f);
     sp = fmaxf(v, 0.0f) + e * p;
     sg = v >= 0.0f ? r : e * r;
 }
