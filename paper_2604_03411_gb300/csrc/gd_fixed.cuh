@@ -13,7 +13,7 @@
 //    64-bit accumulation.  Its scale is the power of two above the row's largest weight times
 //    the one above the point's largest operand, and its error a few 2^-56 of that, whatever the
 //    sum is.  Where the largest terms meet that is below the rounding of the FP64 sum; where a
-//    row's large weights meet the small operands it is not.  Every point's sums are judged
+//    row's large weights meet the small operands it is not.  Every point's sums are checked
 //    (gd_net_fp64.cuh, Trust), and a point that would lose accuracy is evaluated again, with the
 //    second form and scales of its own and, where that does not help, by the FP64 functions.
 // Compiles for the host as well (the tables are constant expressions).
@@ -378,7 +378,7 @@ enum : int { kPath = 3, kRows = 4, kCols = 5, kOuts = 6, kWords = 8 };      // b
 // e[3 w + kPath]: how a network's points start
 enum : int {
     kPlain = 0,
-    kTails = 1,                // biases far below zero: with the activations' tails
+    kTails = 1,                // units in the tail of softplus at rest: with the activations' tails
     kFp64 = 2                  // weights that are not finite or beyond 2^kLargest: the FP64 functions
 };
 constexpr int kZero = -900;    // exponent of a row or column of zeros (its products are exact)

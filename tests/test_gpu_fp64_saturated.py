@@ -84,3 +84,22 @@ def test_small_weights_on_large_activations(env, spread, dim, w):
         A2[:] = 0.0
         a3[:] = 0.0
     check(env, prob)
+
+
+def test_batch_of_ordinary_and_flat_networks(env):
+    """Every specimen of a batch takes its own networks' form: a point's history and branch are those of
+    the specimen alone, to the last bit."""
+    torch, B, _ = env
+    probs, states = [], []
+    for i, (bias, w) in enumerate([(0.0, 8), (-20.0, 17), (-4.0, 24), (0.0, 32), (-60.0, 9)]):
+        prob = problem(2, w)
+        if bias:
+            without_skips(prob.psi, bias)
+            without_skips(prob.yld, bias)
+        probs.append(prob)
+        states.append(smooth_state(prob.mesh, np.random.default_rng(i), u_amp=0.06))
+    alone = [gpu_assemble(B, torch, B.gd_create(p, B.gd_default_options()), d, k)[2:] for p, (d, k) in zip(probs, states)]
+    h = B.gd_create_batch(probs, B.gd_default_options())
+    _, _, kg, lg = gpu_assemble(B, torch, h, np.concatenate([d for d, _ in states]), np.concatenate([k for _, k in states]))
+    assert np.array_equal(kg, np.concatenate([a[0] for a in alone]))
+    assert np.array_equal(lg, np.concatenate([a[1] for a in alone]))
